@@ -17,7 +17,7 @@
 // slot: 8 per row up to 32 entries, 32 per row above), one thread per chain,
 // and rows above 128 entries keep one warp per chunk.
 //
-// The schedule (built on the host from row_ptr, once per P):
+// The schedule (built on the device from row_ptr, once per P):
 //   short CTAs  rows [256 c, 256 c + 256): the chains of their rows of at most
 //               32 entries; then one thread per row adds its 8 slots and
 //               updates the row (rows above 32 entries are left to the others;
@@ -35,10 +35,6 @@
 // of all entries of its chain before the first gather returns.  A CTA starts
 // by prefetching into L2 the streams it reads (chain codes, col and P in chain
 // order, its rows' optimiser state; a hub chunk's col and P).
-#include <algorithm>
-#include <cstring>
-#include <vector>
-
 #include "row_update.cuh"
 #include "storage.cuh"
 #include "tsgne_internal.cuh"
@@ -213,139 +209,306 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
                       a.Ynext, Ynext16, a.upd, a.gains, a.eta, a.min_gain);
 }
 
-template <class PT>
-__global__ void k_plan_gather(int64_t count, const int64_t* __restrict__ perm, const int32_t* __restrict__ col,
-                              const PT* __restrict__ P, int32_t* __restrict__ colS, PT* __restrict__ PS) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += stride) {
-    const int64_t e = perm[k];
-    colS[k] = col[e];
-    PS[k] = P[e];
+// ------------------------------------------------ building the schedule
+//
+// Four small launches over blocks of 256 consecutive rows (a block is a short
+// CTA of the schedule), one host wait for the sizes of the lists:
+//   k_row_totals   what each block's rows add to every list
+//   k_row_scan     exclusive scan of those totals over the blocks (CTA f: list f)
+//   k_row_lists    the hub rows with their chunks, the medium rows, the chunks
+//                  of the rows above 128 entries, each in row order
+//   k_plan_chains  a CTA's chains sorted longest first (by counting: a row's
+//                  chains have at most two lengths, so four counters packed in
+//                  one 64-bit scan give every chain its place), then col and P
+//                  copied level by level, coalesced.
+// Bound by the reads of row_ptr, col and P and the writes of their copies
+// (16 B per entry).  A whole P build of 300,000 rows and 2.0M entries (device
+// arrays) takes 2.72 ms; with the lists built by host loops over a copy of
+// row_ptr, which these kernels replace, it took 16.5 ms.
+enum RowList { kCodes = 0, kEntries, kHeavyRows, kChunks, kMedRows, kMedEntries, kBigChunks, kRowLists };
+
+struct RowAdds {
+  uint32_t v[kRowLists];
+};
+
+// What one row of d entries adds to each list.
+__device__ __forceinline__ RowAdds row_adds(int64_t d) {
+  RowAdds a{};
+  if (d <= kHeavyDeg) {
+    a.v[kCodes] = (uint32_t)(d < kSlotsShort ? d : kSlotsShort);
+    a.v[kEntries] = (uint32_t)d;
+    return a;
+  }
+  a.v[kHeavyRows] = 1u;
+  a.v[kChunks] = (uint32_t)((d + kHeavyChunk - 1) / kHeavyChunk);
+  if (d <= kMedDeg) {
+    a.v[kMedRows] = 1u;
+    a.v[kMedEntries] = (uint32_t)d;
+  } else {
+    a.v[kBigChunks] = a.v[kChunks];
+  }
+  return a;
+}
+
+// tot[list][block] = sum of the block's rows.
+__global__ void __launch_bounds__(kPlanThreads)
+    k_row_totals(int n, const int64_t* __restrict__ rp, int nb, int64_t* __restrict__ tot) {
+  __shared__ uint32_t sum[kRowLists];
+  if (threadIdx.x < kRowLists) sum[threadIdx.x] = 0u;
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * kPlanThreads + threadIdx.x;
+  const RowAdds a = row_adds(i < n ? rp[i + 1] - rp[i] : 0);
+#pragma unroll
+  for (int f = 0; f < kRowLists; ++f) {
+    const uint32_t w = __reduce_add_sync(0xffffffffu, a.v[f]);
+    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&sum[f], w);
+  }
+  __syncthreads();
+  if (threadIdx.x < kRowLists) tot[(int64_t)threadIdx.x * nb + blockIdx.x] = sum[threadIdx.x];
+}
+
+// Exclusive scan over the threads of a CTA (at most 1,024); *total: the sum.
+template <class T>
+__device__ __forceinline__ T cta_excl_scan(T v, T* total) {
+  __shared__ T ws[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  T x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) ws[w] = x;
+  __syncthreads();
+  T base = 0, all = 0;
+  for (int k = 0; k < nw; ++k) {
+    if (k < w) base += ws[k];
+    all += ws[k];
+  }
+  *total = all;
+  __syncthreads();
+  return base + x - v;
+}
+
+// CTA f: tot[f][0..nb) to its exclusive scan, the total to sums[f].
+__global__ void __launch_bounds__(1024) k_row_scan(int nb, int64_t* __restrict__ tot, int64_t* __restrict__ sums) {
+  int64_t* t = tot + (int64_t)blockIdx.x * nb;
+  int64_t carry = 0;
+  for (int c0 = 0; c0 < nb; c0 += 1024) {
+    const int c = c0 + threadIdx.x;
+    int64_t all;
+    const int64_t ex = cta_excl_scan<int64_t>(c < nb ? t[c] : 0, &all);
+    if (c < nb) t[c] = carry + ex;
+    carry += all;
+  }
+  if (threadIdx.x == 0) sums[blockIdx.x] = carry;
+}
+
+// The lists of rows and chunks (see HeavyStore and AttractPlan).  med_ent
+// (NULL: no plan wanted): first entry, in the copies, of each medium CTA.
+__global__ void __launch_bounds__(kPlanThreads)
+    k_row_lists(int n, const int64_t* __restrict__ rp, int nb, const int64_t* __restrict__ tot,
+                int32_t* __restrict__ rows, int32_t* __restrict__ chunk_off, int32_t* __restrict__ chunk_row,
+                int32_t* __restrict__ chunk_heavy, int64_t* __restrict__ chunk_begin, int64_t* __restrict__ chunk_end,
+                int32_t* __restrict__ med_rows, int64_t* __restrict__ med_ent, int32_t* __restrict__ big) {
+  const int64_t i = (int64_t)blockIdx.x * kPlanThreads + threadIdx.x;
+  const int64_t a = i < n ? rp[i] : 0, b = i < n ? rp[i + 1] : 0;
+  const RowAdds ra = row_adds(b - a);
+  if (!__syncthreads_or((int)ra.v[kHeavyRows])) return;
+  uint32_t ex[kRowLists], all;
+#pragma unroll
+  for (int f = kHeavyRows; f < kRowLists; ++f) ex[f] = cta_excl_scan<uint32_t>(ra.v[f], &all);
+  if (!ra.v[kHeavyRows]) return;
+  auto at = [&](int f) { return tot[(int64_t)f * nb + blockIdx.x] + ex[f]; };
+  const int64_t h = at(kHeavyRows), c0 = at(kChunks);
+  rows[h] = (int32_t)i;
+  chunk_off[h + 1] = (int32_t)(c0 + ra.v[kChunks]);
+  const int64_t bg = at(kBigChunks);
+  for (uint32_t k = 0; k < ra.v[kChunks]; ++k) {
+    const int64_t x = a + (int64_t)k * kHeavyChunk;
+    chunk_row[c0 + k] = (int32_t)i;
+    chunk_heavy[c0 + k] = (int32_t)h;
+    chunk_begin[c0 + k] = x;
+    chunk_end[c0 + k] = x + kHeavyChunk < b ? x + kHeavyChunk : b;
+    if (med_ent != nullptr && ra.v[kBigChunks]) big[bg + k] = (int32_t)(c0 + k);
+  }
+  if (med_ent != nullptr && ra.v[kMedRows]) {
+    const int64_t m = at(kMedRows);
+    med_rows[m] = (int32_t)i;
+    if (m % kMedRowsPerCta == 0) med_ent[m / kMedRowsPerCta] = at(kMedEntries);
   }
 }
 
-// Chains of one CTA's rows: codes sorted longest first, per-level counts, and
-// the entry positions of level k, chain q (in that order) appended to perm.
-void plan_cta(const std::vector<int64_t>& rp, const std::vector<int64_t>& rows, int slots, int shift,
-              std::vector<uint16_t>& code, std::vector<int64_t>& perm, PlanCta& pc) {
-  std::vector<uint16_t> by[4];
-  std::vector<int64_t> first[4];
-  for (size_t r = 0; r < rows.size(); ++r) {
-    const int64_t i = rows[r];
-    if (i < 0) continue;
-    const int64_t d = rp[i + 1] - rp[i];
-    for (int s = 0; s < slots && s < d; ++s) {
-      const int depth = (int)((d - s + slots - 1) / slots);  // 1..4
-      by[depth - 1].push_back((uint16_t)((r << shift) | (size_t)s));
-      first[depth - 1].push_back(rp[i] + s);
+// Chain codes, copies of col and P in chain order and the PlanCta of one CTA:
+// medium CTA blockIdx.x < n_med, else short CTA blockIdx.x - n_med.  Chain
+// (row r, slot s) of a row of d = S q + m entries (S slots) holds q + 1
+// entries if s < m, else q; the chains lie longest first, within a length by
+// row and slot.
+template <class PT>
+__global__ void __launch_bounds__(kPlanThreads)
+    k_plan_chains(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const PT* __restrict__ P,
+                  int n_med, int64_t n_med_rows, int64_t med_entries, const int32_t* __restrict__ med_rows,
+                  const int64_t* __restrict__ med_ent, int nb, const int64_t* __restrict__ tot,
+                  PlanCta* __restrict__ cta, uint16_t* __restrict__ code, int32_t* __restrict__ colS,
+                  PT* __restrict__ PS) {
+  __shared__ int64_t sfirst[kPartials];  // first entry of each chain, in chain order
+  __shared__ int64_t sa[kShortRowsPerCta];
+  __shared__ int sq[kShortRowsPerCta], sm[kShortRowsPerCta];
+  __shared__ unsigned long long sex[kShortRowsPerCta];
+  const int tid = threadIdx.x;
+  const bool med = (int)blockIdx.x < n_med;
+  const int c = med ? (int)blockIdx.x : (int)blockIdx.x - n_med;
+  const int shift = med ? 5 : 3, slots = 1 << shift;
+  int64_t r0 = 0;
+  int nrows;
+  int64_t i = -1;
+  if (med) {
+    r0 = (int64_t)c * kMedRowsPerCta;
+    nrows = (int)min((int64_t)kMedRowsPerCta, n_med_rows - r0);
+    if (tid < nrows) i = med_rows[r0 + tid];
+  } else {
+    r0 = (int64_t)c * kShortRowsPerCta;
+    nrows = (int)min((int64_t)kShortRowsPerCta, (int64_t)n - r0);
+    if (tid < nrows) i = r0 + tid;
+  }
+  int64_t a = 0, d = 0;
+  if (i >= 0) {
+    a = rp[i];
+    d = rp[i + 1] - a;
+    if (!med && d > kHeavyDeg) d = 0;  // a medium or big CTA's row
+  }
+  const int q = (int)(d >> shift), m = (int)d & (slots - 1);
+  // chains of length L = 1..4 in bits 16 (L - 1); at most 2,048 of a length
+  unsigned long long cnt = 0ull;
+  if (m > 0) cnt += (unsigned long long)m << (16 * q);
+  if (q > 0) cnt += (unsigned long long)(slots - m) << (16 * (q - 1));
+  unsigned long long all;
+  sex[tid] = cta_excl_scan<unsigned long long>(cnt, &all);
+  sa[tid] = a;
+  sq[tid] = q;
+  sm[tid] = m;
+  __syncthreads();
+  int num[4], start[4];
+  {
+    int at = 0;
+#pragma unroll
+    for (int L = 3; L >= 0; --L) {
+      num[L] = (int)(all >> (16 * L)) & 0xffff;
+      start[L] = at;
+      at += num[L];
     }
   }
-  pc.pair = (int32_t)code.size();
-  pc.ent = (int64_t)perm.size();
-  std::vector<int64_t> start;
-  for (int dep = 3; dep >= 0; --dep) {
-    code.insert(code.end(), by[dep].begin(), by[dep].end());
-    start.insert(start.end(), first[dep].begin(), first[dep].end());
+  const int64_t pair0 = med ? r0 * kSlotsMed : n_med_rows * kSlotsMed + tot[(int64_t)kCodes * nb + c];
+  const int64_t ent0 = med ? med_ent[c] : med_entries + tot[(int64_t)kEntries * nb + c];
+  for (int k = tid; k < nrows << shift; k += kPlanThreads) {
+    const int r = k >> shift, s = k & (slots - 1);
+    const bool lng = s < sm[r];
+    const int len = sq[r] + (lng ? 1 : 0);
+    if (len == 0) continue;
+    int st = start[0];
+#pragma unroll
+    for (int L = 1; L < 4; ++L)
+      if (len == L + 1) st = start[L];
+    const int at = st + ((int)(sex[r] >> (16 * (len - 1))) & 0xffff) + (lng ? s : s - sm[r]);
+    code[pair0 + at] = (uint16_t)((r << shift) | s);
+    sfirst[at] = sa[r] + s;
   }
-  const int64_t total = (int64_t)start.size();
-  pc.cnt[0] = (int32_t)total;
-  for (int k = 1; k < 4; ++k) {
-    int64_t c = 0;
-    for (int dep = k; dep < 4; ++dep) c += (int64_t)by[dep].size();
-    pc.cnt[k] = (int32_t)c;
+  __syncthreads();
+  int64_t ent = ent0;
+  int more = num[0] + num[1] + num[2] + num[3];  // chains of more than k entries: a prefix of the list
+  PlanCta pc{};
+  pc.ent = ent0;
+  pc.pair = (int32_t)pair0;
+  pc.rows = med ? (int32_t)r0 : 0;
+  pc.nrows = nrows;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    pc.cnt[k] = more;
+    for (int x = tid; x < more; x += kPlanThreads) {
+      const int64_t e = sfirst[x] + (int64_t)slots * k;
+      colS[ent + x] = col[e];
+      PS[ent + x] = P[e];
+    }
+    ent += more;
+    more -= num[k];
   }
-  for (int k = 0; k < 4; ++k)
-    for (int32_t q = 0; q < pc.cnt[k]; ++q) perm.push_back(start[q] + (int64_t)slots * k);
+  if (tid == 0) cta[blockIdx.x] = pc;
+}
+
+// The hub rows of a structure and, if plan is not NULL, the schedule.
+tsgne_status build_row_schedule(int n, const int64_t* rp, const int32_t* col, const float* P, const bf16* P16,
+                                HeavyStore& hs, AttractPlan* plan, cudaStream_t s) {
+  const int nb = (n + kPlanThreads - 1) / kPlanThreads;
+  DevBuf<int64_t> tot, med_ent;
+  TS_TRY(tot.alloc((size_t)nb * kRowLists + kRowLists));
+  int64_t* const sums = tot.get() + (size_t)nb * kRowLists;
+  k_row_totals<<<nb, kPlanThreads, 0, s>>>(n, rp, nb, tot.get());
+  k_row_scan<<<kRowLists, 1024, 0, s>>>(nb, tot.get(), sums);
+  TS_CUDA(cudaGetLastError());
+  int64_t h[kRowLists];
+  TS_CUDA(cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s));
+  TS_CUDA(cudaStreamSynchronize(s));
+  auto at_least_1 = [](int64_t v) { return (size_t)(v > 0 ? v : 1); };
+  hs.count = (int)h[kHeavyRows];
+  hs.chunks = (int)h[kChunks];
+  TS_TRY(hs.rows.alloc(at_least_1(h[kHeavyRows])));
+  TS_TRY(hs.chunk_off.alloc((size_t)h[kHeavyRows] + 1));
+  TS_TRY(hs.chunk_row.alloc(at_least_1(h[kChunks])));
+  TS_TRY(hs.chunk_begin.alloc(at_least_1(h[kChunks])));
+  TS_TRY(hs.chunk_end.alloc(at_least_1(h[kChunks])));
+  TS_TRY(hs.fa.alloc(at_least_1(h[kChunks])));
+  TS_TRY(hs.chunk_heavy.alloc(at_least_1(h[kChunks])));
+  TS_TRY(hs.arrivals.alloc(at_least_1(h[kHeavyRows])));
+  TS_CUDA(cudaMemsetAsync(hs.arrivals.get(), 0, sizeof(uint32_t) * at_least_1(h[kHeavyRows]), s));
+  TS_CUDA(cudaMemsetAsync(hs.chunk_off.get(), 0, sizeof(int32_t), s));
+  if (plan) {
+    *plan = AttractPlan();
+    plan->n_med = (int)((h[kMedRows] + kMedRowsPerCta - 1) / kMedRowsPerCta);
+    plan->n_short = nb;
+    plan->n_big = (int)h[kBigChunks];
+    plan->n_med_rows = h[kMedRows];
+    plan->n_codes = h[kMedRows] * kSlotsMed + h[kCodes];
+    plan->entries = h[kMedEntries] + h[kEntries];
+    TS_TRY(plan->cta.alloc((size_t)(plan->n_med + plan->n_short)));
+    TS_TRY(plan->code.alloc((size_t)plan->n_codes));
+    TS_TRY(plan->med_rows.alloc((size_t)plan->n_med_rows));
+    TS_TRY(plan->big.alloc((size_t)plan->n_big));
+    TS_TRY(plan->colS.alloc((size_t)plan->entries));
+    TS_TRY(med_ent.alloc((size_t)plan->n_med));
+    if (P16) TS_TRY(plan->PS16.alloc((size_t)plan->entries));
+    else TS_TRY(plan->PS.alloc((size_t)plan->entries));
+  }
+  if (h[kHeavyRows] > 0)
+    k_row_lists<<<nb, kPlanThreads, 0, s>>>(n, rp, nb, tot.get(), hs.rows.get(), hs.chunk_off.get(),
+                                            hs.chunk_row.get(), hs.chunk_heavy.get(), hs.chunk_begin.get(),
+                                            hs.chunk_end.get(), plan ? plan->med_rows.get() : nullptr,
+                                            plan ? med_ent.get() : nullptr, plan ? plan->big.get() : nullptr);
+  if (plan) {
+    const int grid = plan->n_med + plan->n_short;
+    if (P16)
+      k_plan_chains<bf16><<<grid, kPlanThreads, 0, s>>>(
+          n, rp, col, P16, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), nb,
+          tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS16.get());
+    else
+      k_plan_chains<float><<<grid, kPlanThreads, 0, s>>>(
+          n, rp, col, P, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), nb,
+          tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS.get());
+  }
+  TS_CUDA(cudaGetLastError());
+  TS_CUDA(cudaStreamSynchronize(s));  // tot and med_ent are freed on return
+  if (plan) plan->ready = true;
+  return TSGNE_OK;
 }
 
 }  // namespace
 
-tsgne_status build_attract_plan(int n, const int64_t* rp_dev, const int32_t* col_dev, const float* P_dev,
-                                const bf16* P16_dev, const HeavyStore& hs, AttractPlan& plan, cudaStream_t s) {
-  plan = AttractPlan();
-  std::vector<int64_t> rp((size_t)n + 1);
-  TS_CUDA(cudaMemcpyAsync(rp.data(), rp_dev, sizeof(int64_t) * ((size_t)n + 1), cudaMemcpyDeviceToHost, s));
-  TS_CUDA(cudaStreamSynchronize(s));
-  std::vector<uint16_t> code;
-  std::vector<int64_t> perm;
-  std::vector<PlanCta> med, shorts;
-  std::vector<int32_t> med_rows, big;
-  // medium rows (33..128 entries), 64 per CTA; big rows' chunks
-  int32_t chunk = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t d = rp[i + 1] - rp[i];
-    if (d <= kHeavyDeg) continue;
-    const int32_t nch = (int32_t)((d + kHeavyChunk - 1) / kHeavyChunk);
-    if (d <= kMedDeg) {
-      med_rows.push_back((int32_t)i);
-    } else {
-      for (int32_t k = 0; k < nch; ++k) big.push_back(chunk + k);
-    }
-    chunk += nch;
-  }
-  if (chunk != hs.chunks) {
-    last_msg() = "attraction plan: chunk count differs from the hub-row store";
-    return TSGNE_ERR_CUDA;
-  }
-  for (size_t r0 = 0; r0 < med_rows.size(); r0 += kMedRowsPerCta) {
-    const size_t r1 = std::min(med_rows.size(), r0 + kMedRowsPerCta);
-    std::vector<int64_t> rows(med_rows.begin() + (long)r0, med_rows.begin() + (long)r1);
-    PlanCta pc{};
-    plan_cta(rp, rows, kSlotsMed, 5, code, perm, pc);
-    pc.rows = (int32_t)r0;
-    pc.nrows = (int32_t)(r1 - r0);
-    med.push_back(pc);
-  }
-  for (int64_t r0 = 0; r0 < n; r0 += kShortRowsPerCta) {
-    std::vector<int64_t> rows;
-    for (int64_t i = r0; i < std::min<int64_t>(n, r0 + kShortRowsPerCta); ++i)
-      rows.push_back(rp[i + 1] - rp[i] <= kHeavyDeg ? i : -1);
-    PlanCta pc{};
-    plan_cta(rp, rows, kSlotsShort, 3, code, perm, pc);
-    pc.nrows = (int32_t)rows.size();
-    shorts.push_back(pc);
-  }
-  plan.n_med = (int)med.size();
-  plan.n_short = (int)shorts.size();
-  plan.n_big = (int)big.size();
-  plan.entries = (int64_t)perm.size();
-  plan.n_codes = (int64_t)code.size();
-  plan.n_med_rows = (int64_t)med_rows.size();
-  std::vector<PlanCta> ctas(med);
-  ctas.insert(ctas.end(), shorts.begin(), shorts.end());
-  TS_TRY(plan.cta.alloc(ctas.size()));
-  TS_TRY(plan.code.alloc(code.size()));
-  TS_TRY(plan.med_rows.alloc(med_rows.size()));
-  TS_TRY(plan.big.alloc(big.size()));
-  TS_TRY(plan.colS.alloc((size_t)plan.entries));
-  DevBuf<int64_t> dperm;
-  TS_TRY(dperm.alloc((size_t)plan.entries));
-  TS_CUDA(cudaMemcpyAsync(plan.cta.get(), ctas.data(), sizeof(PlanCta) * ctas.size(), cudaMemcpyHostToDevice, s));
-  if (!code.empty())
-    TS_CUDA(cudaMemcpyAsync(plan.code.get(), code.data(), sizeof(uint16_t) * code.size(), cudaMemcpyHostToDevice, s));
-  if (!med_rows.empty())
-    TS_CUDA(cudaMemcpyAsync(plan.med_rows.get(), med_rows.data(), sizeof(int32_t) * med_rows.size(),
-                            cudaMemcpyHostToDevice, s));
-  if (!big.empty())
-    TS_CUDA(cudaMemcpyAsync(plan.big.get(), big.data(), sizeof(int32_t) * big.size(), cudaMemcpyHostToDevice, s));
-  if (plan.entries > 0)
-    TS_CUDA(cudaMemcpyAsync(dperm.get(), perm.data(), sizeof(int64_t) * perm.size(), cudaMemcpyHostToDevice, s));
-  const int g = (int)std::min<int64_t>(8192, std::max<int64_t>(1, (plan.entries + 255) / 256));
-  if (P16_dev) {
-    TS_TRY(plan.PS16.alloc((size_t)plan.entries));
-    if (plan.entries > 0)
-      k_plan_gather<bf16><<<g, 256, 0, s>>>(plan.entries, dperm.get(), col_dev, P16_dev, plan.colS.get(),
-                                            plan.PS16.get());
-  } else {
-    TS_TRY(plan.PS.alloc((size_t)plan.entries));
-    if (plan.entries > 0)
-      k_plan_gather<float><<<g, 256, 0, s>>>(plan.entries, dperm.get(), col_dev, P_dev, plan.colS.get(),
-                                             plan.PS.get());
-  }
-  TS_CUDA(cudaGetLastError());
-  TS_CUDA(cudaStreamSynchronize(s));  // dperm is freed on return
-  plan.ready = true;
-  return TSGNE_OK;
+tsgne_status find_heavy_rows(int n, const int64_t* rp, HeavyStore& hs, cudaStream_t s) {
+  return build_row_schedule(n, rp, nullptr, nullptr, nullptr, hs, nullptr, s);
+}
+
+tsgne_status build_attract_plan(int n, const int64_t* rp, const int32_t* col, const float* P, const bf16* P16,
+                                HeavyStore& hs, AttractPlan& plan, cudaStream_t s) {
+  return build_row_schedule(n, rp, col, P, P16, hs, &plan, s);
 }
 
 PlanView AttractPlan::view() const {

@@ -23,7 +23,6 @@
 //   fixed-order totals; KL = first + second * ln Z on the host (Eq. 5 with
 //   q = w / Z).
 #include <cmath>
-#include <vector>
 
 #include "reduce.cuh"
 #include "row_update.cuh"
@@ -214,27 +213,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-__global__ void k_heavy_bounds(int H, const int32_t* __restrict__ rows, const int64_t* __restrict__ rp,
-                               int64_t* __restrict__ bounds) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < H; k += gridDim.x * blockDim.x) {
-    bounds[k] = rp[rows[k]];
-    bounds[H + k] = rp[rows[k] + 1];
-  }
-}
-
-__global__ void k_heavy_flags(int n, const int64_t* __restrict__ rp, int32_t* __restrict__ flag) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    flag[i] = (rp[i + 1] - rp[i]) > kHeavyDeg ? 1 : 0;
-}
-
-__global__ void k_heavy_scatter(int n, const int32_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                                int32_t* __restrict__ rows) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    if (flag[i]) rows[pos[i]] = (int32_t)i;
-}
-
 // F^r_i from the fixed-point accumulators (one rounding of the exact integer
 // sum), which are cleared for the next pass; one thread per point.
 __global__ void __launch_bounds__(kAttrCta)
@@ -373,68 +351,6 @@ tsgne_status launch_prefetch_l2(const void* p, int64_t bytes, cudaStream_t s) {
   const int g = (int)((lines + 255) / 256 < 2048 ? (lines + 255) / 256 : 2048);
   k_prefetch_l2<<<g, 256, 0, s>>>(static_cast<const char*>(p), bytes);
   TS_CUDA(cudaGetLastError());
-  return TSGNE_OK;
-}
-
-tsgne_status find_heavy_rows(int n, const int64_t* rp, HeavyStore& hs, cudaStream_t s) {
-  DevBuf<int32_t> flag;
-  DevBuf<int64_t> pos, scr;
-  TS_TRY(flag.alloc((size_t)n));
-  TS_TRY(pos.alloc((size_t)n + 1));
-  TS_TRY(scr.alloc(scan_scratch_bytes(n) / sizeof(int64_t)));
-  const int g = grid_rows(n, 256) < 4096 ? grid_rows(n, 256) : 4096;
-  k_heavy_flags<<<g, 256, 0, s>>>(n, rp, flag.get());
-  TS_TRY(scan_i32_to_i64(flag.get(), pos.get(), n, scr.get(), s));
-  int64_t total = 0;
-  TS_CUDA(cudaMemcpyAsync(&total, pos.get() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  TS_CUDA(cudaStreamSynchronize(s));
-  const int H = (int)total;
-  hs.count = H;
-  TS_TRY(hs.rows.alloc((size_t)(H > 0 ? H : 1)));
-  if (H > 0) k_heavy_scatter<<<g, 256, 0, s>>>(n, flag.get(), pos.get(), hs.rows.get());
-  TS_CUDA(cudaGetLastError());
-  // chunk lists on the host (the hub rows are few)
-  std::vector<int32_t> rows(H > 0 ? H : 1);
-  std::vector<int64_t> b(H > 0 ? H : 1), e(H > 0 ? H : 1);
-  if (H > 0) {
-    DevBuf<int64_t> bounds;
-    TS_TRY(bounds.alloc(2 * (size_t)H));
-    k_heavy_bounds<<<(H + 255) / 256, 256, 0, s>>>(H, hs.rows.get(), rp, bounds.get());
-    TS_CUDA(cudaGetLastError());
-    TS_CUDA(cudaMemcpyAsync(rows.data(), hs.rows.get(), sizeof(int32_t) * H, cudaMemcpyDeviceToHost, s));
-    TS_CUDA(cudaMemcpyAsync(b.data(), bounds.get(), sizeof(int64_t) * H, cudaMemcpyDeviceToHost, s));
-    TS_CUDA(cudaMemcpyAsync(e.data(), bounds.get() + H, sizeof(int64_t) * H, cudaMemcpyDeviceToHost, s));
-    TS_CUDA(cudaStreamSynchronize(s));
-  }
-  std::vector<int32_t> off(1, 0), crow, cheavy;
-  std::vector<int64_t> cb, ce;
-  for (int k = 0; k < H; ++k) {
-    for (int64_t x = b[k]; x < e[k]; x += kHeavyChunk) {
-      crow.push_back(rows[k]);
-      cheavy.push_back(k);
-      cb.push_back(x);
-      ce.push_back(x + kHeavyChunk < e[k] ? x + kHeavyChunk : e[k]);
-    }
-    off.push_back((int32_t)crow.size());
-  }
-  const int C = (int)crow.size();
-  hs.chunks = C;
-  TS_TRY(hs.chunk_off.alloc(off.size()));
-  TS_TRY(hs.chunk_row.alloc((size_t)(C > 0 ? C : 1)));
-  TS_TRY(hs.chunk_begin.alloc((size_t)(C > 0 ? C : 1)));
-  TS_TRY(hs.chunk_end.alloc((size_t)(C > 0 ? C : 1)));
-  TS_TRY(hs.fa.alloc((size_t)(C > 0 ? C : 1)));
-  TS_TRY(hs.chunk_heavy.alloc((size_t)(C > 0 ? C : 1)));
-  TS_TRY(hs.arrivals.alloc((size_t)(H > 0 ? H : 1)));
-  TS_CUDA(cudaMemsetAsync(hs.arrivals.get(), 0, sizeof(uint32_t) * (size_t)(H > 0 ? H : 1), s));
-  TS_CUDA(cudaMemcpyAsync(hs.chunk_off.get(), off.data(), sizeof(int32_t) * off.size(), cudaMemcpyHostToDevice, s));
-  if (C > 0) {
-    TS_CUDA(cudaMemcpyAsync(hs.chunk_heavy.get(), cheavy.data(), sizeof(int32_t) * C, cudaMemcpyHostToDevice, s));
-    TS_CUDA(cudaMemcpyAsync(hs.chunk_row.get(), crow.data(), sizeof(int32_t) * C, cudaMemcpyHostToDevice, s));
-    TS_CUDA(cudaMemcpyAsync(hs.chunk_begin.get(), cb.data(), sizeof(int64_t) * C, cudaMemcpyHostToDevice, s));
-    TS_CUDA(cudaMemcpyAsync(hs.chunk_end.get(), ce.data(), sizeof(int64_t) * C, cudaMemcpyHostToDevice, s));
-  }
-  TS_CUDA(cudaStreamSynchronize(s));
   return TSGNE_OK;
 }
 

@@ -311,6 +311,7 @@ struct HeavyStore {
     return h;
   }
 };
+// The hub rows of a structure (attract_plan.cu).  Synchronises the stream.
 tsgne_status find_heavy_rows(int n, const int64_t* rp, HeavyStore& hs, cudaStream_t s);
 // L2 prefetch of a buffer (no-op below 1 MB).
 tsgne_status launch_prefetch_l2(const void* p, int64_t bytes, cudaStream_t s);
@@ -377,11 +378,10 @@ struct AttractPlan {
   bool ready = false;
   PlanView view() const;
 };
-// Builds the plan for the structure (rp, col) and P (FP32, or its BF16 copy
-// when P16 is not NULL); hs must hold the hub rows of the same structure.
-// Synchronises the stream.
+// Builds the hub rows and the plan for the structure (rp, col) and P (FP32,
+// or its BF16 copy when P16 is not NULL).  Synchronises the stream.
 tsgne_status build_attract_plan(int n, const int64_t* rp, const int32_t* col, const float* P,
-                                const __nv_bfloat16* P16, const HeavyStore& hs, AttractPlan& plan, cudaStream_t s);
+                                const __nv_bfloat16* P16, HeavyStore& hs, AttractPlan& plan, cudaStream_t s);
 // The attraction + update pass on the plan (the update mode of
 // k_attract: same results, bit for bit).
 tsgne_status launch_attract_plan(const AttractArgs& a, const PlanView& pv, cudaStream_t s);
