@@ -232,7 +232,7 @@ tsgne_status tsgne_set_state(tsgne_ctx* ctx, const float* Y, const float* update
  * of each kernel class since the last reset, measured with CUDA events on
  * the context's stream.  Classes: 0 repulsion (the tree walk when
  * cfg.repulsion = 1), 1 attraction+update (hub-row chunks included), 2
- * gradient export, 3 KL, 4 build, 5 repulsion force conversion, 6 hub-row
+ * gradient export, 3 KL, 4 build, 5 sum of the ordered pass's partial forces, 6 hub-row
  * attraction chunks of the gradient export, 7 tree build
  * (bounding box, keys, sort, tree, summaries).  ms and launches hold n
  * entries (n <= 8).
@@ -268,7 +268,9 @@ tsgne_status tsgne_repulsion_shape(tsgne_ctx* ctx, int32_t* grid, int32_t* block
  * 16 i-points, 2 warps once the tile pairs fill four waves of the grid);
  * symmetric = 0: the ordered-pair kernel (every ordered pair, partial forces
  * per j-chunk; FP32 storage only; tile_warps / i_per_lane ignored).  Results
- * depend on the shape only through the order of FP32 partial sums.
+ * depend on the shape only through the order of FP32 partial sums.  Layouts
+ * of at most 45,056 points have one symmetric shape of their own, fixed by
+ * their size, which every symmetric request selects.
  * tsgne_autotune times trial_passes repulsion passes of each shape (in the
  * order (2, 16, 1), (1, 16, 1), (2, 8, 1), (1, 8, 1), (-, -, 0); -1 in
  * ms_per_pass, 5 floats, for a shape that does not apply), keeps the
@@ -372,7 +374,8 @@ tsgne_status tsgne_batch_set_tile(tsgne_batch* b, int32_t tile_warps);
 /* Changes the shape of the batched exact pass: tile_warps 1, 2 or 4 warps
  * per CTA and i_per_lane 8 or 16 i-points per lane (the tile is 32 x
  * i_per_lane x tile_warps points; 8 i-points need half the registers, so
- * twice as many warps per SM are launched).  Members' states are kept; a
+ * twice as many warps per SM are launched).  Members of at most 45,056
+ * points keep the shape of their own.  Members' states are kept; a
  * member's results depend on the shape (the order of its FP32 partial sums)
  * but not on the other members. */
 tsgne_status tsgne_batch_set_shape(tsgne_batch* b, int32_t tile_warps, int32_t i_per_lane);
@@ -515,9 +518,8 @@ tsgne_status tsgne_server_usage(tsgne_server* s, int64_t* used_bytes, int32_t* r
  * One layout over several GPUs (one context per GPU, same P and layout on
  * every context).  The paper runs on one CPU and describes no distribution;
  * the split follows from the form of Eq. 4: the repulsive forces and Z are
- * sums over the unordered pairs, which the exact pass evaluates in tile
- * pairs ("units", nt (nt + 1) / 2 of them for nt tiles of the layout), so the
- * units can be divided among contexts and the sums added afterwards.  Each
+ * sums over pairs, which the exact pass evaluates in "units" (nt (nt + 1) / 2
+ * tile pairs for nt tiles of a large layout), so the units can be divided among contexts and the sums added afterwards.  Each
  * context holds the whole (O(n + nnz)) state and updates every row itself;
  * only the O(n^2) repulsion is divided.
  *

@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "row_update.cuh"
 #include "storage.cuh"
 #include "tsgne_internal.cuh"
 
@@ -128,7 +129,11 @@ struct tsgne_ctx {
   int shard_u0 = 0, shard_u1 = 0;
   bool shard_pending = false;  // a share was enqueued and awaits its finish call
 
-  cudaGraphExec_t g2[2] = {nullptr, nullptr};  // two iterations starting from buffer 0 / 1
+  // slot of the symmetric pass's sums in Sched: the next pass's, and the last one's
+  int zslot = 0, zpass = 0;
+
+  cudaGraphExec_t g2[4] = {nullptr, nullptr, nullptr, nullptr};  // two iterations, by buffer and slot at their start
+  int graph_key() const { return 2 * cur + zslot; }
 
   std::vector<ProfRec> pending;
   std::vector<cudaEvent_t> spare;
@@ -265,6 +270,12 @@ tsgne_status prof_end(tsgne_ctx* ctx, ProfRec* rec) {
 
 // ------------------------------------------------------------- iteration
 
+// The sums of the symmetric pass just enqueued are in slot zpass; the next one uses the other.
+void close_pass(tsgne_ctx* ctx) {
+  ctx->zpass = ctx->zslot;
+  ctx->zslot ^= 1;
+}
+
 tsgne_status enqueue_repulsion(tsgne_ctx* ctx, int advance) {
   const tsgne_config& c = ctx->cfg;
   ProfRec pr;
@@ -291,13 +302,25 @@ tsgne_status enqueue_repulsion(tsgne_ctx* ctx, int advance) {
     return prof_end(ctx, &pr2);
   }
   TS_TRY(launch_repulsion_sym(ctx->shape, ctx->n, ctx->Yread(ctx->cur), ctx->bf16 ? 1 : 0, ctx->facc.get(),
-                              ctx->zpart.get(), ctx->sched.get(), advance, c.early_exag, c.ee_iters, c.momentum0,
+                              ctx->sched.get(), ctx->zslot, advance, c.early_exag, c.ee_iters, c.momentum0,
                               c.momentum1, ctx->stream));
-  TS_TRY(prof_end(ctx, &pr));
-  ProfRec pr2;
-  TS_TRY(prof_begin(ctx, 5, &pr2));
-  TS_TRY(launch_fix_forces(ctx->n, ctx->facc.get(), ctx->fsum.get(), ctx->stream));
-  return prof_end(ctx, &pr2);
+  close_pass(ctx);
+  return prof_end(ctx, &pr);
+}
+
+bool symmetric_pass(const tsgne_ctx* ctx) { return !ctx->use_tree && !ctx->ordered; }
+
+// After a pass whose forces no row takes (the rows clear the accumulators).
+tsgne_status discard_forces(tsgne_ctx* ctx) {
+  if (!symmetric_pass(ctx)) return TSGNE_OK;
+  TS_CUDA(cudaMemsetAsync(ctx->facc.get(), 0, 2 * (size_t)ctx->n * sizeof(unsigned long long), ctx->stream));
+  return TSGNE_OK;
+}
+
+// Z of the last pass, from a copy of the device's scalars.
+double host_z(const tsgne_ctx* ctx, const Sched& h) {
+  if (!symmetric_pass(ctx)) return h.Z;
+  return z_of(h.zacc[ctx->zpass][0], h.zacc[ctx->zpass][1], h.zbad[ctx->zpass], ctx->n);
 }
 
 // Reads of the current layout / P for the force kernels of the context.
@@ -311,9 +334,13 @@ AttractArgs attract_args(tsgne_ctx* ctx) {
   a.Yr = ctx->Yread(ctx->cur);
   a.y_bf16 = ctx->bf16 ? 1 : 0;
   a.Ym = ctx->Y[ctx->cur].get();
-  a.frep = ctx->fsum.get();
-  a.chunks = 1;
-  a.n_pad = ctx->shape.n_pad;
+  if (symmetric_pass(ctx)) {
+    a.facc = ctx->facc.get();
+    a.unscale = fix_unscale(ctx->n);
+    a.zslot = ctx->zpass;
+  } else {
+    a.frep = ctx->fsum.get();
+  }
   a.sched = ctx->sched.get();
   a.hv = ctx->heavy();
   return a;
@@ -399,25 +426,29 @@ tsgne_status check_flags(tsgne_ctx* ctx) {
 
 bool capturable(cudaStream_t s) { return s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread; }
 
-tsgne_status ensure_graph(tsgne_ctx* ctx, int start) {
-  if (ctx->g2[start]) return TSGNE_OK;
-  const int saved = ctx->cur;
-  ctx->cur = start;
+// The graph of two iterations from the context's current buffer and slot
+// (both are the same again after them).
+tsgne_status ensure_graph(tsgne_ctx* ctx) {
+  cudaGraphExec_t& exec = ctx->g2[ctx->graph_key()];
+  if (exec) return TSGNE_OK;
+  const int cur = ctx->cur, zslot = ctx->zslot, zpass = ctx->zpass;
   cudaGraph_t g = nullptr;
   TS_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
   tsgne_status st = enqueue_step(ctx);
   if (st == TSGNE_OK) st = enqueue_step(ctx);
   cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
-  ctx->cur = saved;
+  ctx->cur = cur;
+  ctx->zslot = zslot;
+  ctx->zpass = zpass;
   if (st != TSGNE_OK) {
     if (g) cudaGraphDestroy(g);
     return st;
   }
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture", __FILE__, __LINE__);
-  e = cudaGraphInstantiate(&ctx->g2[start], g, 0);
+  e = cudaGraphInstantiate(&exec, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
-    ctx->g2[start] = nullptr;
+    exec = nullptr;
     return cuda_fail(e, "cudaGraphInstantiate", __FILE__, __LINE__);
   }
   return TSGNE_OK;
@@ -500,6 +531,7 @@ tsgne_status reset_optimizer(tsgne_ctx* ctx, int32_t t) {
   Sched h{};
   h.t = t;
   TS_CUDA(cudaMemcpyAsync(ctx->sched.get(), &h, sizeof(Sched), cudaMemcpyHostToDevice, ctx->stream));
+  ctx->zslot = ctx->zpass = 0;
   return TSGNE_OK;
 }
 
@@ -778,8 +810,10 @@ tsgne_status tsgne_run(tsgne_ctx* ctx, int32_t n_iter) {
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   int32_t k = 0;
   if (!ctx->cfg.profile && capturable(ctx->stream) && n_iter >= 2) {
-    API_TRY(ctx, ensure_graph(ctx, ctx->cur));
-    for (; k + 2 <= n_iter; k += 2) API_CUDA(ctx, cudaGraphLaunch(ctx->g2[ctx->cur], ctx->stream));
+    API_TRY(ctx, ensure_graph(ctx));
+    cudaGraphExec_t two = ctx->g2[ctx->graph_key()];
+    for (; k + 2 <= n_iter; k += 2) API_CUDA(ctx, cudaGraphLaunch(two, ctx->stream));
+    if (symmetric_pass(ctx)) ctx->zpass = ctx->zslot ^ 1;
   }
   for (; k < n_iter; ++k) API_TRY(ctx, enqueue_step(ctx));
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -807,10 +841,11 @@ tsgne_status tsgne_kl(tsgne_ctx* ctx, double* kl_out) {
                          ctx->Yread(ctx->cur), ctx->bf16 ? 1 : 0, ctx->klpart.get(), kl_partial_count(ctx->sms),
                          ctx->sched.get(), ctx->stream));
   API_TRY(ctx, prof_end(ctx, &pr));
+  API_TRY(ctx, discard_forces(ctx));
   Sched h;
   API_TRY(ctx, read_sched(ctx, &h));
   API_TRY(ctx, check_tree_flags(ctx, h));
-  *kl_out = h.red[0] + h.red[1] * std::log(h.Z);
+  *kl_out = h.red[0] + h.red[1] * std::log(host_z(ctx, h));
   if (!std::isfinite(*kl_out)) return fail(ctx, TSGNE_ERR_NONFINITE, "KL is not finite");
   return TSGNE_OK;
 }
@@ -829,7 +864,7 @@ tsgne_status tsgne_gradient(tsgne_ctx* ctx, float alpha, float* g_out, double* z
   Sched h;
   API_TRY(ctx, read_sched(ctx, &h));
   API_TRY(ctx, check_tree_flags(ctx, h));
-  if (z_out) *z_out = h.Z;
+  if (z_out) *z_out = host_z(ctx, h);
   return TSGNE_OK;
 }
 
@@ -998,6 +1033,7 @@ tsgne_status tsgne_autotune(tsgne_ctx* ctx, int32_t trial_passes, int32_t* tile_
     if (st == TSGNE_OK) st = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess ? TSGNE_OK : TSGNE_ERR_CUDA;
     if (st != TSGNE_OK) break;
     ms /= (float)trial_passes;
+    if ((st = discard_forces(ctx)) != TSGNE_OK) break;
     if (ms_per_pass) ms_per_pass[k] = ms;
     if (best < 0 || ms < best_ms) {
       best = k;
@@ -1050,8 +1086,8 @@ tsgne_status tsgne_shard_repulsion(tsgne_ctx* ctx, int64_t* units, int32_t* u0, 
   ProfRec pr;
   API_TRY(ctx, prof_begin(ctx, 0, &pr));
   API_TRY(ctx, launch_repulsion_sym_units(ctx->shape, ctx->n, ctx->Yread(ctx->cur), ctx->bf16 ? 1 : 0,
-                                          ctx->facc.get(), ctx->zpart.get(), ctx->sched.get(), ctx->shard_u0,
-                                          ctx->shard_u1, ctx->stream));
+                                          ctx->facc.get(), ctx->zpart.get(), ctx->sched.get(), ctx->zslot,
+                                          ctx->shard_u0, ctx->shard_u1, ctx->stream));
   API_TRY(ctx, prof_end(ctx, &pr));
   ctx->shard_pending = true;
   if (units) *units = U;
@@ -1064,15 +1100,12 @@ tsgne_status tsgne_shard_repulsion(tsgne_ctx* ctx, int64_t* units, int32_t* u0, 
 }
 
 namespace {
-// Z, schedule and F^r after the shares were summed (advance: an iteration).
+// Z and schedule after the shares were summed (advance: an iteration).
 tsgne_status shard_close(tsgne_ctx* ctx, int advance) {
   const tsgne_config& c = ctx->cfg;
-  TS_TRY(launch_finalize_z(ctx->shape, ctx->n, ctx->zpart.get(), ctx->sched.get(), advance, c.early_exag, c.ee_iters,
-                           c.momentum0, c.momentum1, ctx->stream));
-  ProfRec pr;
-  TS_TRY(prof_begin(ctx, 5, &pr));
-  TS_TRY(launch_fix_forces(ctx->n, ctx->facc.get(), ctx->fsum.get(), ctx->stream));
-  TS_TRY(prof_end(ctx, &pr));
+  TS_TRY(launch_finalize_z(ctx->shape, ctx->zpart.get(), ctx->sched.get(), ctx->zslot, advance, c.early_exag,
+                           c.ee_iters, c.momentum0, c.momentum1, ctx->stream));
+  close_pass(ctx);
   ctx->shard_pending = false;
   return TSGNE_OK;
 }
@@ -1098,7 +1131,7 @@ tsgne_status tsgne_shard_gradient_finish(tsgne_ctx* ctx, float alpha, float* g_o
   API_TRY(ctx, copy_out(g_out, ctx->grad.get(), sizeof(float2) * (size_t)ctx->n, ptr_kind, ctx->stream));
   Sched h;
   API_TRY(ctx, read_sched(ctx, &h));
-  if (z_out) *z_out = h.Z;
+  if (z_out) *z_out = host_z(ctx, h);
   return TSGNE_OK;
 }
 

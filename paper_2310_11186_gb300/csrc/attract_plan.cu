@@ -44,7 +44,7 @@ namespace tsgne {
 namespace {
 
 constexpr int kPlanThreads = 256;
-constexpr int kShortRowsPerCta = 256;
+constexpr int kShortRowsPerCta = 256;  // at most (short_rows)
 constexpr int kMedRowsPerCta = 64;
 constexpr int kSlotsShort = 8;
 constexpr int kSlotsMed = 32;
@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
     k_attract_plan(AttractArgs a, PlanView pv, int big_blocks) {
   __shared__ float2 spart[kPartials];
   __shared__ float2 sfa[kMedRowsPerCta];
+  __shared__ float s_invz;
+  const RowForce rf{a.frep, a.facc, a.unscale};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const PT* __restrict__ P = static_cast<const PT*>(a.P);
   const YT* __restrict__ Y = static_cast<const YT*>(a.Yr);
@@ -111,8 +113,8 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
             sx += f.x;
             sy += f.y;
           }
-          finish_row<false>(i, make_float2(sx, sy), a.frep, a.chunks, a.n_pad, a.sched, 0.f, nullptr, a.Ym,
-                            a.Ynext, Ynext16, a.upd, a.gains, a.eta, a.min_gain);
+          finish_row<false>(i, make_float2(sx, sy), rf, pass_inv_z(a.sched, a.zslot, a.n), a.sched, 0.f, nullptr,
+                            a.Ym, a.Ynext, Ynext16, a.upd, a.gains, a.eta, a.min_gain);
         }
       }
     }
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
   const bool med = cb < pv.n_med;
   const PlanCta m = med ? pv.med[cb] : pv.shorts[cb - pv.n_med];
   const int shift = med ? 5 : 3;
-  const int64_t row0 = med ? 0 : (int64_t)(cb - pv.n_med) * kShortRowsPerCta;
+  const int64_t row0 = med ? 0 : (int64_t)(cb - pv.n_med) * pv.short_rows;
   {
     const int64_t tot = (int64_t)m.cnt[0] + m.cnt[1] + m.cnt[2] + m.cnt[3];
     prefetch_range(pv.code + m.pair, pv.code + m.pair + m.cnt[0], tid, kPlanThreads);
@@ -132,14 +134,16 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
     prefetch_range(PS + m.ent, PS + m.ent + tot, tid, kPlanThreads);
   }
   if (!med) {
-    const int64_t r1 = row0 + kShortRowsPerCta < a.n ? row0 + kShortRowsPerCta : a.n;
+    const int64_t r1 = row0 + m.nrows;
     prefetch_range(a.rp + row0, a.rp + r1 + 1, tid, kPlanThreads);
-    prefetch_range(a.frep + row0, a.frep + r1, tid, kPlanThreads);
+    if (a.facc) prefetch_range(a.facc + 2 * row0, a.facc + 2 * r1, tid, kPlanThreads);
+    else prefetch_range(a.frep + row0, a.frep + r1, tid, kPlanThreads);
     prefetch_range(a.upd + row0, a.upd + r1, tid, kPlanThreads);
     prefetch_range(a.gains + row0, a.gains + r1, tid, kPlanThreads);
     prefetch_range(a.Ym + row0, a.Ym + r1, tid, kPlanThreads);
   }
-  for (int k = tid; k < kPartials; k += kPlanThreads) spart[k] = make_float2(0.f, 0.f);
+  if (tid == 0) s_invz = pass_inv_z(a.sched, a.zslot, a.n);
+  for (int k = tid; k < m.nrows << shift; k += kPlanThreads) spart[k] = make_float2(0.f, 0.f);
   __syncthreads();
 
   // the chains: thread per chain, every entry's loads issued up front
@@ -175,8 +179,8 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
   __syncthreads();
 
   if (!med) {  // one thread per row of at most 32 entries: slots in butterfly order, then the update
+    if (tid >= m.nrows) return;
     const int64_t i = row0 + tid;
-    if (i >= a.n) return;
     if (a.rp[i + 1] - a.rp[i] > kHeavyDeg) return;  // a medium or big CTA updates it
     const float2* sp = spart + tid * kSlotsShort;
     float2 a0 = sp[0], a1 = sp[1], t = sp[4];
@@ -192,8 +196,8 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
     a0 = make_float2(a0.x + a2.x, a0.y + a2.y);  // o = 2
     a1 = make_float2(a1.x + a3.x, a1.y + a3.y);
     const float2 fa = make_float2(a0.x + a1.x, a0.y + a1.y);  // o = 1
-    finish_row<false>(i, fa, a.frep, a.chunks, a.n_pad, a.sched, 0.f, nullptr, a.Ym, a.Ynext, Ynext16, a.upd,
-                      a.gains, a.eta, a.min_gain);
+    finish_row<false>(i, fa, rf, s_invz, a.sched, 0.f, nullptr, a.Ym, a.Ynext, Ynext16, a.upd, a.gains, a.eta,
+                      a.min_gain);
     return;
   }
   // medium rows: the 32 chains of a row with the chunk warps' shuffle
@@ -205,8 +209,8 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
   }
   __syncthreads();
   if (tid < m.nrows && TS_IN(m.rows + tid, 0, pv.n_med_rows, dbg))
-    finish_row<false>(pv.med_rows[m.rows + tid], sfa[tid], a.frep, a.chunks, a.n_pad, a.sched, 0.f, nullptr, a.Ym,
-                      a.Ynext, Ynext16, a.upd, a.gains, a.eta, a.min_gain);
+    finish_row<false>(pv.med_rows[m.rows + tid], sfa[tid], rf, s_invz, a.sched, 0.f, nullptr, a.Ym, a.Ynext, Ynext16,
+                      a.upd, a.gains, a.eta, a.min_gain);
 }
 
 // ------------------------------------------------ building the schedule
@@ -252,12 +256,12 @@ __device__ __forceinline__ RowAdds row_adds(int64_t d) {
 
 // tot[list][block] = sum of the block's rows.
 __global__ void __launch_bounds__(kPlanThreads)
-    k_row_totals(int n, const int64_t* __restrict__ rp, int nb, int64_t* __restrict__ tot) {
+    k_row_totals(int n, const int64_t* __restrict__ rp, int per, int nb, int64_t* __restrict__ tot) {
   __shared__ uint32_t sum[kRowLists];
   if (threadIdx.x < kRowLists) sum[threadIdx.x] = 0u;
   __syncthreads();
-  const int64_t i = (int64_t)blockIdx.x * kPlanThreads + threadIdx.x;
-  const RowAdds a = row_adds(i < n ? rp[i + 1] - rp[i] : 0);
+  const int64_t i = (int64_t)blockIdx.x * per + threadIdx.x;
+  const RowAdds a = row_adds((int)threadIdx.x < per && i < n ? rp[i + 1] - rp[i] : 0);
 #pragma unroll
   for (int f = 0; f < kRowLists; ++f) {
     const uint32_t w = __reduce_add_sync(0xffffffffu, a.v[f]);
@@ -307,12 +311,13 @@ __global__ void __launch_bounds__(1024) k_row_scan(int nb, int64_t* __restrict__
 // The lists of rows and chunks (see HeavyStore and AttractPlan).  med_ent
 // (NULL: no plan wanted): first entry, in the copies, of each medium CTA.
 __global__ void __launch_bounds__(kPlanThreads)
-    k_row_lists(int n, const int64_t* __restrict__ rp, int nb, const int64_t* __restrict__ tot,
+    k_row_lists(int n, const int64_t* __restrict__ rp, int per, int nb, const int64_t* __restrict__ tot,
                 int32_t* __restrict__ rows, int32_t* __restrict__ chunk_off, int32_t* __restrict__ chunk_row,
                 int32_t* __restrict__ chunk_heavy, int64_t* __restrict__ chunk_begin, int64_t* __restrict__ chunk_end,
                 int32_t* __restrict__ med_rows, int64_t* __restrict__ med_ent, int32_t* __restrict__ big) {
-  const int64_t i = (int64_t)blockIdx.x * kPlanThreads + threadIdx.x;
-  const int64_t a = i < n ? rp[i] : 0, b = i < n ? rp[i + 1] : 0;
+  const int64_t i = (int64_t)blockIdx.x * per + threadIdx.x;
+  const bool mine = (int)threadIdx.x < per && i < n;
+  const int64_t a = mine ? rp[i] : 0, b = mine ? rp[i + 1] : 0;
   const RowAdds ra = row_adds(b - a);
   if (!__syncthreads_or((int)ra.v[kHeavyRows])) return;
   uint32_t ex[kRowLists], all;
@@ -348,7 +353,7 @@ template <class PT>
 __global__ void __launch_bounds__(kPlanThreads)
     k_plan_chains(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const PT* __restrict__ P,
                   int n_med, int64_t n_med_rows, int64_t med_entries, const int32_t* __restrict__ med_rows,
-                  const int64_t* __restrict__ med_ent, int nb, const int64_t* __restrict__ tot,
+                  const int64_t* __restrict__ med_ent, int per, int nb, const int64_t* __restrict__ tot,
                   PlanCta* __restrict__ cta, uint16_t* __restrict__ code, int32_t* __restrict__ colS,
                   PT* __restrict__ PS) {
   __shared__ int64_t sfirst[kPartials];  // first entry of each chain, in chain order
@@ -367,8 +372,8 @@ __global__ void __launch_bounds__(kPlanThreads)
     nrows = (int)min((int64_t)kMedRowsPerCta, n_med_rows - r0);
     if (tid < nrows) i = med_rows[r0 + tid];
   } else {
-    r0 = (int64_t)c * kShortRowsPerCta;
-    nrows = (int)min((int64_t)kShortRowsPerCta, (int64_t)n - r0);
+    r0 = (int64_t)c * per;
+    nrows = (int)min((int64_t)per, (int64_t)n - r0);
     if (tid < nrows) i = r0 + tid;
   }
   int64_t a = 0, d = 0;
@@ -435,14 +440,29 @@ __global__ void __launch_bounds__(kPlanThreads)
   if (tid == 0) cta[blockIdx.x] = pc;
 }
 
+// Rows of a short CTA: the fewest (a power of two, at least 32) that still
+// make one wave of the 6 CTAs an SM holds.  A CTA is a chain of dependent
+// loads, so few rows per CTA shorten small passes (2,000 points: 10.5 us with
+// 128 rows, 8.7 us with 32; 30,000: 13.3 us with 256, 11.1 us with 64) and a
+// second wave costs more than that (130,000: 20.8 us with 128, 18.8 us with 256).
+int short_rows(int n, int sms) {
+  int r = 32;
+  while (r < kShortRowsPerCta && (n + r - 1) / r > 6 * sms) r *= 2;
+  return r;
+}
+
 // The hub rows of a structure and, if plan is not NULL, the schedule.
 tsgne_status build_row_schedule(int n, const int64_t* rp, const int32_t* col, const float* P, const bf16* P16,
                                 HeavyStore& hs, AttractPlan* plan, cudaStream_t s) {
-  const int nb = (n + kPlanThreads - 1) / kPlanThreads;
+  int dev = 0, sms = 1;
+  TS_CUDA(cudaGetDevice(&dev));
+  TS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int per = plan ? short_rows(n, sms) : kShortRowsPerCta;
+  const int nb = (n + per - 1) / per;
   DevBuf<int64_t> tot, med_ent;
   TS_TRY(tot.alloc((size_t)nb * kRowLists + kRowLists));
   int64_t* const sums = tot.get() + (size_t)nb * kRowLists;
-  k_row_totals<<<nb, kPlanThreads, 0, s>>>(n, rp, nb, tot.get());
+  k_row_totals<<<nb, kPlanThreads, 0, s>>>(n, rp, per, nb, tot.get());
   k_row_scan<<<kRowLists, 1024, 0, s>>>(nb, tot.get(), sums);
   TS_CUDA(cudaGetLastError());
   int64_t h[kRowLists];
@@ -465,6 +485,7 @@ tsgne_status build_row_schedule(int n, const int64_t* rp, const int32_t* col, co
     *plan = AttractPlan();
     plan->n_med = (int)((h[kMedRows] + kMedRowsPerCta - 1) / kMedRowsPerCta);
     plan->n_short = nb;
+    plan->short_rows = per;
     plan->n_big = (int)h[kBigChunks];
     plan->n_med_rows = h[kMedRows];
     plan->n_codes = h[kMedRows] * kSlotsMed + h[kCodes];
@@ -479,7 +500,7 @@ tsgne_status build_row_schedule(int n, const int64_t* rp, const int32_t* col, co
     else TS_TRY(plan->PS.alloc((size_t)plan->entries));
   }
   if (h[kHeavyRows] > 0)
-    k_row_lists<<<nb, kPlanThreads, 0, s>>>(n, rp, nb, tot.get(), hs.rows.get(), hs.chunk_off.get(),
+    k_row_lists<<<nb, kPlanThreads, 0, s>>>(n, rp, per, nb, tot.get(), hs.rows.get(), hs.chunk_off.get(),
                                             hs.chunk_row.get(), hs.chunk_heavy.get(), hs.chunk_begin.get(),
                                             hs.chunk_end.get(), plan ? plan->med_rows.get() : nullptr,
                                             plan ? med_ent.get() : nullptr, plan ? plan->big.get() : nullptr);
@@ -487,12 +508,12 @@ tsgne_status build_row_schedule(int n, const int64_t* rp, const int32_t* col, co
     const int grid = plan->n_med + plan->n_short;
     if (P16)
       k_plan_chains<bf16><<<grid, kPlanThreads, 0, s>>>(
-          n, rp, col, P16, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), nb,
-          tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS16.get());
+          n, rp, col, P16, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), per,
+          nb, tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS16.get());
     else
       k_plan_chains<float><<<grid, kPlanThreads, 0, s>>>(
-          n, rp, col, P, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), nb,
-          tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS.get());
+          n, rp, col, P, plan->n_med, plan->n_med_rows, h[kMedEntries], plan->med_rows.get(), med_ent.get(), per,
+          nb, tot.get(), plan->cta.get(), plan->code.get(), plan->colS.get(), plan->PS.get());
   }
   TS_CUDA(cudaGetLastError());
   TS_CUDA(cudaStreamSynchronize(s));  // tot and med_ent are freed on return
@@ -523,6 +544,7 @@ PlanView AttractPlan::view() const {
   v.n_med = n_med;
   v.n_short = n_short;
   v.n_big = n_big;
+  v.short_rows = short_rows;
   v.entries = entries;
   v.n_codes = n_codes;
   v.n_med_rows = n_med_rows;

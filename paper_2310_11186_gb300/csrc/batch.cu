@@ -1,22 +1,23 @@
 // Many layouts per launch: the t-SGNE iteration of every member of a batch
-// runs in four launches (five when a member has rows above 32 entries),
-// whatever the number and sizes of the members.
+// runs in at most six launches, whatever the number and sizes of the members.
 //
-//   k_batch_repulsion  one global work queue over the tile pairs of all
-//                      members (prefix offsets per member); each unit is the
-//                      same device code as the single-layout pass (sym_unit)
-//                      on that member's buffers, so every member's forces and
-//                      Z partials are the same bits as when it runs alone
-//   k_batch_finalize   one CTA per member: Z = fixed-order sum of its unit
-//                      partials minus n, schedule (alpha, mu) from its own
-//                      iteration counter t, t += 1
-//   k_batch_reduce     each point's fixed-point force accumulators to F^r,
-//                      cleared for the next iteration
+//   k_batch_small      the units of the members of at most kSmallPoints points
+//   k_batch_repulsion  one global work queue over the units of the larger ones
+//                      (prefix offsets per member; one launch for those of
+//                      at most kMidPoints points, one for the rest); each
+//                      unit is the same
+//                      device code as the single-layout pass (small_unit,
+//                      sym_unit) on that member's buffers, so every member's
+//                      forces and Z are the same bits as when it runs alone
+//   k_batch_finalize   one thread per member: Z from its fixed-point sums,
+//                      schedule (alpha, mu) from its own iteration counter t,
+//                      t += 1
 //   k_batch_hubs       (members with rows above 32 entries) one warp per
 //                      1024-entry chunk of such a row, over all members'
 //                      chunks: the single-layout path's chunk sums
-//   k_batch_attract    attraction + gradient + optimiser step per row (a hub
-//                      row adds its chunk sums in chunk order)
+//   k_batch_attract    F^r from the accumulators (cleared for the next
+//                      iteration), attraction + gradient + optimiser step per
+//                      row (a hub row adds its chunk sums in chunk order)
 //
 // Tree-code members (cfg.repulsion = 1, or per member through
 // tsgne_batch_add_ex) take no units of k_batch_repulsion: each runs the
@@ -30,8 +31,9 @@
 // Members keep their P, layout and optimiser state resident on the device
 // and may differ in size and in iteration count (each has its own t); the
 // current layout of a member is Y[t & 1], so one captured CUDA graph of the
-// launches serves every iteration of a given membership.  All members of
-// a batch use the same tile size T = 512 W; tsgne_batch_autotune picks W.
+// launches serves every iteration of a given membership.  All members of a
+// batch above kMidPoints points use the same tile size T = 512 W;
+// tsgne_batch_autotune picks W.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -59,19 +61,17 @@ struct GraphDesc {
   float2* gains;
   unsigned long long* acc;  // fixed-point force accumulators, 2 per point (scale fix_scale(n))
   float2* fsum;
-  double* zunit;
   Sched* sched;
   HeavyRows hv;  // rows above kHeavyDeg entries, in kHeavyChunk-entry chunks (as the single-layout path)
   int n, nt, n_pad, units;
   float eta;
   float fscale, funscale;
   int tree;  // 1: tree-code repulsion (no units; forces and Z from its walk)
-  int pad_;
+  int split;  // j sub-tiles per tile pair
 };
 
 struct BatchCtr {
-  uint32_t work_next;
-  uint32_t rep_done;
+  uint32_t work_next[2];  // queues of the mid and large members' tile pairs (cleared by k_batch_finalize)
 };
 
 namespace {
@@ -92,73 +92,81 @@ __device__ __forceinline__ int find_owner(const int* __restrict__ off, int count
 template <int W, int RI>
 __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
     k_batch_repulsion(const GraphDesc* __restrict__ descs, const int* __restrict__ unit_off, int members, int U,
-                      BatchCtr* ctr) {
+                      uint32_t* queue) {
   constexpr int T = W * 32 * RI;
+  constexpr int G = T / kGroup;
   extern __shared__ float4 smem[];
   float4* sj = smem;
   float2* sacc = reinterpret_cast<float2*>(smem + T);
+  longlong2* si = reinterpret_cast<longlong2*>(sacc + T);
   __shared__ int s_unit, s_g, s_a, s_b;
+  __shared__ u64 s_z[W];
   const int tid = threadIdx.x;
-  for (;;) {
+  for (bool first = true;; first = false) {
     if (tid == 0) {
-      const int u = (int)atomicAdd(&ctr->work_next, 1u);
-      int g = 0, a = 0, b = 0;
+      const int u = first ? (int)blockIdx.x : (int)(gridDim.x + atomicAdd(queue, 1u));
+      int g = 0;
+      int2 ab = make_int2(0, 0);
       if (u < U) {
         g = find_owner(unit_off, members, u);
-        unit_tiles(u - unit_off[g], descs[g].nt, &a, &b);
+        ab = unit_tiles(u - unit_off[g], descs[g].nt);
       }
       s_unit = u;
       s_g = g;
-      s_a = a;
-      s_b = b;
+      s_a = ab.x;
+      s_b = ab.y;
     }
     __syncthreads();
     const int u = s_unit, g = s_g, a = s_a, b = s_b;
     if (u >= U) break;
     const GraphDesc& d = descs[g];
     if (!(TS_IN(a, 0, d.nt, &d.sched->flags) && TS_IN(b, a, d.nt, &d.sched->flags))) {  // debug build only
-      if (tid == 0) d.zunit[u - unit_off[g]] = 0.0;
       __syncthreads();
       continue;
     }
     const float2* Y = d.Y[d.sched->t & 1];
-    const double zt = sym_unit<W, RI>(Y, d.n, d.acc, d.fscale, a, b, sj, sacc);
-    const double zb = block_sum_d(zt);
-    if (tid == 0) d.zunit[u - unit_off[g]] = zb;
+    bool bad;
+    u64 zt;
+    if (RI == 8 && d.split > 1) {  // only tiles of 8 i-points per lane are cut
+      zt = sym_units<W, 8, float2>(Y, d.n, d.acc, d.fscale, a, b, G / d.split, sj, sacc, si);
+      bad = zt == ~0ull;
+    } else {
+      zt = sym_unit<W, RI, float2, true>(Y, d.n, d.acc, d.fscale, a, b, 0, G, sj, sacc, &bad);
+    }
+    const u64 zb = cta_z<W>(bad ? 0ull : zt, &bad, s_z);
+    if (tid == 0) put_z(zb, bad, nullptr, d.sched->zacc[0], &d.sched->zbad[0]);
     __syncthreads();
   }
-  if (arrive_last(&ctr->rep_done) && tid == 0) ctr->work_next = 0u;
 }
 
-__global__ void k_batch_finalize(const GraphDesc* __restrict__ descs, float ee, int ee_iters, float mom0,
-                                 float mom1) {
-  const GraphDesc& d = descs[blockIdx.x];
-  if (d.tree) return;  // its walk set Z and the schedule
-  const double total = sum_partials(d.zunit, d.units);
-  if (threadIdx.x == 0) {
-    Sched* s = d.sched;
-    s->Z = total - (double)d.n;
-    s->inv_z = (float)(1.0 / s->Z);
-    const int t = s->t;
-    s->alpha = t < ee_iters ? ee : 1.0f;
-    s->mu = t < ee_iters ? mom0 : mom1;
-    s->t = t + 1;
-  }
+// The units of the small members (at most kSmallPoints points), one per CTA.
+__global__ void __launch_bounds__(32 * kSmallWarps)
+    k_batch_small(const GraphDesc* __restrict__ descs, const int* __restrict__ unit_off, int members) {
+  __shared__ float4 sj[kSmallMaxChunk];
+  __shared__ u64 s_z[kSmallWarps];
+  const int g = find_owner(unit_off, members, (int)blockIdx.x);
+  const GraphDesc& d = descs[g];
+  const int u = (int)blockIdx.x - unit_off[g], nc = small_chunks(d.n);
+  bool bad;
+  const u64 zt = small_unit<float2>(d.Y[d.sched->t & 1], d.n, d.acc, d.fscale, u / nc, u % nc, sj, &bad);
+  const u64 zb = cta_z<kSmallWarps>(zt, &bad, s_z);
+  if (threadIdx.x == 0) put_z(zb, bad, nullptr, d.sched->zacc[0], &d.sched->zbad[0]);
 }
 
-__global__ void k_batch_reduce(const GraphDesc* __restrict__ descs, const int* __restrict__ row_off, int members,
-                               int R) {
-  const int stride = gridDim.x * blockDim.x;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += stride) {
-    const int g = find_owner(row_off, members, r);
-    const GraphDesc& d = descs[g];
-    const int i = r - row_off[g];
-    if (d.tree) continue;  // its walk wrote F^r
-    ulonglong2* a = reinterpret_cast<ulonglong2*>(d.acc) + i;
-    const ulonglong2 v = *a;
-    d.fsum[i] = make_float2(__ll2float_rn((long long)v.x) * d.funscale, __ll2float_rn((long long)v.y) * d.funscale);
-    *a = make_ulonglong2(0ull, 0ull);
-  }
+// One thread per exact member: Z and 1 / Z from its units' sums, which are
+// cleared for the next iteration, and its schedule.
+__global__ void k_batch_finalize(const GraphDesc* __restrict__ descs, int members, BatchCtr* ctr, float ee,
+                                 int ee_iters, float mom0, float mom1) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g == 0) ctr->work_next[0] = ctr->work_next[1] = 0u;
+  if (g >= members || descs[g].tree) return;  // a tree member's walk set Z and the schedule
+  Sched* s = descs[g].sched;
+  const double Z = z_of(s->zacc[0][0], s->zacc[0][1], s->zbad[0], descs[g].n);
+  s->Z = Z;
+  s->inv_z = inv_of(Z);
+  s->zacc[0][0] = s->zacc[0][1] = 0ull;
+  s->zbad[0] = 0u;
+  set_schedule(s, 1, ee, ee_iters, mom0, mom1);
 }
 
 // A tree member's current layout Y[t & 1] into the buffer its tree build reads.
@@ -210,8 +218,13 @@ __global__ void __launch_bounds__(256) k_batch_attract(const GraphDesc* __restri
   const GraphDesc& d = descs[g];
   const int64_t i = valid ? r - row_off[g] : 0;
   float ax = 0.f, ay = 0.f;
-  float2 yi = make_float2(0.f, 0.f);
+  float2 yi = make_float2(0.f, 0.f), fr = yi, u = yi, gn = yi;
   int t = 0;
+  if (valid && lane == 0) {  // the row's state, on its way while the neighbours are gathered
+    fr = RowForce{d.fsum, d.tree ? nullptr : d.acc, d.funscale}.take(i);
+    u = d.upd[i];
+    gn = d.gains[i];
+  }
   if (valid) {
     t = d.sched->t;  // already advanced by k_batch_finalize
     const float2* Ycur = d.Y[(t - 1) & 1];
@@ -237,11 +250,9 @@ __global__ void __launch_bounds__(256) k_batch_attract(const GraphDesc* __restri
   ay = group_sum<G>(ay);
   if (!valid || lane != 0) return;
   const Sched* s = d.sched;
-  const float2 fr = d.fsum[i];
   const float invZ = s->inv_z;
   const float gx = 4.0f * (s->alpha * ax - fr.x * invZ);
   const float gy = 4.0f * (s->alpha * ay - fr.y * invZ);
-  float2 u = d.upd[i], gn = d.gains[i];
   const float2 y = optimizer_step(gx, gy, u, gn, s->mu, d.eta, min_gain, yi);
   d.upd[i] = u;
   d.gains[i] = gn;
@@ -252,7 +263,9 @@ __global__ void __launch_bounds__(256) k_batch_attract(const GraphDesc* __restri
 // The compiled shapes of the batched pass: (warps per CTA, i-points per lane).
 constexpr int kShapes[6][2] = {{1, 16}, {2, 16}, {4, 16}, {1, 8}, {2, 8}, {4, 8}};
 
-size_t smem_for(int W, int RI) { return (size_t)(W * 32 * RI) * (sizeof(float4) + sizeof(float2)); }
+size_t smem_for(int W, int RI) {
+  return (size_t)(W * 32 * RI) * (sizeof(float4) + sizeof(float2) + (RI == 8 ? sizeof(longlong2) : 0));
+}
 
 template <int W, int RI>
 tsgne_status prepare_shape() {
@@ -284,10 +297,9 @@ struct Member {
   DevBuf<float> P;
   DevBuf<float2> Y[2], upd, gains, fsum;
   DevBuf<unsigned long long> acc;  // fixed-point force accumulators (2 per point), zero between iterations
-  DevBuf<double> zunit;
   DevBuf<Sched> sched;
   HeavyStore hv;                     // hub rows and their chunks
-  int nt = 0, n_pad = 0, units = 0;  // for the batch's current tile
+  int nt = 0, n_pad = 0, units = 0, split = 1;  // for the batch's current tile
   DevBuf<float2> Y0;                 // initial layout (autotune restores it)
   bool active = true;
   bool tree = false;                 // tree-code repulsion
@@ -318,9 +330,10 @@ struct tsgne_batch {
   int next_id = 0;
   std::vector<std::unique_ptr<Member>> members;
   DevBuf<GraphDesc> d_desc;
-  DevBuf<int> d_unit_off, d_row_off, d_chunk_off;
+  DevBuf<int> d_unit_off, d_mid_off, d_small_off, d_row_off, d_chunk_off;
   DevBuf<BatchCtr> d_ctr;
-  int U = 0, R = 0, G = 0, C = 0;  // of the active members (C: hub-row chunks)
+  // of the active members: units of the large, mid and small ones, rows, members, hub-row chunks
+  int U = 0, Um = 0, Us = 0, R = 0, G = 0, C = 0;
   bool dirty = true;
   cudaGraphExec_t graph = nullptr;
   std::vector<Member*> trees;     // active tree members (refresh)
@@ -362,17 +375,30 @@ tsgne_status bfail(tsgne_batch* b, tsgne_status st, const std::string& msg = std
 // tile size divides kMaxT, so a member's n_pad never exceeds its buffers'.
 static_assert(kMaxT % (32 * 8) == 0 && 32 * 16 * 4 <= kMaxT, "tiles of 1, 2 and 4 warps must divide kMaxT");
 
-void shape_member(Member& m, int W, int RI) {
+// Which of the iteration's three repulsion launches takes a member: the
+// sizes decide as for a layout on its own (kSmallPoints, kMidPoints); only
+// large members run on the batch's shape.
+enum MemberClass { kSmall, kMid, kLarge };
+MemberClass class_of(const Member& m) {
+  return m.n <= kSmallPoints ? kSmall : (m.n <= kMidPoints ? kMid : kLarge);
+}
+
+void shape_member(Member& m, int sms, int W, int RI) {
+  const MemberClass c = class_of(m);
+  if (c == kSmall) {
+    m.units = m.tree ? 0 : small_units(m.n);
+    return;
+  }
+  if (c == kMid) {
+    W = 1;
+    RI = 8;
+  }
   const int T = 32 * RI * W;
   m.nt = (m.n + T - 1) / T;
   m.n_pad = m.nt * T;
-  m.units = m.tree ? 0 : m.nt * (m.nt + 1) / 2;
-}
-
-tsgne_status alloc_scratch(Member& m, int W, int RI) {
-  shape_member(m, W, RI);
-  TS_TRY(m.zunit.alloc((size_t)m.units));
-  return TSGNE_OK;
+  const int pairs = tile_pairs(m.nt);
+  m.split = split_tiles(pairs, sms * (warps_per_sm(RI) / W), RI);
+  m.units = m.tree ? 0 : pairs;
 }
 
 void invalidate(tsgne_batch* b) {
@@ -396,7 +422,7 @@ tsgne_status refresh_impl(tsgne_batch* b) {
   const int G = (int)act.size();
   b->G = G;
   std::vector<GraphDesc> h(G > 0 ? G : 1);
-  std::vector<int> uo(G + 1, 0), ro(G + 1, 0), co(G + 1, 0);
+  std::vector<int> uo(G + 1, 0), um(G + 1, 0), us(G + 1, 0), ro(G + 1, 0), co(G + 1, 0);
   int64_t tu = 0, tr = 0, tc = 0;  // the totals are 32-bit in the kernels
   for (const Member* m : act) {
     tu += m->units;
@@ -419,7 +445,6 @@ tsgne_status refresh_impl(tsgne_batch* b) {
     d.gains = m.gains.get();
     d.acc = m.acc.get();
     d.fsum = m.fsum.get();
-    d.zunit = m.zunit.get();
     d.sched = m.sched.get();
     d.hv = m.hv.view();
     d.n = m.n;
@@ -430,20 +455,30 @@ tsgne_status refresh_impl(tsgne_batch* b) {
     d.fscale = fix_scale(m.n);
     d.funscale = fix_unscale(m.n);
     d.tree = m.tree ? 1 : 0;
+    d.split = m.split;
     h[k] = d;
-    uo[k + 1] = uo[k] + m.units;
+    const MemberClass c = class_of(m);
+    uo[k + 1] = uo[k] + (c == kLarge ? m.units : 0);
+    um[k + 1] = um[k] + (c == kMid ? m.units : 0);
+    us[k + 1] = us[k] + (c == kSmall ? m.units : 0);
     ro[k + 1] = ro[k] + m.n;
     co[k + 1] = co[k] + m.hv.chunks;
   }
   b->U = uo[G];
+  b->Um = um[G];
+  b->Us = us[G];
   b->R = ro[G];
   b->C = co[G];
   TS_TRY(b->d_desc.alloc(h.size()));
   TS_TRY(b->d_unit_off.alloc(uo.size()));
+  TS_TRY(b->d_mid_off.alloc(um.size()));
+  TS_TRY(b->d_small_off.alloc(us.size()));
   TS_TRY(b->d_row_off.alloc(ro.size()));
   TS_TRY(b->d_chunk_off.alloc(co.size()));
   TS_CUDA(cudaMemcpyAsync(b->d_desc.get(), h.data(), sizeof(GraphDesc) * h.size(), cudaMemcpyHostToDevice, b->stream));
   TS_CUDA(cudaMemcpyAsync(b->d_unit_off.get(), uo.data(), sizeof(int) * uo.size(), cudaMemcpyHostToDevice, b->stream));
+  TS_CUDA(cudaMemcpyAsync(b->d_mid_off.get(), um.data(), sizeof(int) * um.size(), cudaMemcpyHostToDevice, b->stream));
+  TS_CUDA(cudaMemcpyAsync(b->d_small_off.get(), us.data(), sizeof(int) * us.size(), cudaMemcpyHostToDevice, b->stream));
   TS_CUDA(cudaMemcpyAsync(b->d_row_off.get(), ro.data(), sizeof(int) * ro.size(), cudaMemcpyHostToDevice, b->stream));
   TS_CUDA(cudaMemcpyAsync(b->d_chunk_off.get(), co.data(), sizeof(int) * co.size(), cudaMemcpyHostToDevice, b->stream));
   TS_CUDA(cudaStreamSynchronize(b->stream));
@@ -498,10 +533,17 @@ tsgne_status enqueue_iteration(tsgne_batch* b) {
   const int slots = b->sms * (warps_per_sm(RI) / W);
   const int grid = b->U < slots ? b->U : slots;
   const size_t sm = smem_for(W, RI);
+  if (b->Us > 0)
+    k_batch_small<<<b->Us, 32 * kSmallWarps, 0, b->stream>>>(b->d_desc.get(), b->d_small_off.get(), G);
+  if (b->Um > 0) {
+    const int mgrid = std::min(b->Um, b->sms * warps_per_sm(8));
+    k_batch_repulsion<1, 8><<<mgrid, 32, smem_for(1, 8), b->stream>>>(b->d_desc.get(), b->d_mid_off.get(), G, b->Um,
+                                                                     b->d_ctr.get()->work_next);
+  }
   if (b->U > 0) {
     const GraphDesc* dd = b->d_desc.get();
     const int* uo = b->d_unit_off.get();
-    BatchCtr* ctr = b->d_ctr.get();
+    uint32_t* ctr = b->d_ctr.get()->work_next + 1;
     if (RI == 16) {
       if (W == 4) k_batch_repulsion<4, 16><<<grid, 128, sm, b->stream>>>(dd, uo, G, b->U, ctr);
       else if (W == 2) k_batch_repulsion<2, 16><<<grid, 64, sm, b->stream>>>(dd, uo, G, b->U, ctr);
@@ -512,10 +554,8 @@ tsgne_status enqueue_iteration(tsgne_batch* b) {
       else k_batch_repulsion<1, 8><<<grid, 32, sm, b->stream>>>(dd, uo, G, b->U, ctr);
     }
   }
-  // 32 W threads: the same reduction tree as the single-layout pass's last CTA
-  k_batch_finalize<<<G, 32 * W, 0, b->stream>>>(b->d_desc.get(), c.early_exag, c.ee_iters, c.momentum0, c.momentum1);
-  const int rgrid = std::max(1, std::min((b->R + 255) / 256, b->sms * 16));
-  k_batch_reduce<<<rgrid, 256, 0, b->stream>>>(b->d_desc.get(), b->d_row_off.get(), G, b->R);
+  k_batch_finalize<<<(G + 127) / 128, 128, 0, b->stream>>>(b->d_desc.get(), G, b->d_ctr.get(), c.early_exag,
+                                                           c.ee_iters, c.momentum0, c.momentum1);
   for (int k = 0; k < ntree; ++k) TS_CUDA(cudaStreamWaitEvent(b->stream, b->ev[1 + k], 0));  // join
   if (b->C > 0) {
     const int hgrid = std::min((b->C + 7) / 8, 4096);  // one warp per chunk
@@ -664,7 +704,7 @@ tsgne_status prepare_member(const tsgne_config& cfg, int sms, int32_t n, const i
 // Adds a prepared member to the batch (its per-tile scratch for the current
 // tile); the membership changes at the next run.
 tsgne_status attach_member(tsgne_batch* b, std::unique_ptr<Member> mem, int32_t* id_out) {
-  TS_TRY(alloc_scratch(*mem, b->W, b->RI));
+  shape_member(*mem, b->sms, b->W, b->RI);
   mem->id = b->next_id++;
   if (id_out) *id_out = mem->id;
   b->members.push_back(std::move(mem));
@@ -798,7 +838,7 @@ tsgne_status tsgne_batch_size(tsgne_batch* b, int32_t* members, int32_t* tile_wa
   B_TRY(b, refresh(b));
   if (members) *members = (int32_t)b->members.size();
   if (tile_warps) *tile_warps = b->W;
-  if (units) *units = b->U;
+  if (units) *units = (int64_t)b->U + b->Um + b->Us;
   return TSGNE_OK;
 }
 
@@ -850,7 +890,7 @@ tsgne_status tsgne_batch_set_shape(tsgne_batch* b, int32_t tile_warps, int32_t i
     return bfail(b, TSGNE_ERR_INVALID_ARG, "tile_warps must be 1, 2 or 4 and i_per_lane 8 or 16");
   if (tile_warps == b->W && i_per_lane == b->RI) return TSGNE_OK;
   B_CUDA(b, cudaStreamSynchronize(b->stream));
-  for (auto& m : b->members) B_TRY(b, alloc_scratch(*m, tile_warps, i_per_lane));
+  for (auto& m : b->members) shape_member(*m, b->sms, tile_warps, i_per_lane);
   b->W = tile_warps;
   b->RI = i_per_lane;
   invalidate(b);

@@ -16,9 +16,6 @@
 //   min_gain; upd = mu upd - eta gain g; y_next = y + upd.  Reading Y_cur and
 //   writing Y_next (double buffer) keeps every row's neighbours at the old
 //   layout.  In export mode it writes g and changes nothing.
-// k_fix_forces (end of S4): converts each point's fixed-point repulsion
-//   accumulators into F^r (the update then reads one float2 per row) and
-//   clears them for the next pass.
 // k_kl (S6): sum_e p_e ln(p_e / w_e) and sum_e p_e in FP64 (terms in FP32),
 //   fixed-order totals; KL = first + second * ln Z on the host (Eq. 5 with
 //   q = w / Z).
@@ -77,18 +74,22 @@ __global__ void __launch_bounds__(kAttrCta, 6)
     k_attract(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const PT* __restrict__ P,
               const YT* __restrict__ Ycur, const float2* __restrict__ Ym, float2* __restrict__ Ynext,
               bf162* __restrict__ Ynext16, float2* __restrict__ upd, float2* __restrict__ gains,
-              const float2* __restrict__ frep_part, int chunks, int n_pad, Sched* sched, float eta, float min_gain,
-              float alpha_export, float2* __restrict__ g_out, HeavyRows hv) {
+              RowForce rf, int zslot, Sched* sched, float eta, float min_gain, float alpha_export,
+              float2* __restrict__ g_out, HeavyRows hv) {
   __shared__ float2 spart[kAttrCta][G];
   __shared__ int64_t srp[kAttrCta + 1];
   __shared__ int soff[kAttrCta + 1];
   __shared__ int swarp[kAttrCta / 32];
   __shared__ uint8_t srow[kAttrCta * G];  // (row, slot) pair -> row
   __shared__ int slevels;
+  __shared__ float s_invz;
   const int64_t row0 = (int64_t)blockIdx.x * kAttrCta;
   const int tid = threadIdx.x;
   for (int t = tid; t <= kAttrCta; t += kAttrCta) srp[t] = row0 + t <= n ? rp[row0 + t] : 0;
-  if (tid == 0) slevels = 0;
+  if (tid == 0) {
+    slevels = 0;
+    s_invz = pass_inv_z(sched, zslot, n);
+  }
   __syncthreads();
   // (1) the slots of this thread's row: slot s < G sums entries s, s + G, ...
   // of the row (short rows only); a hub row's chunk sums go to slot 0
@@ -189,8 +190,7 @@ __global__ void __launch_bounds__(kAttrCta, 6)
   a0 = make_float2(a0.x + a2.x, a0.y + a2.y);  // o = 2
   a1 = make_float2(a1.x + a3.x, a1.y + a3.y);
   const float2 fa = make_float2(a0.x + a1.x, a0.y + a1.y);  // o = 1
-  finish_row<EXPORT>(i, fa, frep_part, chunks, n_pad, sched, alpha_export, g_out, Ym, Ynext, Ynext16, upd, gains,
-                     eta, min_gain);
+  finish_row<EXPORT>(i, fa, rf, s_invz, sched, alpha_export, g_out, Ym, Ynext, Ynext16, upd, gains, eta, min_gain);
 }
 
 // Attraction of the long rows (more than kHeavyDeg entries), in chunks of at
@@ -210,19 +210,6 @@ __global__ void __launch_bounds__(256)
     ax = group_sum<32>(ax);
     ay = group_sum<32>(ay);
     if (lane == 0) hv.fa[c] = make_float2(ax, ay);
-  }
-}
-
-// F^r_i from the fixed-point accumulators (one rounding of the exact integer
-// sum), which are cleared for the next pass; one thread per point.
-__global__ void __launch_bounds__(kAttrCta)
-    k_fix_forces(int n, unsigned long long* __restrict__ acc, float unscale, float2* __restrict__ out) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    ulonglong2* a = reinterpret_cast<ulonglong2*>(acc) + i;
-    const ulonglong2 v = *a;
-    out[i] = make_float2(__ll2float_rn((long long)v.x) * unscale, __ll2float_rn((long long)v.y) * unscale);
-    *a = make_ulonglong2(0ull, 0ull);
   }
 }
 
@@ -338,13 +325,6 @@ tsgne_status launch_reduce_slots(int n, const float2* part, int slots, int n_pad
   return TSGNE_OK;
 }
 
-tsgne_status launch_fix_forces(int n, unsigned long long* acc, float2* out, cudaStream_t s) {
-  const int g = grid_rows(n, kAttrCta);
-  k_fix_forces<<<g, kAttrCta, 0, s>>>(n, acc, fix_unscale(n), out);
-  TS_CUDA(cudaGetLastError());
-  return TSGNE_OK;
-}
-
 tsgne_status launch_prefetch_l2(const void* p, int64_t bytes, cudaStream_t s) {
   if (bytes < (1 << 20)) return TSGNE_OK;  // small layouts stay in L2 anyway
   const int64_t lines = (bytes + 127) / 128;
@@ -376,8 +356,8 @@ template <bool EXPORT, class PT, class YT>
 tsgne_status attract_t(const AttractArgs& a, float alpha, float2* g, cudaStream_t s) {
   k_attract<kG, EXPORT, PT, YT><<<grid_rows(a.n, kAttrCta), kAttrCta, 0, s>>>(
       a.n, a.rp, a.col, static_cast<const PT*>(a.P), static_cast<const YT*>(a.Yr), a.Ym, a.Ynext,
-      static_cast<bf162*>(a.Ynext16), a.upd, a.gains, a.frep, a.chunks, a.n_pad, a.sched, a.eta, a.min_gain, alpha,
-      g, a.hv);
+      static_cast<bf162*>(a.Ynext16), a.upd, a.gains, RowForce{a.frep, a.facc, a.unscale}, a.zslot, a.sched, a.eta,
+      a.min_gain, alpha, g, a.hv);
   TS_CUDA(cudaGetLastError());
   return TSGNE_OK;
 }

@@ -49,9 +49,21 @@ __device__ __forceinline__ bool arrive_last(uint32_t* counter) {
 
 // Sum of parts[0..count) by one CTA in a fixed order (strided per thread, then
 // block_sum_d).  L1 is bypassed so partials written by other CTAs are seen.
+// One CTA does this alone at the end of a pass, waiting on L2 each time, so
+// sixteen loads are in flight per thread.
 __device__ __forceinline__ double sum_partials(const double* parts, int count) {
+  constexpr int U = 16;
+  const int T = (int)blockDim.x;
   double s = 0.0;
-  for (int k = threadIdx.x; k < count; k += blockDim.x) s += __ldcg(parts + k);
+  int k = threadIdx.x;
+  for (; k + (U - 1) * T < count; k += U * T) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = __ldcg(parts + k + u * T);
+#pragma unroll
+    for (int u = 0; u < U; ++u) s += v[u];
+  }
+  for (; k < count; k += T) s += __ldcg(parts + k);
   return block_sum_d(s);
 }
 

@@ -142,24 +142,57 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel_u32(uint32_t* p, uint32_t v
   return old;
 }
 
+// 1 / Z rounded to FP32: a float quotient and one Newton step on the double's
+// two halves (GB300 runs FP64 at 1/64 of the FP32 rate: a double division is
+// a microsecond of waiting).
+__device__ __forceinline__ float inv_of(double Z) {
+  const float zh = (float)Z, zl = (float)(Z - (double)zh);
+  const float r = 1.0f / zh;
+  const float e = fmaf(zh, r, -1.0f) + zl * r;
+  return isfinite(e) ? fmaf(-r, e, r) : r;
+}
+
+// Z of the symmetric exact pass from its fixed-point words (NaN if a kernel
+// value was NaN).
+__host__ __device__ __forceinline__ double z_of(unsigned long long low, unsigned long long high, uint32_t bad, int n) {
+  static_assert(kZShift == 32, "the high word counts whole units");
+  const double z = (double)high + (double)low * (1.0 / (double)(1ull << kZShift)) - (double)n;
+  return bad ? (double)NAN : z;
+}
+
+// 1 / Z of the pass whose forces the rows use (see AttractArgs).
+__device__ __forceinline__ float pass_inv_z(const Sched* sched, int zslot, int n) {
+  if (zslot < 0) return sched->inv_z;
+  return inv_of(z_of(sched->zacc[zslot][0], sched->zacc[zslot][1], sched->zbad[zslot], n));
+}
+
+// Where a row's repulsive force comes from (see AttractArgs): F^r per row, or
+// fixed-point accumulators, cleared for the next pass by the row that reads them.
+struct RowForce {
+  const float2* __restrict__ frep;
+  unsigned long long* __restrict__ facc;
+  float unscale;
+  __device__ __forceinline__ float2 take(int64_t i) const {
+    if (facc == nullptr) return frep[i];
+    ulonglong2* a = reinterpret_cast<ulonglong2*>(facc) + i;
+    const ulonglong2 v = *a;
+    *a = make_ulonglong2(0ull, 0ull);
+    return make_float2(__ll2float_rn((long long)v.x) * unscale, __ll2float_rn((long long)v.y) * unscale);
+  }
+};
+
 // Gradient of row i from its attraction sum fa, then (EXPORT) the gradient
 // export or the optimiser step into the next layout.
 template <bool EXPORT>
-__device__ __forceinline__ void finish_row(int64_t i, float2 fa, const float2* __restrict__ frep_part, int chunks,
-                                           int n_pad, Sched* sched, float alpha_export, float2* __restrict__ g_out,
+__device__ __forceinline__ void finish_row(int64_t i, float2 fa, RowForce rf, float invZ, Sched* sched,
+                                           float alpha_export, float2* __restrict__ g_out,
                                            const float2* __restrict__ Ym, float2* __restrict__ Ynext,
                                            bf162* __restrict__ Ynext16, float2* __restrict__ upd,
                                            float2* __restrict__ gains, float eta, float min_gain) {
-  float rx = 0.f, ry = 0.f;
-  for (int c = 0; c < chunks; ++c) {
-    const float2 f = frep_part[(size_t)c * n_pad + i];
-    rx += f.x;
-    ry += f.y;
-  }
-  const float invZ = sched->inv_z;
+  const float2 r = rf.take(i);
   const float alpha = EXPORT ? alpha_export : sched->alpha;
-  const float gx = 4.0f * (alpha * fa.x - rx * invZ);
-  const float gy = 4.0f * (alpha * fa.y - ry * invZ);
+  const float gx = 4.0f * (alpha * fa.x - r.x * invZ);
+  const float gy = 4.0f * (alpha * fa.y - r.y * invZ);
   if (EXPORT) {
     g_out[i] = make_float2(gx, gy);
     return;

@@ -12,10 +12,13 @@
 //
 // Z: each lane's FP32 partial of a point covers one 64-point ring group
 // (64 terms w in (0, 1]), is then added into a second FP32 partial over the
-// unit's groups (at most 16 for 1,024-point tiles) and leaves the unit in
-// FP64.  The worst-case relative rounding of a unit's row sum is then about
-// (63 + 15) 2^-24 = 4.6e-6, against 1,023 2^-24 = 6.1e-5 for one FP32 sum over
-// the whole tile.
+// unit's groups (at most 16 for 1,024-point tiles), and from there on the
+// sums are exact integers (kZShift).  The worst-case relative rounding of a
+// unit's row sum is then about (63 + 15) 2^-24 = 4.6e-6, against 1,023 2^-24 =
+// 6.1e-5 for one FP32 sum over the whole tile.  The integers also replace the
+// FP64 sums that ended every unit and the last CTA's sum over all of them: on
+// a 2,000-point layout these took 4.2 of 8 us (0.5 us the warp's double
+// butterfly, 1.5 us the fence and the arrival counter, 2.2 us the last CTA).
 #pragma once
 
 #include "f32x2.cuh"
@@ -27,12 +30,15 @@ namespace tsgne {
 constexpr int kRI = 16;             // i-points per lane (default shape)
 constexpr int kWarpsPerSm = 8;      // resident warps per SM the grid is sized for (16 i-points per lane)
 constexpr int kGroup = 64;          // j-points per ring group (32 lanes x 2)
-
 // Resident warps per SM the grid is sized for, by i-points per lane: 16
 // i-points need about 200 registers a thread (8 warps), 8 about half.
 __host__ __device__ constexpr int warps_per_sm(int RI) { return RI >= 16 ? 8 : 16; }
 
-__device__ __forceinline__ int row_start(int a, int nt) { return a * nt - (a * (a - 1)) / 2; }
+// Tile pairs of nt tiles, and the first one of diagonal a (products of two tile numbers pass 2^31 above 46,340 tiles).
+__host__ __device__ __forceinline__ int tile_pairs(int nt) { return (int)((long long)nt * (nt + 1) / 2); }
+__device__ __forceinline__ int row_start(int a, int nt) {
+  return (int)((long long)a * nt - (long long)a * (a - 1) / 2);
+}
 
 // One j-point against the lane's 8 i-points; acc (x, y) is the running sum
 // of w^2 (y_i - y_j) over i for this j.
@@ -67,49 +73,81 @@ __device__ __forceinline__ void ring_pair(const float4 q, float& accx, float& ac
 }
 
 // Adds v (one coordinate of a partial force) to a fixed-point accumulator.
-__device__ __forceinline__ void red_fix(unsigned long long* p, float v, float scale) {
-  const long long q = __float2ll_rn(v * scale);  // v * 2^s is exact: scale is a power of two
+__device__ __forceinline__ void red_int(unsigned long long* p, long long q) {
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)q) : "memory");
 }
+__device__ __forceinline__ void red_fix(unsigned long long* p, float v, float scale) {
+  red_int(p, __float2ll_rn(v * scale));  // v * 2^s is exact: scale is a power of two
+}
 
-// One tile pair (a, b), a <= b, of one layout: stages tile b, evaluates the
-// pairs and adds tile a's forces and (a < b) tile b's forces into the
-// fixed-point accumulators acc[2 p], acc[2 p + 1] of their real points
-// (p < n).  Returns this thread's share of the unit's Z (ordered pairs; the
-// diagonal unit includes the w_ii = 1 terms of its real points).  Every
-// thread of the CTA must call it; it ends with the shared tiles free for reuse
-// only after a __syncthreads by the caller.
-template <int W, int RI = kRI, class YT = float2>
-__device__ __forceinline__ double sym_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
-                                           float fscale, int a, int b, float4* sj, float2* sacc) {
-  constexpr int kH = RI / 2;  // FP32x2 pairs of i-points per lane
-  constexpr int T = W * 32 * RI;
-  constexpr int G = T / kGroup;  // = W RI / 2 groups (a power of two)
-  static_assert((G & (G - 1)) == 0, "ring groups are picked modulo G");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const u64 one2 = pk(1.f, 1.f);
+// The fixed-point value of a Z partial z >= 0 (NaN: the caller's check).
+__device__ __forceinline__ u64 z_fix(float z) { return __float2ull_rn(z * (float)(1ull << kZShift)); }
 
-  // j tile b into shared memory
-  for (int k = tid; k < T; k += W * 32) {
-    const float2 p = ld_y(Y, (size_t)b * T + k);
-    sj[k] = make_float4(-p.x, -p.x, -p.y, -p.y);
-    sacc[k] = make_float2(0.f, 0.f);
+// Sum over the warp's lanes of integers below 2^58, in every lane.
+__device__ __forceinline__ u64 warp_sum_u58(u64 v) {
+  const u64 m = (1ull << 27) - 1;
+  const u64 a = __reduce_add_sync(0xffffffffu, (uint32_t)(v & m));
+  const u64 b = __reduce_add_sync(0xffffffffu, (uint32_t)((v >> 27) & m));
+  const u64 c = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 54));
+  return a + (b << 27) + (c << 54);
+}
+
+// One thread: the Z of a unit to its place: as a double (exact: below 2^53
+// for every shape of a single layout) in zunit, for a share of a sharded pass,
+// or added to the two words of zacc.
+__device__ __forceinline__ void put_z(u64 q, bool bad, double* zunit, u64* zacc, uint32_t* zbad) {
+  if (zunit != nullptr) {
+    *zunit = bad ? (double)NAN : (double)q * (1.0 / (double)(1ull << kZShift));
+    return;
   }
-  // i points of tile a: lane holds i = a*T + warp*32*RI + r*32 + lane, r < RI
-  const int ibase = a * T + warp * (32 * RI) + lane;
-  u64 X2[kH], Y2[kH], FX[kH], FY[kH], Z2[kH], ZG[kH];
-#pragma unroll
-  for (int h = 0; h < kH; ++h) {
-    const float2 p0 = ld_y(Y, ibase + (2 * h) * 32);
-    const float2 p1 = ld_y(Y, ibase + (2 * h + 1) * 32);
-    X2[h] = pk(p0.x, p1.x);
-    Y2[h] = pk(p0.y, p1.y);
-    FX[h] = FY[h] = Z2[h] = ZG[h] = 0ull;
-  }
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(zacc), "l"(q & 0xffffffffull) : "memory");
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(zacc + 1), "l"(q >> 32) : "memory");
+  if (bad) atomicOr(zbad, 1u);
+}
+
+// Sum over a CTA of W warps of the threads' Z (valid in thread 0); *bad: any
+// thread's.  zs: W words of shared memory, free again after a __syncthreads.
+template <int W>
+__device__ __forceinline__ u64 cta_z(u64 q, bool* bad, u64* zs) {
+  const bool any = __any_sync(0xffffffffu, *bad);
+  u64 v = warp_sum_u58(q);
+  *bad = any;
+  if (W == 1) return v;
+  if ((threadIdx.x & 31) == 0) zs[threadIdx.x >> 5] = any ? ~0ull : v;
   __syncthreads();
+  if (threadIdx.x == 0) {
+    v = 0ull;
+    *bad = false;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      *bad |= zs[w] == ~0ull;
+      v += zs[w];
+    }
+  }
+  return v;
+}
 
-  double zt = 0.0;
-  if (a != b) {
+// The schedule of the iteration that follows a pass (one thread).
+__device__ __forceinline__ void set_schedule(Sched* s, int advance, float ee, int ee_iters, float mom0, float mom1) {
+  const int t = s->t;
+  s->alpha = t < ee_iters ? ee : 1.0f;
+  s->mu = t < ee_iters ? mom0 : mom1;
+  if (advance) s->t = t + 1;
+}
+
+// The pairs of a unit: the lane's i-points against the G ring groups in sj,
+// a != b with the j side in sacc, a == b as ordered pairs.  ZG: the lane's Z
+// partials.  Ends, for a != b, with a __syncthreads.
+template <int W, int kH>
+__device__ __forceinline__ void unit_pairs(int G, bool off_diagonal, const float4* sj, float2* sacc,
+                                           const u64 (&X2)[kH], const u64 (&Y2)[kH], u64 (&FX)[kH], u64 (&FY)[kH],
+                                           u64 (&ZG)[kH]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u64 one2 = pk(1.f, 1.f);
+  u64 Z2[kH];
+#pragma unroll
+  for (int h = 0; h < kH; ++h) Z2[h] = 0ull;
+  if (off_diagonal) {
     for (int ph = 0; ph < G; ++ph) {
       const int g = (warp + ph) & (G - 1);
       const float4* gj = sj + g * kGroup;
@@ -138,61 +176,103 @@ __device__ __forceinline__ double sym_unit(const YT* __restrict__ Y, int n, unsi
       }
       __syncthreads();
     }
-#pragma unroll
-    for (int h = 0; h < kH; ++h) {
-      float z0, z1;
-      upk(ZG[h], z0, z1);
-      zt += 2.0 * ((double)z0 + (double)z1);  // tile a holds no padding
-    }
-    // j side: F_j = -sum_i w^2 (y_i - y_j) for tile b's real points
-    const int jb = b * T;
-    for (int k = tid; k < T; k += W * 32)
-      if (jb + k < n) {
-        const float2 v = sacc[k];
-        red_fix(acc + 2 * (size_t)(jb + k), -v.x, fscale);
-        red_fix(acc + 2 * (size_t)(jb + k) + 1, -v.y, fscale);
-      }
-  } else {
-    // diagonal unit: ordered pairs within the tile, i side only, in groups
-    // of 64 j-points for Z
-    for (int j0 = 0; j0 < T; j0 += kGroup) {
+    return;
+  }
+  // diagonal unit: ordered pairs within the tile, i side only, in groups
+  // of 64 j-points for Z
+  for (int j0 = 0; j0 < G * kGroup; j0 += kGroup) {
 #pragma unroll 2
-      for (int j = j0; j < j0 + kGroup; ++j) {
-        const float4 q = sj[j];
-        const u64 nx = pk(q.x, q.y);
-        const u64 ny = pk(q.z, q.w);
-#pragma unroll
-        for (int h = 0; h < kH; ++h) {
-          const u64 dx = add2(X2[h], nx);
-          const u64 dy = add2(Y2[h], ny);
-          u64 qq = fma2(dx, dx, one2);
-          qq = fma2(dy, dy, qq);
-          float q0, q1;
-          upk(qq, q0, q1);
-          const u64 w = pk(rcp_approx(q0), rcp_approx(q1));
-          Z2[h] = add2(Z2[h], w);
-          const u64 w2 = mul2(w, w);
-          FX[h] = fma2(w2, dx, FX[h]);
-          FY[h] = fma2(w2, dy, FY[h]);
-        }
-      }
+    for (int j = j0; j < j0 + kGroup; ++j) {
+      const float4 q = sj[j];
+      const u64 nx = pk(q.x, q.y);
+      const u64 ny = pk(q.z, q.w);
 #pragma unroll
       for (int h = 0; h < kH; ++h) {
-        ZG[h] = add2(ZG[h], Z2[h]);
-        Z2[h] = 0ull;
+        const u64 dx = add2(X2[h], nx);
+        const u64 dy = add2(Y2[h], ny);
+        u64 qq = fma2(dx, dx, one2);
+        qq = fma2(dy, dy, qq);
+        float q0, q1;
+        upk(qq, q0, q1);
+        const u64 w = pk(rcp_approx(q0), rcp_approx(q1));
+        Z2[h] = add2(Z2[h], w);
+        const u64 w2 = mul2(w, w);
+        FX[h] = fma2(w2, dx, FX[h]);
+        FY[h] = fma2(w2, dy, FY[h]);
       }
     }
 #pragma unroll
     for (int h = 0; h < kH; ++h) {
-      float z0, z1;
-      upk(ZG[h], z0, z1);
-      if (ibase + (2 * h) * 32 < n) zt += (double)z0;
-      if (ibase + (2 * h + 1) * 32 < n) zt += (double)z1;
+      ZG[h] = add2(ZG[h], Z2[h]);
+      Z2[h] = 0ull;
     }
   }
-  // i side of tile a's real points
+}
+
+// TJ j-points from jb into shared memory, their accumulators cleared.
+template <int W, class YT>
+__device__ __forceinline__ void stage_j(const YT* __restrict__ Y, int jb, int TJ, float4* sj, float2* sacc) {
+  for (int k = threadIdx.x; k < TJ; k += W * 32) {
+    const float2 p = ld_y(Y, (size_t)jb + k);
+    sj[k] = make_float4(-p.x, -p.x, -p.y, -p.y);
+    sacc[k] = make_float2(0.f, 0.f);
+  }
+}
+
+// Off-diagonal unit, j side: F_j = -sum_i w^2 (y_i - y_j) for the real j-points.
+template <int W>
+__device__ __forceinline__ void add_j(int jb, int TJ, int n, const float2* sacc, unsigned long long* acc,
+                                      float fscale) {
+  for (int k = threadIdx.x; k < TJ; k += W * 32)
+    if (jb + k < n) {
+      const float2 v = sacc[k];
+      red_fix(acc + 2 * (size_t)(jb + k), -v.x, fscale);
+      red_fix(acc + 2 * (size_t)(jb + k) + 1, -v.y, fscale);
+    }
+}
+
+// The thread's Z in fixed point from its lane partials (ordered pairs:
+// twice the off-diagonal units', whose tile a holds no padding; the diagonal
+// units' real points, w_ii = 1 included); *bad: a NaN among them.
+template <int kH>
+__device__ __forceinline__ u64 unit_z(bool off_diagonal, int ibase, int n, const u64 (&ZG)[kH], bool* bad) {
+  u64 zt = 0ull;
+  float zn = 0.f;  // NaN if any partial is
 #pragma unroll
   for (int h = 0; h < kH; ++h) {
+    float z0, z1;
+    upk(ZG[h], z0, z1);
+    if (off_diagonal || ibase + (2 * h) * 32 < n) {
+      zt += z_fix(z0);
+      zn += z0;
+    }
+    if (off_diagonal || ibase + (2 * h + 1) * 32 < n) {
+      zt += z_fix(z1);
+      zn += z1;
+    }
+  }
+  *bad = zn != zn;
+  return off_diagonal ? 2ull * zt : zt;
+}
+
+// Loads of the lane's i-points of tile a: i = a T + warp 32 RI + r 32 + lane, r < RI.
+template <int RI, class YT>
+__device__ __forceinline__ void load_i(const YT* __restrict__ Y, int ibase, u64 (&X2)[RI / 2], u64 (&Y2)[RI / 2]) {
+#pragma unroll
+  for (int h = 0; h < RI / 2; ++h) {
+    const float2 p0 = ld_y(Y, ibase + (2 * h) * 32);
+    const float2 p1 = ld_y(Y, ibase + (2 * h + 1) * 32);
+    X2[h] = pk(p0.x, p1.x);
+    Y2[h] = pk(p0.y, p1.y);
+  }
+}
+
+// i side of tile a's real points.
+template <int RI>
+__device__ __forceinline__ void add_i(int ibase, int n, const u64 (&FX)[RI / 2], const u64 (&FY)[RI / 2],
+                                      unsigned long long* acc, float fscale) {
+#pragma unroll
+  for (int h = 0; h < RI / 2; ++h) {
     float fx0, fx1, fy0, fy1;
     upk(FX[h], fx0, fx1);
     upk(FY[h], fy0, fy1);
@@ -206,23 +286,223 @@ __device__ __forceinline__ double sym_unit(const YT* __restrict__ Y, int n, unsi
       red_fix(acc + 2 * (size_t)p1 + 1, fy1, fscale);
     }
   }
+}
+
+// sym_unit of a diagonal pair (a, a).  Out of line, as unit_tiles is: how the
+// compiler schedules the ring loop, where a large pass spends its time,
+// depends on what else is inlined beside it (300,000 points: 15.86 ms with
+// both calls, 16.07 with this one alone, 16.2 with neither; 100,000: 1.80,
+// 1.83, 1.92 ms).  A NaN comes back as ~0.
+template <int W, int RI, class YT>
+static __device__ __noinline__ u64 diag_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+                                             float fscale, int a, int sub, int G, float4* sj, float2* sacc) {
+  constexpr int kH = RI / 2;
+  const int TJ = G * kGroup;
+  const int ibase = a * (W * 32 * RI) + (int)(threadIdx.x >> 5) * (32 * RI) + (int)(threadIdx.x & 31);
+  u64 X2[kH], Y2[kH], FX[kH], FY[kH], ZG[kH];
+  stage_j<W>(Y, a * (W * 32 * RI) + sub * TJ, TJ, sj, sacc);
+  load_i<RI>(Y, ibase, X2, Y2);
+#pragma unroll
+  for (int h = 0; h < kH; ++h) FX[h] = FY[h] = ZG[h] = 0ull;
+  __syncthreads();
+  unit_pairs<W, kH>(G, false, sj, sacc, X2, Y2, FX, FY, ZG);
+  bool bad;
+  const u64 zt = unit_z<kH>(false, ibase, n, ZG, &bad);
+  add_i<RI>(ibase, n, FX, FY, acc, fscale);
+  return bad ? ~0ull : zt;
+}
+
+// One unit of a layout: the points of tile a against the G ring groups of
+// tile b that start at group sub * G (a <= b; G = groups, or T / 64, the whole
+// tile, and sub = 0 for kWhole; see split_tiles).  Stages those j-points,
+// evaluates the pairs and adds tile a's forces and (a < b) the j-points'
+// forces into the fixed-point accumulators acc[2 p], acc[2 p + 1] of the real
+// points (p < n).  Returns this thread's share of the unit's Z in fixed point
+// (unit_z).  Every thread of the CTA must call it; it ends with the shared
+// tiles free for reuse only after a __syncthreads by the caller.  G is a power
+// of two, at least W.
+template <int W, int RI, class YT, bool kWhole>
+__device__ __forceinline__ u64 sym_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+                                        float fscale, int a, int b, int sub, int groups, float4* sj, float2* sacc,
+                                        bool* bad) {
+  constexpr int kH = RI / 2;  // FP32x2 pairs of i-points per lane
+  constexpr int T = W * 32 * RI;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int G = kWhole ? T / kGroup : groups;  // a constant for whole tiles
+  const int TJ = G * kGroup;
+  if (a == b) {
+    const u64 z = diag_unit<W, RI, YT>(Y, n, acc, fscale, a, sub, G, sj, sacc);
+    *bad = z == ~0ull;
+    return *bad ? 0ull : z;
+  }
+  const int jb = b * T + sub * TJ;  // first j-point
+  stage_j<W>(Y, jb, TJ, sj, sacc);
+  const int ibase = a * T + warp * (32 * RI) + lane;
+  u64 X2[kH], Y2[kH], FX[kH], FY[kH], ZG[kH];
+  load_i<RI>(Y, ibase, X2, Y2);
+#pragma unroll
+  for (int h = 0; h < kH; ++h) FX[h] = FY[h] = ZG[h] = 0ull;
+  __syncthreads();
+  unit_pairs<W, kH>(G, true, sj, sacc, X2, Y2, FX, FY, ZG);
+  const u64 zt = unit_z<kH>(true, ibase, n, ZG, bad);
+  add_j<W>(jb, TJ, n, sacc, acc, fscale);
+  add_i<RI>(ibase, n, FX, FY, acc, fscale);
   return zt;
 }
 
-// (a, b) of unit u of a layout with nt tiles, numbered diagonal by diagonal:
+// All S = T / (64 G) units of one tile pair by one CTA: the same FP32 partials,
+// so the same bits, as S calls of sym_unit.  For a batch, whose members fill
+// the GPU together: both tiles are loaded once, the i-points' integer sums
+// stay in shared memory (si: T long2, each thread its own points) and reach
+// the accumulators once instead of S times.  Returns the thread's Z.
+template <int W, int RI, class YT>
+static __device__ __noinline__ u64 sym_units(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+                                             float fscale, int a, int b, int G, float4* sj, float2* sacc,
+                                             longlong2* si) {
+  constexpr int kH = RI / 2;
+  constexpr int T = W * 32 * RI;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ibase = a * T + warp * (32 * RI) + lane;
+  longlong2* const mine = si + warp * (32 * RI) + lane;
+  u64 X2[kH], Y2[kH];
+  stage_j<W>(Y, b * T, T, sj, sacc);
+  load_i<RI>(Y, ibase, X2, Y2);
+  __syncthreads();
+  u64 zt = 0ull;
+  bool bad = false;
+  for (int j0 = 0; j0 < T; j0 += G * kGroup) {
+    u64 FX[kH], FY[kH], ZG[kH];
+#pragma unroll
+    for (int h = 0; h < kH; ++h) FX[h] = FY[h] = ZG[h] = 0ull;
+    unit_pairs<W, kH>(G, a != b, sj + j0, sacc + j0, X2, Y2, FX, FY, ZG);
+    bool nan;
+    zt += unit_z<kH>(a != b, ibase, n, ZG, &nan);
+    bad |= nan;
+#pragma unroll
+    for (int h = 0; h < kH; ++h) {
+      float fx[2], fy[2];
+      upk(FX[h], fx[0], fx[1]);
+      upk(FY[h], fy[0], fy[1]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        longlong2 v = j0 == 0 ? make_longlong2(0, 0) : mine[(2 * h + k) * 32];
+        v.x += __float2ll_rn(fx[k] * fscale);
+        v.y += __float2ll_rn(fy[k] * fscale);
+        mine[(2 * h + k) * 32] = v;
+      }
+    }
+  }
+  if (a != b) add_j<W>(b * T, T, n, sacc, acc, fscale);
+#pragma unroll
+  for (int r = 0; r < RI; ++r)
+    if (ibase + r * 32 < n) {
+      const longlong2 v = mine[r * 32];
+      red_int(acc + 2 * (size_t)(ibase + r * 32), v.x);
+      red_int(acc + 2 * (size_t)(ibase + r * 32) + 1, v.y);
+    }
+  return bad ? ~0ull : zt;
+}
+
+// The small pass (layouts of at most kSmallPoints points).  Such a pass has
+// too few pairs to fill the GPU: what counts is the length of the chain of
+// dependent instructions, not the work.  Every ordered pair is evaluated, so
+// no accumulator travels round a ring (a step of the ring waits 190 cycles
+// for its shuffle; the whole 64-point group takes 3 us) and nothing is added
+// on the j side.  A unit is one CTA of 4 warps: 256 i-points, two per lane,
+// against a chunk of j-points in shared memory.  Twice the arithmetic of the
+// symmetric pass, on units a quarter of its smallest: 2,000 points make 256
+// CTAs.  The chunk is the FP32 partial of a point's force and depends on n
+// alone, so a member of a batch gets the bits of a layout on its own.
+constexpr int kSmallWarps = 4;
+constexpr int kSmallBlock = 64 * kSmallWarps;  // i-points per unit
+constexpr int kSmallMaxChunk = 128;
+__host__ __device__ inline int small_chunk(int n) { return n <= 3072 ? 64 : 128; }
+__host__ __device__ inline int small_chunks(int n) { return (n + small_chunk(n) - 1) / small_chunk(n); }
+__host__ __device__ inline int small_units(int n) { return ((n + kSmallBlock - 1) / kSmallBlock) * small_chunks(n); }
+
+template <class YT>
+__device__ __forceinline__ u64 small_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+                                          float fscale, int ib, int c, float4* sj, bool* bad) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u64 one2 = pk(1.f, 1.f);
+  const int TJ = small_chunk(n);
+  const int i0 = ib * kSmallBlock + warp * 64 + lane, i1 = i0 + 32;
+  const float2 p0 = ld_y(Y, i0), p1 = ld_y(Y, i1);  // padded: the sentinel above n
+  for (int k = tid; k < TJ; k += 32 * kSmallWarps) {
+    const float2 p = ld_y(Y, c * TJ + k);
+    sj[k] = make_float4(-p.x, -p.x, -p.y, -p.y);
+  }
+  const u64 X2 = pk(p0.x, p1.x), Y2 = pk(p0.y, p1.y);
+  u64 FX = 0ull, FY = 0ull, ZG = 0ull;
+  __syncthreads();
+  for (int j0 = 0; j0 < TJ; j0 += kGroup) {
+    u64 Z2 = 0ull;
+#pragma unroll 16
+    for (int j = j0; j < j0 + kGroup; ++j) {
+      const float4 q = sj[j];
+      const u64 dx = add2(X2, pk(q.x, q.y));
+      const u64 dy = add2(Y2, pk(q.z, q.w));
+      u64 qq = fma2(dx, dx, one2);
+      qq = fma2(dy, dy, qq);
+      float q0, q1;
+      upk(qq, q0, q1);
+      const u64 w = pk(rcp_approx(q0), rcp_approx(q1));
+      Z2 = add2(Z2, w);
+      const u64 w2 = mul2(w, w);
+      FX = fma2(w2, dx, FX);
+      FY = fma2(w2, dy, FY);
+    }
+    ZG = add2(ZG, Z2);
+  }
+  float z0, z1, fx0, fx1, fy0, fy1;
+  upk(ZG, z0, z1);
+  upk(FX, fx0, fx1);
+  upk(FY, fy0, fy1);
+  u64 zt = 0ull;
+  float zn = 0.f;
+  if (i0 < n) {
+    red_fix(acc + 2 * (size_t)i0, fx0, fscale);
+    red_fix(acc + 2 * (size_t)i0 + 1, fy0, fscale);
+    zt += z_fix(z0);
+    zn += z0;
+  }
+  if (i1 < n) {
+    red_fix(acc + 2 * (size_t)i1, fx1, fscale);
+    red_fix(acc + 2 * (size_t)i1 + 1, fy1, fscale);
+    zt += z_fix(z1);
+    zn += z1;
+  }
+  *bad = zn != zn;
+  return zt;
+}
+
+// Units per tile pair: j sub-tiles, a power of two.  Passes on tiles of 8
+// i-points per lane (see kMidPoints) cut their tile pairs until the units make 2.2 waves of
+// the grid, down to one ring group per warp: 10,000 points take 30.8 us with
+// four sub-tiles and 40.1 us whole, 20,000 points 95.8 us with two and 98.5 us
+// whole; at 30,000 (whole tiles: 2.8 waves) cutting gains nothing.  Tiles of 16
+// i-points are not cut.  The cut depends on the layout's size and the shape
+// alone: a member of a batch is cut as the layout on its own.
+inline int split_tiles(long pairs, long slots, int RI) {
+  int s = 1;
+  while (RI == 8 && s < RI / 2 && 5 * pairs * s < 11 * slots) s *= 2;
+  return s;
+}
+
+// (a, b) of tile pair u of a layout with nt tiles, numbered diagonal by diagonal:
 // diagonal d = b - a holds the nt - d units (0, d), (1, d + 1), ..., so it
 // starts at sum_{d' < d} (nt - d') = row_start(d, nt).  Units taken one after
 // the other by the persistent grid then touch different tiles: the integer
 // atomics of concurrently finishing units go to different points instead of
 // all to the shared tile a of one row of the triangle.
-__device__ __forceinline__ void unit_tiles(int u, int nt, int* a_out, int* b_out) {
-  int lo = 0, hi = nt - 1;  // largest d with row_start(d) <= u
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (row_start(mid, nt) <= u) lo = mid; else hi = mid - 1;
+static __device__ __noinline__ int2 unit_tiles(int u, int nt) {
+  int d = 0, hi = nt - 1;  // largest d with row_start(d) <= u
+  while (d < hi) {
+    const int mid = (d + hi + 1) >> 1;
+    if (row_start(mid, nt) <= u) d = mid; else hi = mid - 1;
   }
-  *a_out = u - row_start(lo, nt);
-  *b_out = *a_out + lo;
+  const int a = u - row_start(d, nt);
+  return make_int2(a, a + d);
 }
 
 }  // namespace tsgne

@@ -40,10 +40,23 @@ struct Sched {
   uint32_t flags;      // bit 0: non-finite layout seen; bit 1: non-finite P
   uint32_t rep_done;   // last-CTA counter of the repulsion pass
   uint32_t red_done;   // last-CTA counter of the generic reductions
-  uint32_t work_next;  // work-queue head of the symmetric repulsion pass
   float inv_z;         // (float)(1 / Z), written with Z: the rows read it instead of dividing in FP64
   double red[4];       // results of the generic reductions
+  // Symmetric exact pass, one slot for this pass and one for the next (each
+  // pass clears the other slot, so none has to wait for its last CTA):
+  unsigned long long zacc[2][2];  // Z + n in fixed point: low and high 32 bits of every unit's value, summed
+  uint32_t zbad[2];               // 1: a pair's kernel value was NaN
+  uint32_t work_next[2];          // work-queue head
 };
+
+// Z of the symmetric exact pass in fixed point.  A thread's partial of a
+// point (FP32 sums of at most 64 kernel values, then over a unit's groups) is
+// rounded to a multiple of 2^-32; integers add in any order to the same bits,
+// so the units need no partials in memory, no last CTA and no order.  2^-33
+// per partial is far below the FP32 rounding of the partials that hold a
+// point's own term (2^-25).  The low 32 bits of a unit's sum and the rest are
+// added apart: neither sum can pass 2^63 below 2^31 units.
+constexpr int kZShift = 32;
 
 constexpr uint32_t kFlagNonfiniteY = 1u;
 constexpr uint32_t kFlagNonfiniteP = 2u;
@@ -77,7 +90,9 @@ struct RepShape {
   int n_pad = 0;     // padded length of Y buffers
   int n_iblk = 0;    // i-blocks of block*R points
   int n_jtiles = 0;  // j-tiles of jtile points
-  int units = 0;     // work units of one pass (symmetric: tile pairs a <= b)
+  int units = 0;     // work units of one pass (symmetric: tile pairs a <= b, times split)
+  int split = 1;     // j sub-tiles per tile pair (symmetric)
+  bool small = false;  // k_repulsion_small: units are (256 points, jtile points)
   int warps = 0;     // warps per CTA (symmetric)
   size_t smem = 0;   // dynamic shared memory per CTA (symmetric)
 };
@@ -103,6 +118,23 @@ tsgne_status host_guard(F&& f) {
     return TSGNE_ERR_OOM;
   }
 }
+
+// Layouts of at most this many points run k_repulsion_small whatever
+// symmetric shape is asked for (a pass, small against symmetric: 8.6 and 16.7
+// us at 2,000 points, 10.2 and 12.3 at 3,000, 18.5 and 18.4 at 6,000; it does
+// twice the arithmetic, which a batch of many small members pays for: 32
+// members of 500 to 20,000 points take 432 us an iteration with the line
+// here, 460 us with it at 7,168).
+constexpr int kSmallPoints = 4096;
+// Larger layouts of at most this many points run the symmetric pass on tiles
+// of one warp and 8 i-points per lane, whatever symmetric shape is asked for:
+// they have too few tile pairs for even waves of the larger tiles (a pass with
+// 8 and 16 i-points: 30.8 and 37.3 us at 10,000 points, 50.8 and 54.8 at
+// 14,000, 95.8 and 96.9 at 20,000, 318 and 340 at 40,000, but 482 and 471 at
+// 50,000).  Members of a batch follow the same two lines, so that a layout
+// gets the same bits alone and in a batch (an iteration of 32 members of 500
+// to 20,000 points: 398 us, with 16 i-points 432 us).
+constexpr int kMidPoints = 45056;
 
 // Returns TSGNE_ERR_OOM or TSGNE_ERR_CUDA for e and records a message.
 tsgne_status cuda_fail(cudaError_t e, const char* what, const char* file, int line);
@@ -240,35 +272,34 @@ tsgne_status launch_repulsion(const RepShape& sh, int n, const float2* Y, float2
 // Symmetric pass: every unordered pair once (repulsion_sym.cu).  Adds the
 // forces of the n real points into the fixed-point accumulators acc[2 n]
 // (int64 pairs at scale fix_scale(n); zero before the pass, read and
-// cleared by launch_fix_forces after it); Z and the schedule into sched as
-// launch_repulsion does; zpart needs sh.units doubles.
+// cleared by the rows that use them); Z into
+// sched->zacc[slot] (zero before the pass, which clears the other slot) and
+// the schedule into sched as launch_repulsion does.
 // repulsion_sym_prepare sets kernel attributes (call it outside stream
 // capture, once per shape).
 RepShape repulsion_shape_sym(int n, int sm_count);
-// A given shape: W warps per CTA (1 or 2), RI i-points per lane (8 or 16).
+// A given shape: W warps per CTA (1 or 2), RI i-points per lane (8 or 16);
+// layouts of at most kMidPoints points get their own shape whatever is given.
 RepShape repulsion_shape_sym_fixed(int n, int sm_count, int W, int RI);
 tsgne_status repulsion_sym_prepare(const RepShape& sh);
 // Y is float2[n_pad] (y_bf16 = 0) or __nv_bfloat162[n_pad] (y_bf16 = 1).
 tsgne_status launch_repulsion_sym(const RepShape& sh, int n, const void* Y, int y_bf16, unsigned long long* acc,
-                                  double* zpart, Sched* sched, int advance, float ee, int ee_iters, float mom0,
+                                  Sched* sched, int slot, int advance, float ee, int ee_iters, float mom0,
                                   float mom1, cudaStream_t s);
 // A share of the pass for sharding one layout over several GPUs: only units
-// [u0, u1) of the sh.units tile pairs (forces into acc, unit partials into
+// [u0, u1) of the sh.units units (forces into acc, unit partials into
 // zpart[u0..u1)); Z and the schedule are left to launch_finalize_z, after
 // the caller has summed acc and zpart over the shares.
 tsgne_status launch_repulsion_sym_units(const RepShape& sh, int n, const void* Y, int y_bf16,
-                                        unsigned long long* acc, double* zpart, Sched* sched, int u0, int u1,
-                                        cudaStream_t s);
-// Z = fixed-order sum of zpart[0..sh.units) - n and the schedule, as the last
-// CTA of a whole pass sets them (same block size, so the same bits).
-tsgne_status launch_finalize_z(const RepShape& sh, int n, const double* zpart, Sched* sched, int advance, float ee,
+                                        unsigned long long* acc, double* zpart, Sched* sched, int slot, int u0,
+                                        int u1, cudaStream_t s);
+// Z and 1 / Z from zpart[0..sh.units) and the schedule: the bits that a whole
+// pass's sums give.
+tsgne_status launch_finalize_z(const RepShape& sh, const double* zpart, Sched* sched, int slot, int advance, float ee,
                                int ee_iters, float mom0, float mom1, cudaStream_t s);
 // F^r[i] = sum_k part[k * n_pad + i] for k < slots, in slot order (the
 // ordered-pair kernel's partial forces).
 tsgne_status launch_reduce_slots(int n, const float2* part, int slots, int n_pad, float2* out, cudaStream_t s);
-// F^r[i] = acc[2 i .. 2 i + 1] / fix_scale(n) (one FP32 rounding of the exact
-// integer sum), and the accumulators back to zero for the next pass.
-tsgne_status launch_fix_forces(int n, unsigned long long* acc, float2* out, cudaStream_t s);
 
 // ------------------------------------------------------------ iteration
 // Rows with more than kHeavyDeg entries get their attraction from chunks of
@@ -334,9 +365,13 @@ struct AttractArgs {
   void* Ynext16 = nullptr;
   float2* upd = nullptr;
   float2* gains = nullptr;
+  // the repulsion: F^r per row in frep and 1 / Z in sched->inv_z, or (zslot >=
+  // 0) the symmetric pass's accumulators, which the row's thread clears, and Z
+  // in sched->zacc[zslot]
   const float2* frep = nullptr;
-  int chunks = 1;
-  int n_pad = 0;
+  unsigned long long* facc = nullptr;
+  float unscale = 0.f;
+  int zslot = -1;
   Sched* sched = nullptr;
   float eta = 0.f;
   float min_gain = 0.f;
@@ -365,6 +400,7 @@ struct PlanView {
   const int32_t* med_rows = nullptr;
   const int32_t* big = nullptr;     // hub chunks of the rows above 128 entries
   int n_med = 0, n_short = 0, n_big = 0;
+  int short_rows = 256;  // rows of a short CTA
   int64_t entries = 0, n_codes = 0, n_med_rows = 0;  // array lengths (index checks)
 };
 struct AttractPlan {
@@ -373,7 +409,7 @@ struct AttractPlan {
   DevBuf<int32_t> colS, med_rows, big;
   DevBuf<float> PS;
   DevBuf<__nv_bfloat16> PS16;
-  int n_med = 0, n_short = 0, n_big = 0;
+  int n_med = 0, n_short = 0, n_big = 0, short_rows = 256;
   int64_t entries = 0, n_codes = 0, n_med_rows = 0;
   bool ready = false;
   PlanView view() const;

@@ -31,7 +31,7 @@ EDGES = [0, 1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129]
 @pytest.mark.parametrize("degrees,n", [
     ([], 2), ([1], 255), ([3] * 200, 256), ([5] * 200, 257), (EDGES, 513),
     ([33] * 64, 1000), ([33] * 65, 1000), ([128] * 130, 1500),
-    (EDGES + [1023, 1024, 1025, 2047, 2048, 2049], 4099),
+    (EDGES + [1023, 1024, 1025, 2047, 2048, 2049], 4099), (EDGES, 20011), (EDGES, 50021),
 ])
 def test_layout_equals_batch_of_one(degrees, n):
     rp, col = _graph(degrees, n)
