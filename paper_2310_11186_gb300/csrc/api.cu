@@ -680,7 +680,7 @@ tsgne_status tsgne_build_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, co
     DevBuf<int64_t> wrp;
     DevBuf<int32_t> wcol;
     int64_t wnnz = 0;
-    API_TRY(ctx, random_walk_affinities(n, rp.get(), col.get(), nnz, X_d, d, ctx->cfg.p_walks,
+    API_TRY(ctx, random_walk_affinities(n, rp.get(), col.get(), tslot.get(), nnz, X_d, d, ctx->cfg.p_walks,
                                         ctx->cfg.p_walk_length, ctx->cfg.seed, wrp, wcol, P, &wnnz, ctx->sched.get(),
                                         ctx->stream));
     rp = std::move(wrp);

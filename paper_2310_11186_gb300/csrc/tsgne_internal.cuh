@@ -241,6 +241,12 @@ tsgne_status build_affinities(int n, const int64_t* rp, const int32_t* col, cons
                               const float* X, int d, float perplexity, float tol, int max_iter, float* P,
                               Sched* sched, cudaStream_t s);
 
+// dist[e] = ||x_i - x_j||^2 for every entry e = (i, j) of a symmetric structure,
+// FP64, products and sums rounded apart in dimension order (the random
+// walks' definition).
+tsgne_status walk_distances(int64_t nnz, const int64_t* rp, const int32_t* col, const int64_t* tslot, const float* X,
+                            int d, double* dist, cudaStream_t s);
+
 // Eq. 3 from conditional affinities pcond on a symmetric structure with
 // transpose slots: P = (pcond + pcond^T) / total, total into sched->red[0].
 // Synchronises the stream.
@@ -250,7 +256,8 @@ tsgne_status joint_affinities(int64_t nnz, const float* pcond, const int64_t* ts
 // Random-walk estimate (Eq. 6, random_walk.cu): R walks of L steps from
 // every node over the structure (rp, col); allocates the symmetrised
 // structure of the walk pairs and its joint P.  Synchronises the stream.
-tsgne_status random_walk_affinities(int n, const int64_t* rp, const int32_t* col, int64_t nnz, const float* X, int d,
+tsgne_status random_walk_affinities(int n, const int64_t* rp, const int32_t* col, const int64_t* tslot, int64_t nnz,
+                                    const float* X, int d,
                                     int R, int L, uint64_t seed, DevBuf<int64_t>& rp_out, DevBuf<int32_t>& col_out,
                                     DevBuf<float>& P_out, int64_t* nnz_out, Sched* sched, cudaStream_t s);
 
