@@ -247,7 +247,9 @@ tsgne_status tsgne_kernel_times(tsgne_ctx* ctx, double* ms, int64_t* launches, i
  * fails with TSGNE_ERR_OOM before cudaMalloc is called; the object that
  * asked stays usable (a later call may retry).  The paper has no
  * counterpart: the limit serves hosts that share a GPU among tenants, and
- * tests of the out-of-memory paths.
+ * tests of the out-of-memory paths.  Freed memory of the library's objects
+ * stays with the library for its next allocations, at most 256 MiB of it per
+ * device; this call gives all of it back (as a failed allocation does).
  */
 void tsgne_set_device_memory_limit(int64_t bytes);
 
@@ -334,8 +336,8 @@ tsgne_status tsgne_batch_add_ex(tsgne_batch* b, int32_t n, const int64_t* row_pt
  * member (structure, P, buffers, state; same arguments as
  * tsgne_batch_add_ex) on cuda_stream (not NULL, not the batch's stream)
  * without touching the batch's membership, so it may run on another thread
- * while tsgne_batch_run runs; its device memory is allocated stream-ordered
- * on cuda_stream (cudaMallocAsync), which must outlive the member.  It
+ * while tsgne_batch_run runs; the uses of its device memory are ordered
+ * on cuda_stream, which must outlive the member.  It
  * synchronises cuda_stream; on error *out is NULL and tsgne_last_error(NULL)
  * on that thread says why.  tsgne_batch_attach adds a prepared member (it
  * joins at the next run) and consumes the handle; tsgne_batch_discard frees

@@ -2,7 +2,6 @@
 // argument validation, host/device copies, CUDA-graph replay of iterations
 // and per-kernel CUDA-event profiling.  All arithmetic runs in the kernels of
 // structure.cu, affinity.cu, repulsion.cu and iterate.cu.
-#include <atomic>
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -23,28 +22,6 @@ std::string& last_msg() {
   thread_local std::string m;
   return m;
 }
-
-cudaStream_t& alloc_stream() {
-  thread_local cudaStream_t s = nullptr;
-  return s;
-}
-
-namespace {
-std::atomic<int64_t> g_dev_bytes{0};
-std::atomic<int64_t> g_dev_limit{0};  // 0: no limit
-}  // namespace
-
-bool device_bytes_reserve(size_t bytes) {
-  const int64_t b = (int64_t)bytes;
-  const int64_t lim = g_dev_limit.load();
-  int64_t cur = g_dev_bytes.load();
-  do {
-    if (lim > 0 && cur + b > lim) return false;
-  } while (!g_dev_bytes.compare_exchange_weak(cur, cur + b));
-  return true;
-}
-
-void device_bytes_release(size_t bytes) { g_dev_bytes.fetch_sub((int64_t)bytes); }
 
 tsgne_status cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
   std::string s = std::string(what) + ": " + cudaGetErrorString(e) + " (" + file + ":" + std::to_string(line) + ")";
@@ -81,8 +58,8 @@ using namespace tsgne;
 
 struct tsgne_ctx {
   tsgne_config cfg{};
+  OwnedStream own;  // first: outlives the buffers
   cudaStream_t stream = nullptr;
-  bool own_stream = false;
   int device = 0;
   int sms = 1;
   std::string err;
@@ -147,7 +124,6 @@ struct tsgne_ctx {
       cudaEventDestroy(r.b);
     }
     for (auto e : spare) cudaEventDestroy(e);
-    if (own_stream && stream) cudaStreamDestroy(stream);
   }
   void reset_graphs() {
     for (auto& g : g2)
@@ -163,7 +139,8 @@ namespace {
 struct DeviceGuard {
   int prev = -1;
   bool ok = true;
-  explicit DeviceGuard(int dev) {
+  AllocScope as;
+  DeviceGuard(int dev, cudaStream_t s) : as(s) {
     if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
     if (prev != dev) ok = cudaSetDevice(dev) == cudaSuccess;
   }
@@ -614,12 +591,13 @@ tsgne_status tsgne_create(tsgne_ctx** out, const tsgne_config* cfg, void* cuda_s
     if (cuda_stream) {
       ctx->stream = static_cast<cudaStream_t>(cuda_stream);
     } else {
-      e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
-      ctx->own_stream = (e == cudaSuccess);
+      e = cudaStreamCreateWithFlags(&ctx->own.s, cudaStreamNonBlocking);
+      ctx->stream = ctx->own.s;
     }
   }
   tsgne_status st = TSGNE_OK;
   if (e != cudaSuccess) st = cuda_fail(e, "tsgne_create", __FILE__, __LINE__);
+  AllocScope as(ctx->stream);
   if (st == TSGNE_OK) st = ctx->sched.alloc(1);
   if (st == TSGNE_OK) {
     e = cudaMemsetAsync(ctx->sched.get(), 0, sizeof(Sched), ctx->stream);
@@ -636,9 +614,10 @@ tsgne_status tsgne_create(tsgne_ctx** out, const tsgne_config* cfg, void* cuda_s
 
 void tsgne_destroy(tsgne_ctx* ctx) {
   if (!ctx) return;
-  DeviceGuard g(ctx->device);
+  DeviceGuard g(ctx->device, ctx->stream);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   delete ctx;
+  trim_pool();
 }
 
 const char* tsgne_last_error(const tsgne_ctx* ctx) { return ctx ? ctx->err.c_str() : last_msg().c_str(); }
@@ -646,7 +625,7 @@ const char* tsgne_last_error(const tsgne_ctx* ctx) { return ctx ? ctx->err.c_str
 tsgne_status tsgne_build_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, const int32_t* col_idx, const float* X,
                            int32_t d, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (n < 2 || d < 1 || !row_ptr || !X || !valid_kind(ptr_kind))
     return fail(ctx, TSGNE_ERR_INVALID_ARG, "need n >= 2, d >= 1, non-NULL row_ptr and X, a valid ptr_kind");
   int64_t first = 0, m = 0;
@@ -698,13 +677,14 @@ tsgne_status tsgne_build_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, co
   if (h.flags & kFlagNonfiniteP) return fail(ctx, TSGNE_ERR_NONFINITE, "non-finite affinity (check X)");
   API_TRY(ctx, install(ctx, n, nnz, rp, col, P));
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  trim_pool();
   return TSGNE_OK;
 }
 
 tsgne_status tsgne_build_P_shortest_path(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, const int32_t* col_idx,
                                          const int32_t* targets, int32_t d, int32_t l0, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (n < 2 || d < 1 || d > 1024 || !row_ptr || !targets || !valid_kind(ptr_kind))
     return fail(ctx, TSGNE_ERR_INVALID_ARG, "need n >= 2, 1 <= d <= 1024, row_ptr, targets, a valid ptr_kind");
   int64_t first = 0, m = 0;
@@ -726,7 +706,7 @@ tsgne_status tsgne_build_P_shortest_path(tsgne_ctx* ctx, int32_t n, const int64_
 tsgne_status tsgne_set_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, const int32_t* col_idx, const float* Pv,
                          int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (n < 2 || !row_ptr || !valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "need n >= 2 and row_ptr");
   int64_t first = 0, m = 0;
   API_TRY(ctx, read_ends(row_ptr, n, ptr_kind, ctx->stream, &first, &m));
@@ -754,6 +734,7 @@ tsgne_status tsgne_set_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, cons
   API_CUDA(ctx, cudaMemsetAsync(ctx->sched.get(), 0, sizeof(Sched), ctx->stream));
   API_TRY(ctx, install(ctx, n, nnz, rp, col, P));
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  trim_pool();
   return TSGNE_OK;
 }
 
@@ -767,7 +748,7 @@ tsgne_status tsgne_get_sizes(tsgne_ctx* ctx, int32_t* n, int64_t* nnz) {
 
 tsgne_status tsgne_get_P(tsgne_ctx* ctx, int64_t* row_ptr, int32_t* col, float* val, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "bad ptr_kind");
   if (!ctx->have_P) return fail(ctx, TSGNE_ERR_NOT_BUILT, "no affinities yet");
   if (row_ptr) API_TRY(ctx, copy_out(row_ptr, ctx->rp.get(), sizeof(int64_t) * ((size_t)ctx->n + 1), ptr_kind, ctx->stream));
@@ -779,7 +760,7 @@ tsgne_status tsgne_get_P(tsgne_ctx* ctx, int64_t* row_ptr, int32_t* col, float* 
 
 tsgne_status tsgne_init_Y(tsgne_ctx* ctx, const float* Y0, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "bad ptr_kind");
   if (!ctx->have_P) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P first");
   ctx->cur = 0;
@@ -797,7 +778,7 @@ tsgne_status tsgne_init_Y(tsgne_ctx* ctx, const float* Y0, int32_t ptr_kind) {
 
 tsgne_status tsgne_step(tsgne_ctx* ctx) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   API_TRY(ctx, enqueue_step(ctx));
   return TSGNE_OK;
@@ -805,7 +786,7 @@ tsgne_status tsgne_step(tsgne_ctx* ctx) {
 
 tsgne_status tsgne_run(tsgne_ctx* ctx, int32_t n_iter) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (n_iter < 0) return fail(ctx, TSGNE_ERR_INVALID_ARG, "n_iter < 0");
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   int32_t k = 0;
@@ -823,7 +804,7 @@ tsgne_status tsgne_run(tsgne_ctx* ctx, int32_t n_iter) {
 
 tsgne_status tsgne_sync(tsgne_ctx* ctx) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   if (ctx->have_P) API_TRY(ctx, check_flags(ctx));
   return TSGNE_OK;
@@ -831,7 +812,7 @@ tsgne_status tsgne_sync(tsgne_ctx* ctx) {
 
 tsgne_status tsgne_kl(tsgne_ctx* ctx, double* kl_out) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!kl_out) return fail(ctx, TSGNE_ERR_INVALID_ARG, "kl_out is NULL");
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   API_TRY(ctx, enqueue_repulsion(ctx, 0));
@@ -852,7 +833,7 @@ tsgne_status tsgne_kl(tsgne_ctx* ctx, double* kl_out) {
 
 tsgne_status tsgne_gradient(tsgne_ctx* ctx, float alpha, float* g_out, double* z_out, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!g_out || !valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "g_out is NULL or bad ptr_kind");
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   API_TRY(ctx, enqueue_repulsion(ctx, 0));
@@ -870,7 +851,7 @@ tsgne_status tsgne_gradient(tsgne_ctx* ctx, float alpha, float* g_out, double* z
 
 tsgne_status tsgne_get_Y(tsgne_ctx* ctx, float* Y_out, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!Y_out || !valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "Y_out is NULL or bad ptr_kind");
   if (!ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "no layout yet");
   API_TRY(ctx, copy_out(Y_out, ctx->Y[ctx->cur].get(), sizeof(float2) * (size_t)ctx->n, ptr_kind, ctx->stream));
@@ -880,7 +861,7 @@ tsgne_status tsgne_get_Y(tsgne_ctx* ctx, float* Y_out, int32_t ptr_kind) {
 
 tsgne_status tsgne_get_state(tsgne_ctx* ctx, float* Y, float* update, float* gains, int32_t* iter, int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "bad ptr_kind");
   if (!ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "no layout yet");
   const size_t bytes = sizeof(float2) * (size_t)ctx->n;
@@ -896,7 +877,7 @@ tsgne_status tsgne_get_state(tsgne_ctx* ctx, float* Y, float* update, float* gai
 tsgne_status tsgne_set_state(tsgne_ctx* ctx, const float* Y, const float* update, const float* gains, int32_t iter,
                              int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!valid_kind(ptr_kind) || iter < 0 || !Y) return fail(ctx, TSGNE_ERR_INVALID_ARG, "need Y, iter >= 0, ptr_kind");
   if (!ctx->have_P) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P first");
   const size_t bytes = sizeof(float2) * (size_t)ctx->n;
@@ -913,7 +894,7 @@ tsgne_status tsgne_set_state(tsgne_ctx* ctx, const float* Y, const float* update
 
 tsgne_status tsgne_kernel_times(tsgne_ctx* ctx, double* ms, int64_t* launches, int32_t n, int32_t reset) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (n < 0 || n > kClasses) return fail(ctx, TSGNE_ERR_INVALID_ARG, "n outside [0, 8]");
   API_TRY(ctx, prof_collect(ctx));
   for (int k = 0; k < n; ++k) {
@@ -927,10 +908,6 @@ tsgne_status tsgne_kernel_times(tsgne_ctx* ctx, double* ms, int64_t* launches, i
     }
   return TSGNE_OK;
 }
-
-void tsgne_set_device_memory_limit(int64_t bytes) { tsgne::g_dev_limit.store(bytes > 0 ? bytes : 0); }
-
-int64_t tsgne_device_memory_in_use(void) { return tsgne::g_dev_bytes.load(); }
 
 tsgne_status tsgne_repulsion_shape(tsgne_ctx* ctx, int32_t* grid, int32_t* block, int32_t* i_per_thread,
                                    int32_t* j_tile, int32_t* j_chunks, int32_t* n_pad) {
@@ -988,7 +965,7 @@ tsgne_status set_shape(tsgne_ctx* ctx, int warps, int ri, int symmetric) {
 
 tsgne_status tsgne_set_repulsion_shape(tsgne_ctx* ctx, int32_t tile_warps, int32_t i_per_lane, int32_t symmetric) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!ctx->have_P) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P first");
   if (ctx->use_tree) return fail(ctx, TSGNE_ERR_INVALID_ARG, "the tree code has no exact-pass shape");
   if (ctx->shard_pending) return fail(ctx, TSGNE_ERR_INVALID_ARG, "a share is awaiting its finish call");
@@ -1000,7 +977,7 @@ tsgne_status tsgne_set_repulsion_shape(tsgne_ctx* ctx, int32_t tile_warps, int32
 tsgne_status tsgne_autotune(tsgne_ctx* ctx, int32_t trial_passes, int32_t* tile_warps, int32_t* i_per_lane,
                             int32_t* symmetric, float* ms_per_pass) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (trial_passes < 1) return fail(ctx, TSGNE_ERR_INVALID_ARG, "trial_passes < 1");
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   if (ctx->use_tree) return fail(ctx, TSGNE_ERR_INVALID_ARG, "the tree code has no exact-pass shape");
@@ -1072,7 +1049,7 @@ tsgne_status tsgne_shard_set(tsgne_ctx* ctx, int32_t rank, int32_t world) {
 tsgne_status tsgne_shard_repulsion(tsgne_ctx* ctx, int64_t* units, int32_t* u0, int32_t* u1, void** acc,
                                    int64_t* acc_count, void** zunit) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!ctx->have_P || !ctx->have_Y) return fail(ctx, TSGNE_ERR_NOT_BUILT, "build P and set Y first");
   if (ctx->use_tree || ctx->ordered)
     return fail(ctx, TSGNE_ERR_INVALID_ARG, "sharding applies to the symmetric exact repulsion");
@@ -1113,7 +1090,7 @@ tsgne_status shard_close(tsgne_ctx* ctx, int advance) {
 
 tsgne_status tsgne_shard_step_finish(tsgne_ctx* ctx) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!ctx->shard_pending) return fail(ctx, TSGNE_ERR_INVALID_ARG, "no share awaits its finish call");
   API_TRY(ctx, shard_close(ctx, 1));
   API_TRY(ctx, enqueue_update(ctx));
@@ -1123,7 +1100,7 @@ tsgne_status tsgne_shard_step_finish(tsgne_ctx* ctx) {
 tsgne_status tsgne_shard_gradient_finish(tsgne_ctx* ctx, float alpha, float* g_out, double* z_out,
                                          int32_t ptr_kind) {
   TS_TRY(enter(ctx));
-  DeviceGuard dg(ctx->device);
+  DeviceGuard dg(ctx->device, ctx->stream);
   if (!g_out || !valid_kind(ptr_kind)) return fail(ctx, TSGNE_ERR_INVALID_ARG, "g_out is NULL or bad ptr_kind");
   if (!ctx->shard_pending) return fail(ctx, TSGNE_ERR_INVALID_ARG, "no share awaits its finish call");
   API_TRY(ctx, shard_close(ctx, 0));

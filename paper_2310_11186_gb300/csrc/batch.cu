@@ -320,9 +320,9 @@ struct tsgne_member {
 };
 
 struct tsgne_batch {
+  OwnedStream own;  // first: outlives the buffers
   tsgne_config cfg{};
   cudaStream_t stream = nullptr;
-  bool own_stream = false;
   int device = 0, sms = 1;
   int W = 1;
   int RI = kRI;  // i-points per lane of the batched pass
@@ -344,11 +344,10 @@ struct tsgne_batch {
     // admission worker is freed on the worker's stream, not on these
     if (stream) cudaStreamSynchronize(stream);
     for (auto a : aux) cudaStreamSynchronize(a);
-    members.clear();  // stream-ordered frees need their streams
+    members.clear();  // before the streams that order their frees
     if (graph) cudaGraphExecDestroy(graph);
     for (auto e : ev) cudaEventDestroy(e);
     for (auto a : aux) cudaStreamDestroy(a);
-    if (own_stream && stream) cudaStreamDestroy(stream);
   }
 };
 
@@ -486,7 +485,10 @@ tsgne_status refresh_impl(tsgne_batch* b) {
   return TSGNE_OK;
 }
 
-tsgne_status refresh(tsgne_batch* b) { return host_guard([&] { return refresh_impl(b); }); }
+tsgne_status refresh(tsgne_batch* b) {
+  AllocScope as(b->stream);
+  return host_guard([&] { return refresh_impl(b); });
+}
 
 constexpr int kAuxStreams = 8;
 
@@ -739,11 +741,12 @@ tsgne_status tsgne_batch_create(tsgne_batch** out, const tsgne_config* cfg, int3
     if (cuda_stream) {
       b->stream = static_cast<cudaStream_t>(cuda_stream);
     } else {
-      e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
-      b->own_stream = (e == cudaSuccess);
+      e = cudaStreamCreateWithFlags(&b->own.s, cudaStreamNonBlocking);
+      b->stream = b->own.s;
     }
   }
   tsgne_status st = e == cudaSuccess ? TSGNE_OK : cuda_fail(e, "tsgne_batch_create", __FILE__, __LINE__);
+  AllocScope as(b->stream);
   if (st == TSGNE_OK) st = b->d_ctr.alloc(1);
   if (st == TSGNE_OK && cudaMemsetAsync(b->d_ctr.get(), 0, sizeof(BatchCtr), b->stream) != cudaSuccess)
     st = TSGNE_ERR_CUDA;
@@ -762,6 +765,7 @@ void tsgne_batch_destroy(tsgne_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
   delete b;
+  trim_pool();
 }
 
 const char* tsgne_batch_last_error(const tsgne_batch* b) { return b ? b->err.c_str() : ""; }
@@ -778,6 +782,7 @@ tsgne_status tsgne_batch_add_ex(tsgne_batch* b, int32_t n, const int64_t* row_pt
   if (!b) return TSGNE_ERR_INVALID_ARG;
   b->err.clear();
   last_msg().clear();
+  AllocScope as(b->stream);
   std::unique_ptr<Member> mem;
   B_TRY(b, host_guard([&] {
           return prepare_member(b->cfg, b->sms, n, row_ptr, col_idx, X, d, Y0, ptr_kind, repulsion, b->stream, mem);
@@ -796,13 +801,10 @@ tsgne_status tsgne_batch_prepare(tsgne_batch* b, int32_t n, const int64_t* row_p
   int dev = 0;
   TS_CUDA(cudaGetDevice(&dev));
   if (dev != b->device) TS_CUDA(cudaSetDevice(b->device));
-  cudaStream_t& as = alloc_stream();
-  const cudaStream_t saved = as;
-  as = s;  // stream-ordered allocations: no device-wide wait in cudaFree
+  AllocScope as(s);
   std::unique_ptr<Member> mem;
   const tsgne_status st = host_guard(
       [&] { return prepare_member(b->cfg, b->sms, n, row_ptr, col_idx, X, d, Y0, ptr_kind, repulsion, s, mem); });
-  as = saved;
   if (st != TSGNE_OK) return st;
   tsgne_member* h = new (std::nothrow) tsgne_member();
   if (!h) return TSGNE_ERR_OOM;

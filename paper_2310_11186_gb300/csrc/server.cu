@@ -21,9 +21,7 @@
 //      freed.
 // Admission overlaps with the running iterations: an admitted request is
 // handed to a worker thread that builds its member (structure, P, buffers,
-// tree) with tsgne_batch_prepare on the worker's own stream, with
-// stream-ordered allocations (cudaFree would wait for the whole device),
-// while the tick launches the resident layouts' iterations; prepared members
+// tree) with tsgne_batch_prepare on the worker's own stream while the tick launches the resident layouts' iterations; prepared members
 // are attached at the start of the next tick.  A tick with nothing resident
 // waits for all admitted requests to be prepared instead of running nothing.
 // Every member's arithmetic is independent of the others (batch.cu), so a

@@ -158,6 +158,7 @@ extern "C" tsgne_status tsgne_shortest_path_embedding(int32_t n, const int64_t* 
     return TSGNE_ERR_INVALID_ARG;
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  AllocScope as(s ? s : cudaStreamLegacy);
   const cudaMemcpyKind kin = ptr_kind == TSGNE_PTR_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   int64_t first = 0, m = 0;
   if (ptr_kind == TSGNE_PTR_HOST) {

@@ -157,19 +157,44 @@ tsgne_status cuda_fail(cudaError_t e, const char* what, const char* file, int li
 bool device_bytes_reserve(size_t bytes);
 void device_bytes_release(size_t bytes);
 
-// Stream for stream-ordered allocation by the calling thread (NULL: plain
-// cudaMalloc / cudaFree).  cudaFree waits for the whole device, so a thread
-// that prepares work while kernels of others run (the server's admission
-// worker) allocates with cudaMallocAsync / cudaFreeAsync on its own stream.
+// Stream that orders the uses of what the calling thread allocates (NULL:
+// plain cudaMalloc / cudaFree); every entry point sets it to its object's
+// stream (AllocScope).  See memory.cu.
 cudaStream_t& alloc_stream();
+struct AllocScope {
+  cudaStream_t saved;
+  explicit AllocScope(cudaStream_t s) : saved(alloc_stream()) { alloc_stream() = s; }
+  ~AllocScope() { alloc_stream() = saved; }
+  AllocScope(const AllocScope&) = delete;
+  AllocScope& operator=(const AllocScope&) = delete;
+};
+// Device memory, from the kept blocks when alloc_stream() is set (*owner is
+// then that stream, else NULL), and back once everything enqueued on owner is
+// done.
+cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t* owner);
+void device_free(void* p, cudaStream_t owner);
+// Gives idle blocks above the bound (all of them) back to the device.
+void trim_pool();
+void release_idle_blocks();
 
-// Owning device buffer released with cudaFree (or cudaFreeAsync on the
-// stream it was allocated on, if the thread's alloc_stream was set then).
+// A stream that its object destroys after everything declared behind it
+// (buffers are freed on it).
+struct OwnedStream {
+  cudaStream_t s = nullptr;
+  OwnedStream() = default;
+  ~OwnedStream() {
+    if (s) cudaStreamDestroy(s);
+  }
+  OwnedStream(const OwnedStream&) = delete;
+  OwnedStream& operator=(const OwnedStream&) = delete;
+};
+
+// Owning device buffer.
 template <class T>
 struct DevBuf {
   T* p = nullptr;
   size_t n = 0;
-  cudaStream_t as = nullptr;  // stream of a stream-ordered allocation
+  cudaStream_t as = nullptr;  // its owner's stream (device_alloc)
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
@@ -181,7 +206,7 @@ struct DevBuf {
   ~DevBuf() { reset(); }
   void reset() {
     if (p) {
-      if (as) cudaFreeAsync(p, as); else cudaFree(p);
+      device_free(p, as);
       device_bytes_release(n * sizeof(T));
     }
     p = nullptr;
@@ -195,11 +220,12 @@ struct DevBuf {
       last_msg() = "device memory limit reached (tsgne_set_device_memory_limit)";
       return TSGNE_ERR_OOM;
     }
-    cudaStream_t s = alloc_stream();
-    cudaError_t e = s ? cudaMallocAsync(&p, count * sizeof(T), s) : cudaMalloc(&p, count * sizeof(T));
-    if (e == cudaSuccess) as = s;
+    void* q = nullptr;
+    const cudaError_t e = device_alloc(&q, count * sizeof(T), &as);
+    p = static_cast<T*>(q);
     if (e != cudaSuccess) {
       p = nullptr;
+      as = nullptr;
       device_bytes_release(count * sizeof(T));
       return cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
     }
