@@ -34,13 +34,14 @@
 // also gathers the layout into sorted order.  Tree, summaries and group
 // starts: one bottom-up pass, one thread per leaf climbing (each node's
 // parent follows from two neighbouring key prefixes) until it is the first of
-// two children to arrive; a scan numbers the groups in sorted order.  Walk: a persistent grid takes groups from a queue, one warp per
-// group, lane = point; per round the lanes decide up to 32 stack entries at
-// once and then all apply the round's accepted nodes and exact points, so
-// the dependent node loads along the tree are issued 32 at a time.  Z: FP32
-// partial sums flushed into FP64 every round, a fixed xor butterfly per warp,
-// one FP64 partial per group, and the group partials added in group order by
-// the last CTA -- bit-reproducible from run to run.
+// two children to arrive; the marks of the group starts are then listed.
+// Walk: a persistent grid takes groups from a queue, one warp per group,
+// lane = point; per round the lanes decide up to 32 stack entries at once and
+// then all apply the round's accepted nodes and exact points, so the dependent
+// node loads along the tree are issued 32 at a time.  Z: FP32 partial sums of a
+// round, added without loss into a pair of FP32 sums per lane, the pairs over
+// the warp's lanes, and every group's total as an integer multiple of 2^-32 --
+// the same bits in whatever order groups finish.
 #include <cmath>
 
 #include "f32x2.cuh"
@@ -95,15 +96,18 @@ __device__ __forceinline__ float4 block_box(float lx, float ly, float hx, float 
 }
 
 // Also clears the sort's digit counts, tile counters and tile status words
-// (zero[0..nzero)), the group starts (is_start[0..n)) and the stall mark for
-// the build that follows.
+// (zero[0..nzero)), the group starts, the number of groups and the stall mark
+// for the build that follows.
 __global__ void __launch_bounds__(256) k_tree_box(const float2* __restrict__ Y, int n, float4* __restrict__ part,
                                                   TreeState* st, uint32_t* __restrict__ zero, int64_t nzero,
-                                                  int32_t* __restrict__ is_start) {
+                                                  uint32_t* __restrict__ starts) {
   __shared__ float4 ws[8];
   for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < nzero; k += (int64_t)gridDim.x * 256) zero[k] = 0u;
-  for (int k = blockIdx.x * 256 + threadIdx.x; k < n; k += gridDim.x * 256) is_start[k] = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->sort_stall = 0u;
+  for (int k = blockIdx.x * 256 + threadIdx.x; k <= n / 32; k += gridDim.x * 256) starts[k] = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->sort_stall = 0u;
+    st->groups = 0u;
+  }
   float lx = INFINITY, ly = INFINITY, hx = -INFINITY, hy = -INFINITY;
   for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
     const float2 p = Y[i];
@@ -155,12 +159,16 @@ __device__ __forceinline__ uint32_t cell32(float v, double lo, double scale) {
 
 // Keys and the identity permutation, plus the counts of every 8-bit digit
 // of every key for all eight passes at once (ghist[pass][digit], zeroed by
-// k_tree_box): one read of the layout serves the whole sort.
-__global__ void __launch_bounds__(256) k_tree_keys(const float2* __restrict__ Y, int n,
+// k_tree_box): one read of the layout serves the whole sort.  One large CTA
+// per SM: the counts of a CTA are 2,048 global additions, and the FP64 pipe
+// (14 instructions per point and warp, 16 cycles each) needs warps to overlap
+// with (300,000 points: 13.7 us with 8 warps per SM, 11.2 us with 32).
+constexpr int kKeyThreads = 1024;
+__global__ void __launch_bounds__(kKeyThreads) k_tree_keys(const float2* __restrict__ Y, int n,
                                                    const TreeState* __restrict__ st, uint64_t* __restrict__ keys,
                                                    int32_t* __restrict__ vals, uint32_t* __restrict__ ghist) {
   __shared__ uint32_t h[kRadixPasses * kRadixBins];
-  for (int k = threadIdx.x; k < kRadixPasses * kRadixBins; k += 256) h[k] = 0u;
+  for (int k = threadIdx.x; k < kRadixPasses * kRadixBins; k += kKeyThreads) h[k] = 0u;
   __syncthreads();
   const double lx = st->lo_x, ly = st->lo_y, sc = st->scale;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -172,7 +180,7 @@ __global__ void __launch_bounds__(256) k_tree_keys(const float2* __restrict__ Y,
     for (int q = 0; q < kRadixPasses; ++q) atomicAdd(&h[q * kRadixBins + (int)((key >> (8 * q)) & 255u)], 1u);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < kRadixPasses * kRadixBins; k += 256)
+  for (int k = threadIdx.x; k < kRadixPasses * kRadixBins; k += kKeyThreads)
     if (h[k]) atomicAdd(ghist + k, h[k]);
 }
 
@@ -396,13 +404,15 @@ __device__ __forceinline__ unsigned long long atom_exch_acq_rel(unsigned long lo
   return old;
 }
 
+__device__ __forceinline__ void mark_start(uint32_t* starts, int k) { atomicOr(starts + (k >> 5), 1u << (k & 31)); }
+
 __global__ void k_tree_climb(int n, const uint64_t* __restrict__ keys, const float2* __restrict__ ys,
                              unsigned long long* slot, float4* box, float2* sum, float4* __restrict__ nodeA,
-                             int4* __restrict__ nodeB, int32_t* __restrict__ is_start, TreeState* st) {
+                             int4* __restrict__ nodeB, uint32_t* __restrict__ starts, TreeState* st) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n || __ldcg(&st->sort_stall)) return;
   if (n == 1) {
-    is_start[0] = 1;
+    mark_start(starts, 0);
     st->root = ~0;
     return;
   }
@@ -452,12 +462,12 @@ __global__ void k_tree_climb(int n, const uint64_t* __restrict__ keys, const flo
     nodeA[p] = make_float4(__fdiv_rn(sc.x, cnt), __fdiv_rn(sc.y, cnt), __fmul_rn(r, r), cnt);
     nodeB[p] = toward_right ? make_int4(id, sid, pL, pR) : make_int4(sid, id, pL, pR);
     if (cntp > kGroupMax) {
-      if (p - pL + 1 <= kGroupMax) is_start[pL] = 1;     // left child [pL, p]
-      if (pR - p <= kGroupMax) is_start[p + 1] = 1;      // right child [p + 1, pR]
+      if (p - pL + 1 <= kGroupMax) mark_start(starts, pL);  // left child [pL, p]
+      if (pR - p <= kGroupMax) mark_start(starts, p + 1);   // right child [p + 1, pR]
     }
     if (pL == 0 && pR == n - 1) {  // the root
       st->root = p;
-      if (cntp <= kGroupMax) is_start[0] = 1;
+      if (cntp <= kGroupMax) mark_start(starts, 0);
       return;
     }
     L = pL;
@@ -468,13 +478,31 @@ __global__ void k_tree_climb(int n, const uint64_t* __restrict__ keys, const flo
 
 // --------------------------------------------------------------- 6. groups
 
-// gstart[g] = first position of group g; gstart[ngroups] = n.
-__global__ void k_tree_group_list(int n, const TreeState* st, const int32_t* __restrict__ is_start,
-                                  const int64_t* __restrict__ gscan, int32_t* __restrict__ gstart) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n || __ldcg(&st->sort_stall)) return;
-  if (is_start[k]) gstart[gscan[k]] = k;
-  if (k == 0) gstart[gscan[n]] = n;
+// The groups (first position, end) from the marks, one thread per 32
+// positions; a CTA's groups are listed in order at a place of its own, CTAs in
+// any order (nothing depends on it).  A group holds at most 32 points, so it
+// ends at the next mark of its word or of the next one, or at n.
+__global__ void __launch_bounds__(256) k_tree_groups(int n, TreeState* st, const uint32_t* __restrict__ starts,
+                                                     int2* __restrict__ groups) {
+  __shared__ uint2 wsum[8];
+  __shared__ uint32_t base;
+  if (__ldcg(&st->sort_stall)) return;
+  const int words = (n + 31) / 32;
+  const int w = blockIdx.x * 256 + threadIdx.x;
+  const uint32_t m = w < words ? starts[w] : 0u;
+  const uint32_t next = w + 1 < words ? starts[w + 1] : 0u;
+  uint32_t at, unused;
+  const uint32_t cnt = (uint32_t)__popc(m);
+  block_excl_scan2(cnt, 0u, at, unused, wsum);
+  if (threadIdx.x == 255) base = atomicAdd(&st->groups, at + cnt);
+  __syncthreads();
+  const int after = next ? 32 * (w + 1) + __ffs((int)next) - 1 : n;
+  uint32_t left = m;
+  for (uint32_t k = 0; k < cnt; ++k) {
+    const int b = __ffs((int)left) - 1;
+    left &= left - 1u;
+    groups[base + at + k] = make_int2(32 * w + b, left ? 32 * w + __ffs((int)left) - 1 : after);
+  }
 }
 
 // ---------------------------------------------------------------- 7. walk
@@ -492,7 +520,7 @@ __global__ void k_tree_group_list(int n, const TreeState* st, const int32_t* __r
 // definition's; only the order of the sums differs from a depth-first walk.
 // A round's interactions form one list: an accepted node is one item
 // (centre, count), an exact entry is one item per point (point, 1).  The
-// deciding lanes write their items at offsets from a warp scan of the item
+// deciding lanes write their items at offsets from ballots over the item
 // counts, as negated x, negated y and weight arrays, so two items are read as
 // three FP32x2 words and go through the packed arithmetic unchanged.  A
 // lane's own point, when an exact entry holds it, is summed like any other
@@ -508,6 +536,7 @@ __global__ void k_tree_group_list(int n, const TreeState* st, const int32_t* __r
 // per tree level, and the tree has at most 94 levels: 64 key bits and 30
 // index bits), so the stack stays below kWalkStack - 74.
 constexpr int kWalkStack = 512;
+static_assert(kTreeBucket <= 7, "a lane's items of a round are counted in three bits");
 constexpr int kWalkList = 32 * kTreeBucket + 4;  // items of one round at most, plus padding (even)
 
 // Two interactions at once: items (-x, -y, c) packed in pairs against p; FX,
@@ -527,12 +556,35 @@ __device__ __forceinline__ void interact2(u64 PX, u64 PY, u64 NX, u64 NY, u64 C,
   FY = fma2(cw2, dy, FY);
 }
 
+// Sums without loss: two FP32 sums (s, e) whose exact sum is that of the terms
+// up to about 2^-47 of it (Knuth's two-sum; e collects its errors).  Packed
+// FP32x2 for the two halves a lane accumulates, scalar across lanes.  FP64
+// would be as exact, but a double conversion or addition occupies the SM's FP64
+// pipe for 16 cycles: with four a round it was 59 % busy and the walk waited
+// for it (a walk over 300,000 spread
+// points: 157 us, 139 us with these sums and the item counts from ballots).
+__device__ __forceinline__ void two_sum2(u64& S, u64& E, u64 z) {
+  const u64 m1 = pk(-1.f, -1.f);
+  const u64 s = add2(S, z);
+  const u64 b = fma2(S, m1, s);          // s - S
+  const u64 a = fma2(b, m1, s);          // s - b
+  const u64 e = add2(fma2(a, m1, S), fma2(b, m1, z));
+  S = s;
+  E = add2(E, e);
+}
+__device__ __forceinline__ void two_sum(float& s, float& e, float t, float te) {
+  const float r = __fadd_rn(s, t);
+  const float b = __fsub_rn(r, s);
+  const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(r, b)), __fsub_rn(t, b));
+  s = r;
+  e = __fadd_rn(__fadd_rn(e, te), d);
+}
+
 __global__ void __launch_bounds__(32 * kWalkWarps, 4)
     k_tree_walk(int n, const float2* __restrict__ ys, const int32_t* __restrict__ perm,
-                const float4* __restrict__ nodeA, const int4* __restrict__ nodeB, const int32_t* __restrict__ gstart,
-                const int64_t* __restrict__ gscan, float theta2, float2* __restrict__ frep,
-                double* __restrict__ zgroup, Sched* sched, TreeState* st, int advance, float ee, int ee_iters,
-                float mom0, float mom1) {
+                const float4* __restrict__ nodeA, const int4* __restrict__ nodeB, const int2* __restrict__ groups,
+                float theta2, float2* __restrict__ frep, Sched* sched, TreeState* st, int advance, float ee,
+                int ee_iters, float mom0, float mom1) {
   __shared__ int stk[kWalkWarps][kWalkStack];
   __shared__ __align__(8) float lnx[kWalkWarps][kWalkList];
   __shared__ __align__(8) float lny[kWalkWarps][kWalkList];
@@ -542,7 +594,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
   // A sort wait that ran out leaves no valid tree: the pass only zeroes the
   // forces and reports the timeout.
   const bool stalled = __ldcg(&st->sort_stall) != 0u;
-  const int ngroups = stalled ? 0 : (int)gscan[n];
+  const int ngroups = stalled ? 0 : (int)__ldcg(&st->groups);
   const int root = __ldcg(&st->root);  // internal node id, or ~0 for a single point
   if (stalled)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -552,14 +604,15 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
     if (lane == 0) g = (int)atomicAdd(&st->next_group, 1u);
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= ngroups) break;
-    const int k0 = gstart[g], k1 = gstart[g + 1];
+    const int2 gr = groups[g];
+    const int k0 = gr.x, k1 = gr.y;
     const int k = k0 + lane;
     const bool act = k < k1;
     const float2 p = ys[act ? k : k0];
     const float gx0 = warp_min(p.x), gy0 = warp_min(p.y), gx1 = warp_max(p.x), gy1 = warp_max(p.y);
     const u64 PX = pk(p.x, p.x), PY = pk(p.y, p.y);
     u64 FX = 0ull, FY = 0ull;
-    double zd = 0.0;
+    u64 ZS = 0ull, ZE = 0ull;
     bool overflow = false;
     uint32_t seen = 0u;  // lanes whose own point an exact entry held
     if (lane == 0) stk[w][0] = root;
@@ -589,16 +642,17 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
         kind = A.z < __fmul_rn(theta2, d2) ? 1 : (B.w - B.z + 1 <= kTreeBucket ? 2 : 3);
       }
       const uint32_t mo = __ballot_sync(0xffffffffu, kind == 3);
-      // list offsets: exclusive scan of the items per lane
+      // list offsets: the items per lane, summed over the lanes below bit by
+      // bit; from ballots, so that the compiler knows the number of items to
+      // be the same in every lane (uniform loop and addresses below: 5 %)
       const int cnt = kind == 1 ? 1 : (kind == 2 ? B.w - B.z + 1 : 0);
-      int off = cnt;
+      int off = 0, ni = 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, off, o);
-        if (lane >= o) off += u;
+      for (int bit = 0; bit < 3; ++bit) {
+        const uint32_t m = __ballot_sync(0xffffffffu, (cnt >> bit) & 1);
+        off += __popc(m & lt) << bit;
+        ni += __popc(m) << bit;
       }
-      const int ni = __shfl_sync(0xffffffffu, off, 31);
-      off -= cnt;
       if (kind == 1 && TS_IN(off, 0, kWalkList, &sched->flags)) {
         lnx[w][off] = -A.x;
         lny[w][off] = -A.y;
@@ -640,16 +694,24 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
       for (int t = 0; t < ni && TS_IN(t + 1, 0, kWalkList, &sched->flags); t += 2)
         interact2(PX, PY, *reinterpret_cast<const u64*>(&lnx[w][t]), *reinterpret_cast<const u64*>(&lny[w][t]),
                   *reinterpret_cast<const u64*>(&lc[w][t]), FX, FY, Z);
-      float z0, z1;
-      upk(Z, z0, z1);
-      zd += (double)z0 + (double)z1;
+      two_sum2(ZS, ZE, Z);
     }
-    if ((seen >> lane) & 1u) zd -= (double)rcp_approx(1.0f);  // the lane's own term out
-    if (!act) zd = 0.0;                                          // idle lanes add nothing
+    float zs, ze, z1, e1;
+    upk(ZS, zs, z1);
+    upk(ZE, ze, e1);
+    two_sum(zs, ze, z1, e1);
+    if ((seen >> lane) & 1u) two_sum(zs, ze, -rcp_approx(1.0f), 0.f);  // the lane's own term out
+    if (!act) zs = ze = 0.f;                                          // idle lanes add nothing
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) zd += __shfl_xor_sync(0xffffffffu, zd, o);
+    for (int o = 16; o > 0; o >>= 1)
+      two_sum(zs, ze, __shfl_xor_sync(0xffffffffu, zs, o), __shfl_xor_sync(0xffffffffu, ze, o));
     if (lane == 0) {
-      zgroup[g] = zd;
+      const double z = (double)zs + (double)ze;
+      const long long whole = __double2ll_rd(z);
+      const unsigned long long part = __double2ull_rn((z - (double)whole) * 4294967296.0);
+      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&st->zsum[0]), "l"(part) : "memory");
+      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&st->zsum[1]), "l"(whole) : "memory");
+      if (z != z) atomicOr(&st->zbad, 1u);
       if (overflow) atomicOr(&sched->flags, kFlagTreeOverflow);
     }
     if (act) {
@@ -660,8 +722,12 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
     }
   }
   if (arrive_last(&st->walk_done)) {
-    const double total = sum_partials(zgroup, ngroups);
     if (threadIdx.x == 0) {
+      const long long whole = (long long)__ldcg(&st->zsum[1]);
+      const double total = __ldcg(&st->zbad) ? (double)NAN
+                                             : (double)whole + (double)__ldcg(&st->zsum[0]) * (1.0 / 4294967296.0);
+      st->zsum[0] = st->zsum[1] = 0ull;
+      st->zbad = 0u;
       st->next_group = 0u;
       if (stalled)
         atomicOr(&sched->flags, kFlagWaitTimeout);
@@ -694,7 +760,7 @@ tsgne_status TreeBufs::alloc(int n_points, int sm_count, cudaStream_t s) {
   }
   ntiles = (n + kSortTile - 1) / kSortTile;
   box_blocks = grid_for(n, 256, 2 * sm_count);
-  keys_blocks = grid_for(n, 1024, sm_count);
+  keys_blocks = grid_for(n, kKeyThreads, sm_count);
   int per_sm = 0;
   TS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree_walk, 32 * kWalkWarps, 0));
   walk_blocks = sm_count * (per_sm > 0 ? per_sm : 1);
@@ -705,17 +771,14 @@ tsgne_status TreeBufs::alloc(int n_points, int sm_count, cudaStream_t s) {
   TS_TRY(vals[1].alloc((size_t)n));
   TS_TRY(ys.alloc((size_t)n));
   TS_TRY(sortmem.alloc(sort_words()));
-  TS_TRY(scan_scr.alloc(scan_scratch_bytes(n) / sizeof(int64_t)));
-  TS_TRY(is_start.alloc((size_t)n));
-  TS_TRY(gscan.alloc((size_t)n + 1));
-  TS_TRY(gstart.alloc((size_t)n + 1));
+  TS_TRY(starts.alloc((size_t)n / 32 + 1));
+  TS_TRY(groups.alloc((size_t)n));
   TS_TRY(nodeA.alloc(nn));
   TS_TRY(nodeB.alloc(nn));
   TS_TRY(box.alloc(nn));
   TS_TRY(sum.alloc(nn));
   TS_TRY(slot.alloc(nn));
   TS_TRY(boxpart.alloc((size_t)box_blocks));
-  TS_TRY(zgroup.alloc((size_t)n));
   TS_TRY(state.alloc(1));
   TS_CUDA(cudaMemsetAsync(slot.get(), 0xff, sizeof(unsigned long long) * nn, s));  // every slot empty
   TS_CUDA(cudaMemsetAsync(state.get(), 0, sizeof(TreeState), s));
@@ -729,8 +792,8 @@ tsgne_status launch_tree_build(TreeBufs& tb, const float2* Y, cudaStream_t s) {
   uint32_t* ctl = ghist + kRadixPasses * kRadixBins;
   uint32_t* status = ctl + kRadixPasses;
   k_tree_box<<<tb.box_blocks, 256, 0, s>>>(Y, n, tb.boxpart.get(), st, tb.sortmem.get(), (int64_t)tb.sort_words(),
-                                           tb.is_start.get());
-  k_tree_keys<<<tb.keys_blocks, 256, 0, s>>>(Y, n, st, tb.keys[0].get(), tb.vals[0].get(), ghist);
+                                           tb.starts.get());
+  k_tree_keys<<<tb.keys_blocks, kKeyThreads, 0, s>>>(Y, n, st, tb.keys[0].get(), tb.vals[0].get(), ghist);
   TS_CUDA(cudaGetLastError());
   for (int pass = 0; pass < kRadixPasses; ++pass) {
     const int in = pass & 1, out = in ^ 1;
@@ -745,11 +808,8 @@ tsgne_status launch_tree_build(TreeBufs& tb, const float2* Y, cudaStream_t s) {
   static_assert(kRadixPasses % 2 == 0, "sorted keys end in slot 0");
   k_tree_climb<<<grid_for(n, 256, 1 << 30), 256, 0, s>>>(n, tb.keys[0].get(), tb.ys.get(), tb.slot.get(),
                                                          tb.box.get(), tb.sum.get(), tb.nodeA.get(), tb.nodeB.get(),
-                                                         tb.is_start.get(), st);
-  TS_CUDA(cudaGetLastError());
-  TS_TRY(scan_i32_to_i64(tb.is_start.get(), tb.gscan.get(), n, tb.scan_scr.get(), s));
-  k_tree_group_list<<<grid_for(n, 256, 1 << 30), 256, 0, s>>>(n, st, tb.is_start.get(), tb.gscan.get(),
-                                                               tb.gstart.get());
+                                                         tb.starts.get(), st);
+  k_tree_groups<<<grid_for((n + 31) / 32, 256, 1 << 30), 256, 0, s>>>(n, st, tb.starts.get(), tb.groups.get());
   TS_CUDA(cudaGetLastError());
   return TSGNE_OK;
 }
@@ -758,9 +818,8 @@ tsgne_status launch_tree_walk(TreeBufs& tb, float theta, float2* frep, Sched* sc
                               int ee_iters, float mom0, float mom1, cudaStream_t s) {
   const float theta2 = theta * theta;
   k_tree_walk<<<tb.walk_blocks, 32 * kWalkWarps, 0, s>>>(tb.n, tb.ys.get(), tb.vals[0].get(), tb.nodeA.get(),
-                                                         tb.nodeB.get(), tb.gstart.get(), tb.gscan.get(), theta2,
-                                                         frep, tb.zgroup.get(), sched, tb.state.get(), advance, ee,
-                                                         ee_iters, mom0, mom1);
+                                                         tb.nodeB.get(), tb.groups.get(), theta2, frep, sched,
+                                                         tb.state.get(), advance, ee, ee_iters, mom0, mom1);
   TS_CUDA(cudaGetLastError());
   return TSGNE_OK;
 }

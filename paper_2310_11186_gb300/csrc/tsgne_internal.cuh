@@ -478,6 +478,9 @@ struct TreeState {
   uint32_t next_group;           // work-queue head of the walk
   uint32_t sort_stall;           // 1: a look-back wait of this pass's sort ran out of its budget
   int32_t root;                  // root of the last tree: an internal node id, or ~0 (one point)
+  uint32_t groups;               // groups of the last tree
+  uint32_t zbad;                 // 1: a group's Z was NaN
+  unsigned long long zsum[2];    // Z of the walk: fractions of 2^-32 and whole units, summed apart
 };
 
 // Device buffers of the tree code for n points.
@@ -488,17 +491,14 @@ struct TreeBufs {
   DevBuf<int32_t> vals[2];    // vals[0] after a build: sorted position -> point
   DevBuf<float2> ys;          // layout in sorted order
   DevBuf<uint32_t> sortmem;   // sort: digit counts [8][256], tile counters [8], tile status [8][ntiles][256]
-  DevBuf<int64_t> scan_scr;
   DevBuf<float4> nodeA;       // internal node: centre x, y, r2, count
   DevBuf<int4> nodeB;         // internal node: left, right, first, last
   DevBuf<float4> box;         // internal node: x0, y0, x1, y1
   DevBuf<float2> sum;         // internal node: coordinate sums
   DevBuf<unsigned long long> slot;  // bottom-up exchange slots (kept empty, all ones, between passes)
   DevBuf<float4> boxpart;
-  DevBuf<int32_t> is_start;   // 1 where a group begins (sorted positions)
-  DevBuf<int64_t> gscan;      // exclusive scan of is_start; gscan[n] = number of groups
-  DevBuf<int32_t> gstart;     // first sorted position of each group, then n
-  DevBuf<double> zgroup;      // FP64 Z partial per group
+  DevBuf<uint32_t> starts;    // bit k: a group begins at sorted position k
+  DevBuf<int2> groups;        // first sorted position and end of each group, in any order
   DevBuf<TreeState> state;
   size_t sort_words() const { return (size_t)8 * 256 + 8 + (size_t)8 * ntiles * 256; }
   tsgne_status alloc(int n_points, int sm_count, cudaStream_t s);
