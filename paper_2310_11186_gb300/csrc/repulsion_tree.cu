@@ -32,9 +32,9 @@
 // warps, offsets across warps) and takes the tile's global offsets from the
 // tiles before it by a decoupled look-back (a bounded wait).  The last pass
 // also gathers the layout into sorted order.  Tree, summaries and group
-// starts: one bottom-up pass, one thread per leaf climbing (each node's
-// parent follows from two neighbouring key prefixes) until it is the first of
-// two children to arrive; the marks of the group starts are then listed.
+// starts: bottom up in shared memory, tile by tile, one thread per leaf climbing
+// (each node's parent follows from two neighbouring key prefixes) until it is the
+// first of two children to arrive; the marks of the group starts are then listed.
 // Walk: a persistent grid takes groups from a queue, one warp per group,
 // lane = point; per round the lanes decide up to 32 stack entries at once and
 // then all apply the round's accepted nodes and exact points, so the dependent
@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(256) k_tree_box(const float2* __restrict__ Y, 
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->sort_stall = 0u;
     st->groups = 0u;
+    st->climb_global = 0u;
   }
   float lx = INFINITY, ly = INFINITY, hx = -INFINITY, hy = -INFINITY;
   for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
@@ -372,22 +373,42 @@ __global__ void __launch_bounds__(kSortThreads)
 
 // ---------------------------------------------------------------- 4. tree
 
-// Tree, summaries and group starts in one bottom-up pass (agglomerative
-// construction of the binary radix tree, Apetrei 2014): the thread of leaf k
-// holds a node with range [L, R] and climbs.  The parent of [L, R] is the
-// node split between R and R + 1 if the augmented keys R, R + 1 share a
-// longer prefix than keys L - 1, L (a range end counts as -1), else the node
-// split between L - 1 and L; this gives exactly the tree of the definition
-// (the one whose node over [f, l] splits at the highest differing bit).
-// Internal node ids are their split positions (node g has children over
-// [f, g] and [g + 1, l]); leaves are ~position.  A child reaching its parent
-// exchanges (the end of the parent's range it knows, its own id) with the
-// parent's slot: the first arrival leaves, the second learns the sibling,
-// computes the parent (left + right: FP32 addition is commutative, so it
-// does not matter which child's thread that is) and climbs on.  A completed
-// node of more than kGroupMax points marks the first positions of its
-// children that hold at most kGroupMax (the groups: maximal subtrees of at
-// most kGroupMax points).
+// Tree, summaries and group starts bottom up (agglomerative construction of the
+// binary radix tree, Apetrei 2014): the thread of leaf k holds a node with
+// range [L, R] and climbs.  The parent of [L, R] is the node split between R
+// and R + 1 if the augmented keys R, R + 1 share a longer prefix than keys
+// L - 1, L (a range end counts as -1), else the node split between L - 1 and L;
+// this gives exactly the tree of the definition (the one whose node over
+// [f, l] splits at the highest differing bit).  Internal node ids are their
+// split positions (node g has children over [f, g] and [g + 1, l]); leaves are
+// ~position.  A child reaching its parent exchanges (the end of the parent's
+// range it knows, its own id) with the parent's slot: the first arrival
+// leaves, the second learns the sibling, computes the parent (left + right:
+// FP32 addition is commutative, so it does not matter which child's thread
+// that is) and climbs on.  A completed node of more than kGroupMax points marks
+// the first positions of its children that hold at most kGroupMax (the groups:
+// maximal subtrees of at most kGroupMax points).
+//
+// A climb is a chain of exchanges, 32 deep for 300,000 spread points.  Through
+// L2 an exchange with its fence and the load of the sibling's summary take
+// 2 us, so nearly all of them are made in shared memory, over tiles of
+// at most 1,024 consecutive nodes:
+//   1. the leaves: a tile builds every node whose range lies inside it and
+//      hands on the rest of its forest, about 11 subtrees;
+//   2. while there are more than kUpTiles tiles: the subtrees of kUpTiles tiles
+//      each, likewise;
+//   3. what is left, by one CTA.
+// The finished nodes are written afterwards, thread j the one split before
+// starting node j: side by side, and all divisions at once (written in the climb,
+// each exchange waits for the stores: 66 us for 300,000 points instead of 52).
+// Whether a node's parent lies inside the tile is known beforehand: it does not
+// exactly if the prefix it splits at is also shared with the key beyond the
+// tile's end, i.e. if no shorter prefix lies between (a running minimum over
+// the tile).  If a tile of steps 2 or 3 would hold more than 1,024 subtrees
+// (points nested around the tiles' ends; one tile can leave 193), step 3
+// climbs from all subtrees of step 1 through global memory instead.
+// 300,000 points: 69 us with every exchange in L2, 17 + 14 + 11 us now; 2,097,152
+// points: 237 us, 85 + 15 + 14 us now.
 constexpr int kGroupMax = 32;
 constexpr unsigned long long kSlotEmpty = ~0ull;
 
@@ -396,84 +417,367 @@ __device__ __forceinline__ int aug_prefix(uint64_t ka, uint64_t kb, int a, int b
   return ka != kb ? __clzll((long long)(ka ^ kb)) : 64 + __clz((uint32_t)a ^ (uint32_t)b);
 }
 
-// Exchange at a node: acquire-release, so the summary a child's thread
-// stored before its exchange is visible to the sibling's thread after its own.
+__device__ __forceinline__ void mark_start(uint32_t* starts, int k) { atomicOr(starts + (k >> 5), 1u << (k & 31)); }
+
+// Where finished nodes go.
+struct TreeOut {
+  float4* nodeA;
+  int4* nodeB;
+  uint32_t* starts;
+  TreeState* st;
+};
+
+// The node split after position p with range [pL, pR], children left and right.
+__device__ __forceinline__ void put_node(const TreeOut& o, int p, int pL, int pR, int left, int right, float4 box,
+                                         float2 sum) {
+  const int count = pR - pL + 1;
+  const float cnt = (float)count;
+  const float r = fmaxf(__fsub_rn(box.z, box.x), __fsub_rn(box.w, box.y));
+  o.nodeA[p] = make_float4(__fdiv_rn(sum.x, cnt), __fdiv_rn(sum.y, cnt), __fmul_rn(r, r), cnt);
+  o.nodeB[p] = make_int4(left, right, pL, pR);
+  if (count > kGroupMax) {
+    if (p - pL + 1 <= kGroupMax) mark_start(o.starts, pL);  // left child [pL, p]
+    if (pR - p <= kGroupMax) mark_start(o.starts, p + 1);   // right child [p + 1, pR]
+  }
+}
+__device__ __forceinline__ void put_root(const TreeOut& o, int id, int count) {
+  o.st->root = id;
+  if (count <= kGroupMax) mark_start(o.starts, 0);
+}
+__device__ __forceinline__ float4 box_union(float4 a, float4 b) {
+  return make_float4(fminf(a.x, b.x), fminf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
+}
+
+// Subtrees handed on by tiles: tile t's are entries t kItemCap ... in
+// position order, counts[t] of them.
+constexpr int kTileLeaves = 1024;  // nodes a tile starts from, one per thread
+constexpr int kItemCap = 256;      // a tile leaves at most 2 * 96 + 1 subtrees: one per prefix length and side
+constexpr int kUpTiles = 48;       // tiles whose subtrees one CTA of step 2 joins (about 520)
+struct Items {
+  int4* at;  // first, last position, id
+  float4* box;
+  float2* sum;
+  int32_t* counts;
+};
+
+// Shared memory of a tile.  Boundary j lies between nodes j - 1 and j.
+struct ClimbTile {
+  uint32_t slot[kTileLeaves];            // exchange at boundary j: far end << 16 | ref
+  float4 box[kTileLeaves];               // of the node built at boundary j
+  float4 ibox[kTileLeaves];              // of starting node j
+  float2 sum[kTileLeaves], isum[kTileLeaves];
+  ushort2 child[kTileLeaves];            // refs of the children of the node built at boundary j
+  short2 ends[kTileLeaves];              // starting nodes it reaches from and to (y < 0: none built)
+  int32_t first[kTileLeaves], last[kTileLeaves], id[kTileLeaves];  // of starting node j
+  int8_t d[kTileLeaves + 1];   // common prefix across boundary j (-1: no key beyond)
+  int8_t dl[kTileLeaves + 1];  // least of d[0..j]
+  int8_t dr[kTileLeaves + 1];  // least of d[j..c]
+  uint32_t on[kTileLeaves];    // subtree from starting node j that is handed on: to << 16 | ref
+  uint32_t more[kTileLeaves];  // climbs that go on: from << 22 | to << 12 | ref (11 bits, kBuilt as bit 10)
+  int32_t wl[32], wr[32];
+  uint32_t nmore;
+};
+
+// Exclusive scan of v over the CTA's 1,024 threads; *total its sum.
+__device__ __forceinline__ int climb_scan(ClimbTile& t, int v, int* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (lane == 31) t.wl[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    int u = t.wl[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int p = __shfl_up_sync(0xffffffffu, u, o);
+      if (lane >= o) u += p;
+    }
+    t.wl[lane] = u;
+  }
+  __syncthreads();
+  const int before = (w > 0 ? t.wl[w - 1] : 0) + inc - v;
+  *total = t.wl[31];
+  __syncthreads();
+  return before;
+}
+
+// Running minima of d over the boundaries 0..c (c <= 1,024; boundary 0 apart).
+__device__ __forceinline__ void climb_minima(ClimbTile& t, int c) {
+  const int x = threadIdx.x, lane = x & 31, w = x >> 5;
+  // prefix: thread x covers boundary x; suffix: boundary x + 1
+  int a = x <= c ? t.d[x] : 127, b = x + 1 <= c ? t.d[x + 1] : 127;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, a, o), v = __shfl_down_sync(0xffffffffu, b, o);
+    if (lane >= o) a = min(a, u);
+    if (lane + o < 32) b = min(b, v);
+  }
+  if (lane == 31) t.wl[w] = a;
+  if (lane == 0) t.wr[w] = b;
+  __syncthreads();
+  if (w == 0) {
+    int u = t.wl[lane], v = t.wr[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int p = __shfl_up_sync(0xffffffffu, u, o), q = __shfl_down_sync(0xffffffffu, v, o);
+      if (lane >= o) u = min(u, p);
+      if (lane + o < 32) v = min(v, q);
+    }
+    t.wl[lane] = u;
+    t.wr[lane] = v;
+  }
+  __syncthreads();
+  if (w > 0) a = min(a, t.wl[w - 1]);
+  if (w < 31) b = min(b, t.wr[w + 1]);
+  if (x <= c) t.dl[x] = (int8_t)a;
+  if (x + 1 <= c) t.dr[x + 1] = (int8_t)b;
+  __syncthreads();
+}
+
+// Order of a thread's shared memory accesses around an exchange.  (No store to
+// global memory is in flight in the climb: the fence would wait for it.)
+__device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
+
+constexpr uint32_t kBuilt = 0x8000u;
+__device__ __forceinline__ int ref_id(const ClimbTile& t, uint32_t ref) {
+  return ref & kBuilt ? t.last[(ref & ~kBuilt) - 1] : t.id[ref];
+}
+
+// At most `steps` exchanges of the climb from the node over starting nodes
+// [a, b]; false once it has ended.
+__device__ __forceinline__ bool climb_steps(ClimbTile& t, bool top, const TreeOut& o, int steps, int& a, int& b,
+                                            uint32_t& ref) {
+  float4 bc = ref & kBuilt ? t.box[ref & ~kBuilt] : t.ibox[ref];
+  float2 sc = ref & kBuilt ? t.sum[ref & ~kBuilt] : t.isum[ref];
+  for (int k = 0; k < steps; ++k) {
+    const int dl = t.d[a], dr = t.d[b + 1];
+    if (dl < 0 && dr < 0) {
+      put_root(o, ref_id(t, ref), t.last[b] - t.first[a] + 1);
+      return false;
+    }
+    const bool toward_right = dr > dl;  // this node is the left child
+    if (!top && (toward_right ? dr == t.dr[b + 1] : dl == t.dl[a])) {
+      t.on[a] = ((uint32_t)b << 16) | ref;
+      return false;
+    }
+    const int j = toward_right ? b + 1 : a;  // the parent's boundary
+    fence_cta();                             // the summary before the exchange
+    const uint32_t old = atomicExch(&t.slot[j], ((uint32_t)(toward_right ? a : b) << 16) | ref);
+    if (old == 0xffffffffu) return false;
+    fence_cta();
+    const uint32_t sref = old & 0xffffu;
+    const float4 bs = sref & kBuilt ? t.box[sref & ~kBuilt] : t.ibox[sref];
+    const float2 ss = sref & kBuilt ? t.sum[sref & ~kBuilt] : t.isum[sref];
+    if (toward_right) b = (int)(old >> 16); else a = (int)(old >> 16);
+    sc = make_float2(__fadd_rn(sc.x, ss.x), __fadd_rn(sc.y, ss.y));
+    bc = box_union(bc, bs);
+    t.box[j] = bc;
+    t.sum[j] = sc;
+    t.child[j] = toward_right ? make_ushort2(ref, sref) : make_ushort2(sref, ref);
+    t.ends[j] = make_short2((short)a, (short)b);
+    ref = kBuilt | (uint32_t)j;
+  }
+  return true;
+}
+
+// Climbs from the tile's c starting nodes, one per thread, whose first, last,
+// id, ibox, isum and boundary prefixes are in shared memory.  ref: a node within
+// the tile, starting node j (j) or the one built at boundary j (kBuilt | j).
+// Subtrees whose parent reaches beyond the tile go to out (tile index tile);
+// out.counts == NULL: the top, where none does.  An exchange ends one climb of
+// two, so after kFirstSteps of them 1 in 15 is left: those go on side by side
+// in full warps (all in their own warps: 32 warps issue each step to the end,
+// 21 us for the leaves of 300,000 points instead of 17).
+constexpr int kFirstSteps = 3;
+__device__ void climb_tile(ClimbTile& t, int c, const TreeOut& o, Items out, int tile, float4* gbox, float2* gsum) {
+  const int x = threadIdx.x;
+  const bool top = out.counts == nullptr;
+  t.slot[x] = 0xffffffffu;
+  t.on[x] = 0xffffffffu;
+  t.ends[x] = make_short2(0, -1);
+  if (x == 0) t.nmore = 0u;
+  climb_minima(t, c);
+  int a = x, b = x;
+  uint32_t ref = (uint32_t)x;
+  if (x < c && climb_steps(t, top, o, kFirstSteps, a, b, ref))
+    t.more[atomicAdd(&t.nmore, 1u)] =
+        ((uint32_t)a << 22) | ((uint32_t)b << 12) | (ref & kBuilt ? 0x400u : 0u) | (ref & 0x3ffu);
+  __syncthreads();
+  if (x < (int)t.nmore) {
+    const uint32_t m = t.more[x];
+    a = (int)(m >> 22);
+    b = (int)((m >> 12) & 0x3ffu);
+    ref = (m & 0x3ffu) | (m & 0x400u ? kBuilt : 0u);
+    climb_steps(t, top, o, kTileLeaves, a, b, ref);  // ends: each step takes in a starting node at least
+  }
+  __syncthreads();
+  if (x < c && t.ends[x].y >= 0)
+    put_node(o, t.last[x - 1], t.first[t.ends[x].x], t.last[t.ends[x].y], ref_id(t, t.child[x].x),
+             ref_id(t, t.child[x].y), t.box[x], t.sum[x]);
+  if (top) return;
+  const uint32_t on = t.on[x];
+  const bool hand_on = on != 0xffffffffu;
+  int total;
+  const int rank = climb_scan(t, hand_on ? 1 : 0, &total);
+  if (hand_on) {
+    ref = on & 0xffffu;
+    const int id = ref_id(t, ref);
+    const float4 bc = ref & kBuilt ? t.box[ref & ~kBuilt] : t.ibox[ref];
+    const float2 sc = ref & kBuilt ? t.sum[ref & ~kBuilt] : t.isum[ref];
+    if (rank < kItemCap) {
+      const size_t at = (size_t)tile * kItemCap + rank;
+      out.at[at] = make_int4(t.first[x], t.last[on >> 16], id, 0);
+      out.box[at] = bc;
+      out.sum[at] = sc;
+    }
+    if (id >= 0) {  // where the climb through global memory looks for it
+      gbox[id] = bc;
+      gsum[id] = sc;
+    }
+  }
+  if (x == 0) out.counts[tile] = total;
+}
+
+// Prefix across the boundary after position r (-1 at the last key).
+__device__ __forceinline__ int8_t prefix_after(const uint64_t* __restrict__ keys, int r, int n) {
+  return r < n - 1 ? (int8_t)aug_prefix(keys[r], keys[r + 1], r, r + 1) : (int8_t)-1;
+}
+
+// Step 1: the leaves.
+__global__ void __launch_bounds__(kTileLeaves)
+    k_climb_leaves(int n, const uint64_t* __restrict__ keys, const float2* __restrict__ ys, TreeOut o, Items out,
+                   float4* gbox, float2* gsum) {
+  extern __shared__ __align__(16) unsigned char climb_smem[];
+  ClimbTile& t = *reinterpret_cast<ClimbTile*>(climb_smem);
+  if (__ldcg(&o.st->sort_stall)) return;
+  const int x = threadIdx.x, t0 = (int)blockIdx.x * kTileLeaves;
+  const int c = min(kTileLeaves, n - t0), k = t0 + x;
+  if (x < c) {
+    const float2 q = ys[k];
+    t.ibox[x] = make_float4(q.x, q.y, q.x, q.y);
+    t.isum[x] = q;
+    t.first[x] = t.last[x] = k;
+    t.id[x] = ~k;
+    t.d[x + 1] = prefix_after(keys, k, n);
+    if (x == 0) t.d[0] = t0 > 0 ? prefix_after(keys, t0 - 1, n) : (int8_t)-1;
+  }
+  __syncthreads();
+  climb_tile(t, c, o, out, (int)blockIdx.x, gbox, gsum);
+}
+
+// Loads the subtrees of tiles [t0, t1) of `in` (t1 - t0 <= 1,024) into a tile;
+// returns how many there are, nothing loaded above 1,024.
+__device__ int load_items(ClimbTile& t, const Items& in, int t0, int t1, int n, const uint64_t* __restrict__ keys) {
+  const int x = threadIdx.x;
+  const int mine = t0 + x < t1 ? in.counts[t0 + x] : 0;
+  int total;
+  const int before = climb_scan(t, mine, &total);
+  if (total > kTileLeaves) return total;
+  int32_t* src = reinterpret_cast<int32_t*>(t.more);  // free until the climb
+  for (int q = 0; q < mine; ++q) src[before + q] = (t0 + x) * kItemCap + q;
+  __syncthreads();
+  if (x < total) {
+    const int4 it = in.at[src[x]];
+    t.first[x] = it.x;
+    t.last[x] = it.y;
+    t.id[x] = it.z;
+    t.ibox[x] = in.box[src[x]];
+    t.isum[x] = in.sum[src[x]];
+    t.d[x + 1] = prefix_after(keys, it.y, n);
+    if (x == 0) t.d[0] = it.x > 0 ? prefix_after(keys, it.x - 1, n) : (int8_t)-1;
+  }
+  __syncthreads();
+  return total;
+}
+
+// Step 2: the subtrees of kUpTiles tiles of the launch before.
+__global__ void __launch_bounds__(kTileLeaves)
+    k_climb_items(int n, const uint64_t* __restrict__ keys, Items in, int ntiles, TreeOut o, Items out, float4* gbox,
+                  float2* gsum) {
+  extern __shared__ __align__(16) unsigned char climb_smem[];
+  ClimbTile& t = *reinterpret_cast<ClimbTile*>(climb_smem);
+  if (__ldcg(&o.st->sort_stall)) return;
+  const int t0 = (int)blockIdx.x * kUpTiles, t1 = min(ntiles, t0 + kUpTiles);
+  const int c = load_items(t, in, t0, t1, n, keys);
+  if (c > kTileLeaves) {
+    if (threadIdx.x == 0) {
+      o.st->climb_global = 1u;
+      out.counts[blockIdx.x] = 0;
+    }
+    return;
+  }
+  climb_tile(t, c, o, out, (int)blockIdx.x, gbox, gsum);
+}
+
+// Exchange at a node in global memory: acquire-release, so the summary a
+// child's thread stored before its exchange is visible to the sibling's thread
+// after its own.
 __device__ __forceinline__ unsigned long long atom_exch_acq_rel(unsigned long long* p, unsigned long long v) {
   unsigned long long old;
   asm volatile("atom.acq_rel.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
   return old;
 }
 
-__device__ __forceinline__ void mark_start(uint32_t* starts, int k) { atomicOr(starts + (k >> 5), 1u << (k & 31)); }
-
-__global__ void k_tree_climb(int n, const uint64_t* __restrict__ keys, const float2* __restrict__ ys,
-                             unsigned long long* slot, float4* box, float2* sum, float4* __restrict__ nodeA,
-                             int4* __restrict__ nodeB, uint32_t* __restrict__ starts, TreeState* st) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n || __ldcg(&st->sort_stall)) return;
-  if (n == 1) {
-    mark_start(starts, 0);
-    st->root = ~0;
-    return;
-  }
-  int L = k, R = k, id = ~k;
-  const float2 q = ys[k];
-  float4 bc = make_float4(q.x, q.y, q.x, q.y);
-  float2 sc = q;
-  uint64_t kL = keys[k], kR = kL;
-  uint64_t kLm = k > 0 ? keys[k - 1] : 0ull, kRp = k < n - 1 ? keys[k + 1] : 0ull;
+// The climb of subtree (L, R, id) through global memory to the root.
+__device__ void climb_global(int n, const uint64_t* __restrict__ keys, const float2* __restrict__ ys,
+                             unsigned long long* slot, float4* box, float2* sum, const TreeOut& o, int4 it, float4 bc,
+                             float2 sc) {
+  int L = it.x, R = it.y, id = it.z;
   for (;;) {
-    const int dl = L > 0 ? aug_prefix(kLm, kL, L - 1, L) : -1;
-    const int dr = R < n - 1 ? aug_prefix(kR, kRp, R, R + 1) : -1;
-    const bool toward_right = dr > dl;  // this node is the left child
+    const int dl = L > 0 ? prefix_after(keys, L - 1, n) : -1;
+    const int dr = prefix_after(keys, R, n);
+    if (dl < 0 && dr < 0) {
+      put_root(o, id, R - L + 1);
+      return;
+    }
+    const bool toward_right = dr > dl;
     const int p = toward_right ? R : L - 1;
-    const int bound = toward_right ? L : R;
     const unsigned long long old =
-        atom_exch_acq_rel(slot + p, ((unsigned long long)(uint32_t)bound << 32) | (uint32_t)id);
+        atom_exch_acq_rel(slot + p, ((unsigned long long)(uint32_t)(toward_right ? L : R) << 32) | (uint32_t)id);
     if (old == kSlotEmpty) return;
     slot[p] = kSlotEmpty;  // both arrivals are in: ready for the next pass
-    const int sbound = (int)(old >> 32), sid = (int)(uint32_t)old;
-    const int pL = toward_right ? L : sbound, pR = toward_right ? sbound : R;
-    // the sibling's summary and the keys at the parent's new end, at once
+    const int sid = (int)(uint32_t)old;
     float4 bs;
     float2 ss;
     if (sid < 0) {
-      const float2 t = ys[~sid];
-      bs = make_float4(t.x, t.y, t.x, t.y);
-      ss = t;
+      ss = ys[~sid];
+      bs = make_float4(ss.x, ss.y, ss.x, ss.y);
     } else {
       bs = __ldcg(box + sid);
       ss = __ldcg(sum + sid);
     }
-    if (toward_right) {
-      kR = keys[pR];
-      kRp = pR < n - 1 ? keys[pR + 1] : 0ull;
-    } else {
-      kL = keys[pL];
-      kLm = pL > 0 ? keys[pL - 1] : 0ull;
-    }
+    if (toward_right) R = (int)(old >> 32); else L = (int)(old >> 32);
     sc = make_float2(__fadd_rn(sc.x, ss.x), __fadd_rn(sc.y, ss.y));
-    bc = make_float4(fminf(bc.x, bs.x), fminf(bc.y, bs.y), fmaxf(bc.z, bs.z), fmaxf(bc.w, bs.w));
+    bc = box_union(bc, bs);
     box[p] = bc;
     sum[p] = sc;
-    const int cntp = pR - pL + 1;
-    const float cnt = (float)cntp;
-    const float r = fmaxf(__fsub_rn(bc.z, bc.x), __fsub_rn(bc.w, bc.y));
-    nodeA[p] = make_float4(__fdiv_rn(sc.x, cnt), __fdiv_rn(sc.y, cnt), __fmul_rn(r, r), cnt);
-    nodeB[p] = toward_right ? make_int4(id, sid, pL, pR) : make_int4(sid, id, pL, pR);
-    if (cntp > kGroupMax) {
-      if (p - pL + 1 <= kGroupMax) mark_start(starts, pL);  // left child [pL, p]
-      if (pR - p <= kGroupMax) mark_start(starts, p + 1);   // right child [p + 1, pR]
-    }
-    if (pL == 0 && pR == n - 1) {  // the root
-      st->root = p;
-      if (cntp <= kGroupMax) mark_start(starts, 0);
-      return;
-    }
-    L = pL;
-    R = pR;
+    put_node(o, p, L, R, toward_right ? id : sid, toward_right ? sid : id, bc, sc);
     id = p;
   }
+}
+
+// Step 3: the subtrees of all tiles of `in` by one CTA; or, if they are too
+// many or a tile of step 2 gave up, those of step 1 (leaf) by all CTAs.
+__global__ void __launch_bounds__(kTileLeaves)
+    k_climb_top(int n, const uint64_t* __restrict__ keys, const float2* __restrict__ ys, Items in, int ntiles,
+                Items leaf, int leaf_tiles, unsigned long long* slot, float4* gbox, float2* gsum, TreeOut o) {
+  extern __shared__ __align__(16) unsigned char climb_smem[];
+  ClimbTile& t = *reinterpret_cast<ClimbTile*>(climb_smem);
+  if (__ldcg(&o.st->sort_stall)) return;
+  int c = kTileLeaves + 1;
+  if (ntiles <= kTileLeaves && !__ldcg(&o.st->climb_global)) c = load_items(t, in, 0, ntiles, n, keys);
+  if (c <= kTileLeaves) {
+    if (blockIdx.x == 0 && c > 0) climb_tile(t, c, o, Items{}, 0, gbox, gsum);
+    return;
+  }
+  const int64_t entries = (int64_t)leaf_tiles * kItemCap, stride = (int64_t)gridDim.x * kTileLeaves;
+  for (int64_t e = (int64_t)blockIdx.x * kTileLeaves + threadIdx.x; e < entries; e += stride)
+    if ((int)(e % kItemCap) < leaf.counts[e / kItemCap])
+      climb_global(n, keys, ys, slot, gbox, gsum, o, leaf.at[e], leaf.box[e], leaf.sum[e]);
 }
 
 // --------------------------------------------------------------- 6. groups
@@ -778,6 +1082,17 @@ tsgne_status TreeBufs::alloc(int n_points, int sm_count, cudaStream_t s) {
   TS_TRY(box.alloc(nn));
   TS_TRY(sum.alloc(nn));
   TS_TRY(slot.alloc(nn));
+  size_t tiles = ((size_t)n + kTileLeaves - 1) / kTileLeaves;
+  for (int k = 0; k < 3; ++k, tiles = (tiles + kUpTiles - 1) / kUpTiles) {
+    TS_TRY(item_at[k].alloc(tiles * kItemCap));
+    TS_TRY(item_box[k].alloc(tiles * kItemCap));
+    TS_TRY(item_sum[k].alloc(tiles * kItemCap));
+    TS_TRY(item_count[k].alloc(tiles));
+  }
+  climb_blocks = sm_count;
+  TS_CUDA(cudaFuncSetAttribute(k_climb_leaves, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
+  TS_CUDA(cudaFuncSetAttribute(k_climb_items, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
+  TS_CUDA(cudaFuncSetAttribute(k_climb_top, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
   TS_TRY(boxpart.alloc((size_t)box_blocks));
   TS_TRY(state.alloc(1));
   TS_CUDA(cudaMemsetAsync(slot.get(), 0xff, sizeof(unsigned long long) * nn, s));  // every slot empty
@@ -806,9 +1121,27 @@ tsgne_status launch_tree_build(TreeBufs& tb, const float2* Y, cudaStream_t s) {
   }
   // an even number of passes: sorted keys / permutation are back in slot 0
   static_assert(kRadixPasses % 2 == 0, "sorted keys end in slot 0");
-  k_tree_climb<<<grid_for(n, 256, 1 << 30), 256, 0, s>>>(n, tb.keys[0].get(), tb.ys.get(), tb.slot.get(),
-                                                         tb.box.get(), tb.sum.get(), tb.nodeA.get(), tb.nodeB.get(),
-                                                         tb.starts.get(), st);
+  const TreeOut o{tb.nodeA.get(), tb.nodeB.get(), tb.starts.get(), st};
+  const size_t smem = sizeof(ClimbTile);
+  const int leaf_tiles = (n + kTileLeaves - 1) / kTileLeaves;
+  auto items = [&](int k) {
+    return Items{tb.item_at[k].get(), tb.item_box[k].get(), tb.item_sum[k].get(), tb.item_count[k].get()};
+  };
+  k_climb_leaves<<<leaf_tiles, kTileLeaves, smem, s>>>(n, tb.keys[0].get(), tb.ys.get(), o, items(0), tb.box.get(),
+                                                       tb.sum.get());
+  int tiles = leaf_tiles, at = 0;
+  while (tiles > kUpTiles) {
+    const int up = (tiles + kUpTiles - 1) / kUpTiles, to = at == 1 ? 2 : 1;
+    k_climb_items<<<up, kTileLeaves, smem, s>>>(n, tb.keys[0].get(), items(at), tiles, o, items(to), tb.box.get(),
+                                                tb.sum.get());
+    tiles = up;
+    at = to;
+  }
+  if (tiles > 1)
+    k_climb_top<<<tb.climb_blocks, kTileLeaves, smem, s>>>(n, tb.keys[0].get(), tb.ys.get(), items(at), tiles,
+                                                          items(0), leaf_tiles, tb.slot.get(), tb.box.get(),
+                                                          tb.sum.get(), o);
+  TS_CUDA(cudaGetLastError());
   k_tree_groups<<<grid_for((n + 31) / 32, 256, 1 << 30), 256, 0, s>>>(n, st, tb.starts.get(), tb.groups.get());
   TS_CUDA(cudaGetLastError());
   return TSGNE_OK;

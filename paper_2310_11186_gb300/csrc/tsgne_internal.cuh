@@ -480,12 +480,13 @@ struct TreeState {
   int32_t root;                  // root of the last tree: an internal node id, or ~0 (one point)
   uint32_t groups;               // groups of the last tree
   uint32_t zbad;                 // 1: a group's Z was NaN
+  uint32_t climb_global;         // 1: a tile of the tree's second step held too many subtrees
   unsigned long long zsum[2];    // Z of the walk: fractions of 2^-32 and whole units, summed apart
 };
 
 // Device buffers of the tree code for n points.
 struct TreeBufs {
-  int n = 0, ntiles = 0, box_blocks = 0, keys_blocks = 0, walk_blocks = 0;
+  int n = 0, ntiles = 0, box_blocks = 0, keys_blocks = 0, walk_blocks = 0, climb_blocks = 0;
   long long spin_budget = 2000000000LL;  // clock cycles a look-back wait of the sort may last
   DevBuf<uint64_t> keys[2];
   DevBuf<int32_t> vals[2];    // vals[0] after a build: sorted position -> point
@@ -496,6 +497,10 @@ struct TreeBufs {
   DevBuf<float4> box;         // internal node: x0, y0, x1, y1
   DevBuf<float2> sum;         // internal node: coordinate sums
   DevBuf<unsigned long long> slot;  // bottom-up exchange slots (kept empty, all ones, between passes)
+  DevBuf<int4> item_at[3];    // subtrees that the tree's tiles hand on: range and id, box, sums, count per tile
+  DevBuf<float4> item_box[3];
+  DevBuf<float2> item_sum[3];
+  DevBuf<int32_t> item_count[3];
   DevBuf<float4> boxpart;
   DevBuf<uint32_t> starts;    // bit k: a group begins at sorted position k
   DevBuf<int2> groups;        // first sorted position and end of each group, in any order
