@@ -28,8 +28,8 @@
 //
 // GPU mapping.  Keys: one thread per point, which also counts the digits of
 // all eight sort passes.  Sort: LSD radix sort, 8 stable passes of 8 bits,
-// one launch each: a CTA ranks a tile of 2048 keys (__match_any_sync within
-// warps, offsets across warps) and takes the tile's global offsets from the
+// one launch each: a CTA ranks a tile of 2048 keys (ballots within warps,
+// offsets across warps) and takes the tile's global offsets from the
 // tiles before it by a decoupled look-back (a bounded wait).  The last pass
 // also gathers the layout into sorted order.  Tree, summaries and group
 // starts: bottom up in shared memory, tile by tile, one thread per leaf climbing
@@ -54,11 +54,7 @@ namespace {
 
 constexpr int kRadixPasses = 8;  // 8-bit digits of the 64-bit keys
 constexpr int kRadixBins = 256;
-constexpr int kSortWarps = 8;
-constexpr int kSortThreads = 32 * kSortWarps;        // one thread per digit in the look-back
-constexpr int kSortItems = 8;                        // keys per lane
-constexpr int kSortTile = kSortThreads * kSortItems;  // keys per tile (per CTA)
-static_assert(kSortThreads == kRadixBins, "the look-back maps one thread to one digit");
+constexpr int kSortTile = 2048;  // keys per tile (per CTA)
 constexpr int kWalkWarps = 8;
 
 __device__ __forceinline__ float warp_min(float v) {
@@ -195,11 +191,13 @@ __global__ void __launch_bounds__(kKeyThreads) k_tree_keys(const float2* __restr
 //
 // A CTA takes tiles in launch order from a counter (ctl[pass]), so it only
 // ever waits on tiles that running CTAs own.  Tile t covers keys
-// [t T, t T + T), T = kSortTile; warp w holds keys w 256 + 32 r + lane,
-// r < 8, so (w, r, lane) order is input order.
-//  1. ranks within the warp: per round of 32 keys __match_any_sync groups
-//     equal digits; rank = running count of the digit in the warp + the
-//     number of lower lanes with the same digit;
+// [t T, t T + T), T = kSortTile; warp w holds K = T / (32 kWarps) rounds of 32
+// keys, w 32 K + 32 r + lane, r < K, so (w, r, lane) order is input order.
+//  1. ranks within the warp: per round of 32 keys eight ballots, one per bit of
+//     the digit, group equal digits (__match_any_sync takes longer for 32
+//     digits that mostly differ: an iteration of 2,097,152 points 1466 us, 1439
+//     with ballots); rank = running count of the digit in the warp + the number
+//     of lower lanes with the same digit;
 //  2. per digit d (thread d): the warps' exclusive offsets and the tile's
 //     count c_d, published at once as status[pass][t][d] = (AGG, c_d)
 //     (tile 0: (INCL, c_d));
@@ -230,7 +228,7 @@ __device__ __forceinline__ void st_relaxed_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Exclusive scans over the 256 threads of a CTA of two values at once
+// Exclusive scans over the threads of a CTA of two values at once
 // (thread x gets the sums over threads < x).
 __device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_t& ea, uint32_t& eb,
                                                  uint2* wsum) {
@@ -255,44 +253,56 @@ __device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_
   eb = ob + ib - b;
 }
 
-__global__ void __launch_bounds__(kSortThreads)
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps)
     k_radix_onesweep(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, int n, int pass,
                      const uint32_t* __restrict__ ghist, uint32_t* ctl, uint32_t* status, int ntiles,
                      long long budget, TreeState* st, uint64_t* __restrict__ kout, int32_t* __restrict__ vout,
                      const float2* __restrict__ Y, float2* __restrict__ ys) {
-  __shared__ uint32_t hw[kSortWarps][kRadixBins];
+  constexpr int kThreads = 32 * kWarps, kItems = kSortTile / kThreads;  // keys per lane
+  static_assert(kThreads >= kRadixBins, "the look-back maps one thread to one digit");
+  __shared__ uint32_t hw[kWarps][kRadixBins];
   __shared__ uint64_t skey[kSortTile];
   __shared__ int32_t sval[kSortTile];
   __shared__ uint32_t lstart[kRadixBins], gbase[kRadixBins];
-  __shared__ uint2 wsum[kSortWarps];
+  __shared__ uint2 wsum[kWarps];
   __shared__ int tile_s;
-  if (__ldcg(&st->sort_stall)) return;  // an earlier pass gave up: nothing of this build is valid
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   if (tid == 0) tile_s = (int)atomicAdd(ctl + pass, 1u);
-  for (int k = tid; k < kSortWarps * kRadixBins; k += kSortThreads) (&hw[0][0])[k] = 0u;
+  for (int k = tid; k < kWarps * kRadixBins; k += kThreads) (&hw[0][0])[k] = 0u;
+  // up to here beside the end of the pass before (its CTAs release this launch
+  // after their own wait, so everything older is complete)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
+  if (__ldcg(&st->sort_stall)) return;  // an earlier pass gave up: nothing of this build is valid
   const int t = tile_s;
   if (t >= ntiles) return;  // uniform: more CTAs than tiles never happens, kept as a guard
   const int64_t t0 = (int64_t)t * kSortTile;
   const int tn = (int)min((int64_t)kSortTile, (int64_t)n - t0);
   const int shift = 8 * pass;
   const uint32_t lt = (1u << lane) - 1u;
-  const int wb = w * (32 * kSortItems) + lane;
-  uint64_t key[kSortItems];
-  int32_t val[kSortItems];
-  uint32_t rk[kSortItems];
+  const int wb = w * (32 * kItems) + lane;
+  uint64_t key[kItems];
+  int32_t val[kItems];
+  uint32_t rk[kItems];
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {  // all loads of the tile in flight at once
+  for (int r = 0; r < kItems; ++r) {  // all loads of the tile in flight at once
     const int i = wb + 32 * r;
     key[r] = i < tn ? kin[t0 + i] : 0ull;
     val[r] = i < tn ? vin[t0 + i] : 0;
   }
   // 1. ranks within the warp
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r) {
+  for (int r = 0; r < kItems; ++r) {
     const bool valid = wb + 32 * r < tn;
-    const uint32_t d = valid ? (uint32_t)(key[r] >> shift) & 255u : 256u + (uint32_t)lane;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+    uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool one = (d >> q) & 1u;
+      const uint32_t ones = __ballot_sync(0xffffffffu, one);
+      peers &= one ? ones : ~ones;
+    }
     const uint32_t before = valid ? hw[w][d] : 0u;
     rk[r] = before + (uint32_t)__popc(peers & lt);
     __syncwarp();
@@ -302,20 +312,23 @@ __global__ void __launch_bounds__(kSortThreads)
   __syncthreads();
   // 2. per digit: offsets of the warps, count of the tile, published
   const int d = tid;
+  const bool digit = kThreads == kRadixBins || d < kRadixBins;
   uint32_t cnt = 0u;
+  if (digit) {
 #pragma unroll
-  for (int v = 0; v < kSortWarps; ++v) {
-    const uint32_t x = hw[v][d];
-    hw[v][d] = cnt;
-    cnt += x;
+    for (int v = 0; v < kWarps; ++v) {
+      const uint32_t x = hw[v][d];
+      hw[v][d] = cnt;
+      cnt += x;
+    }
   }
   uint32_t* const sbase = status + (size_t)pass * ntiles * kRadixBins;
-  st_relaxed_u32(sbase + (size_t)t * kRadixBins + d, (t == 0 ? kStIncl : kStAgg) | cnt);
+  if (digit) st_relaxed_u32(sbase + (size_t)t * kRadixBins + d, (t == 0 ? kStIncl : kStAgg) | cnt);
   uint32_t dstart, lst;
-  block_excl_scan2(__ldg(ghist + pass * kRadixBins + d), cnt, dstart, lst, wsum);
+  block_excl_scan2(digit ? __ldg(ghist + pass * kRadixBins + d) : 0u, cnt, dstart, lst, wsum);
   // 3. look-back
   uint32_t excl = 0u;
-  if (t > 0) {
+  if (t > 0 && digit) {
     const long long c0 = clock64();
     bool stalled = false, done = false;
     // windows of kLookWindow predecessors, loaded at once, read nearest first
@@ -345,12 +358,15 @@ __global__ void __launch_bounds__(kSortThreads)
     if (stalled) atomicExch(&st->sort_stall, 1u);
     st_relaxed_u32(sbase + (size_t)t * kRadixBins + d, kStIncl | ((excl + cnt) & kStCount));
   }
-  gbase[d] = dstart + excl;
-  lstart[d] = lst;
+  if (digit) {
+    gbase[d] = dstart + excl;
+    lstart[d] = lst;
+  }
   __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;");  // the next pass may set up beside the writes
   // 4. stage in (digit, input) order, then write out
 #pragma unroll
-  for (int r = 0; r < kSortItems; ++r)
+  for (int r = 0; r < kItems; ++r)
     if (wb + 32 * r < tn) {
       const uint32_t dg = (uint32_t)(key[r] >> shift) & 255u;
       const uint32_t lp = lstart[dg] + hw[w][dg] + rk[r];
@@ -358,7 +374,7 @@ __global__ void __launch_bounds__(kSortThreads)
       sval[lp] = val[r];
     }
   __syncthreads();
-  for (int i = tid; i < tn; i += kSortThreads) {
+  for (int i = tid; i < tn; i += kThreads) {
     const uint64_t kk = skey[i];
     const uint32_t dg = (uint32_t)(kk >> shift) & 255u;
     const uint32_t pos = gbase[dg] + ((uint32_t)i - lstart[dg]);
@@ -1089,7 +1105,7 @@ tsgne_status TreeBufs::alloc(int n_points, int sm_count, cudaStream_t s) {
     TS_TRY(item_sum[k].alloc(tiles * kItemCap));
     TS_TRY(item_count[k].alloc(tiles));
   }
-  climb_blocks = sm_count;
+  this->sm_count = sm_count;
   TS_CUDA(cudaFuncSetAttribute(k_climb_leaves, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
   TS_CUDA(cudaFuncSetAttribute(k_climb_items, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
   TS_CUDA(cudaFuncSetAttribute(k_climb_top, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClimbTile)));
@@ -1110,14 +1126,37 @@ tsgne_status launch_tree_build(TreeBufs& tb, const float2* Y, cudaStream_t s) {
                                            tb.starts.get());
   k_tree_keys<<<tb.keys_blocks, kKeyThreads, 0, s>>>(Y, n, st, tb.keys[0].get(), tb.vals[0].get(), ghist);
   TS_CUDA(cudaGetLastError());
+  // 16 warps of 4 keys a lane while every SM has at most one tile: a tile is a
+  // serial chain, shorter with fewer keys a lane (an iteration at 300,000 points,
+  // 147 tiles: 291 us with 8 warps, 281 with 16).  With more tiles the SMs are
+  // full and half the counts in shared memory are cheaper (2,097,152 points: 1439
+  // us with 8 warps, 1476 with 16).
+  // A pass may set up beside the end of the one before.  Its CTAs are then
+  // placed among those still running, unevenly, which costs more than the
+  // set-up where the tiles fill the SMs almost exactly once or twice
+  // (us per iteration without / with it: 98 tiles 228 / 226, 147 tiles 280 /
+  // 291, 293 tiles 480 / 494, 489 tiles 740.6 / 739.3; launched one by one
+  // the eight passes gain 10 to 23 us outside that range).
+  const int sms = tb.sm_count;
+  const bool one_wave = tb.ntiles <= sms, beside = 3 * tb.ntiles <= 2 * sms || tb.ntiles >= 3 * sms;
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)tb.ntiles);
+  cfg.blockDim = dim3(one_wave ? 512u : 256u);
+  cfg.stream = s;
+  cfg.attrs = &early;
+  cfg.numAttrs = 0;  // the first pass waits for the keys as usual
   for (int pass = 0; pass < kRadixPasses; ++pass) {
     const int in = pass & 1, out = in ^ 1;
     const bool last = pass == kRadixPasses - 1;
-    k_radix_onesweep<<<tb.ntiles, kSortThreads, 0, s>>>(tb.keys[in].get(), tb.vals[in].get(), n, pass, ghist, ctl,
-                                                        status, tb.ntiles, tb.spin_budget, st, tb.keys[out].get(),
-                                                        tb.vals[out].get(), last ? Y : nullptr,
-                                                        last ? tb.ys.get() : nullptr);
-    TS_CUDA(cudaGetLastError());
+    TS_CUDA(cudaLaunchKernelEx(&cfg, one_wave ? k_radix_onesweep<16> : k_radix_onesweep<8>,
+                               (const uint64_t*)tb.keys[in].get(), (const int32_t*)tb.vals[in].get(), n, pass,
+                               (const uint32_t*)ghist, ctl, status, tb.ntiles, (long long)tb.spin_budget, st,
+                               tb.keys[out].get(), tb.vals[out].get(), last ? Y : (const float2*)nullptr,
+                               last ? tb.ys.get() : (float2*)nullptr));
+    if (beside) cfg.numAttrs = 1;
   }
   // an even number of passes: sorted keys / permutation are back in slot 0
   static_assert(kRadixPasses % 2 == 0, "sorted keys end in slot 0");
@@ -1138,7 +1177,7 @@ tsgne_status launch_tree_build(TreeBufs& tb, const float2* Y, cudaStream_t s) {
     at = to;
   }
   if (tiles > 1)
-    k_climb_top<<<tb.climb_blocks, kTileLeaves, smem, s>>>(n, tb.keys[0].get(), tb.ys.get(), items(at), tiles,
+    k_climb_top<<<tb.sm_count, kTileLeaves, smem, s>>>(n, tb.keys[0].get(), tb.ys.get(), items(at), tiles,
                                                           items(0), leaf_tiles, tb.slot.get(), tb.box.get(),
                                                           tb.sum.get(), o);
   TS_CUDA(cudaGetLastError());

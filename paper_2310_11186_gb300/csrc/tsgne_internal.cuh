@@ -486,7 +486,7 @@ struct TreeState {
 
 // Device buffers of the tree code for n points.
 struct TreeBufs {
-  int n = 0, ntiles = 0, box_blocks = 0, keys_blocks = 0, walk_blocks = 0, climb_blocks = 0;
+  int n = 0, ntiles = 0, box_blocks = 0, keys_blocks = 0, walk_blocks = 0, sm_count = 0;
   long long spin_budget = 2000000000LL;  // clock cycles a look-back wait of the sort may last
   DevBuf<uint64_t> keys[2];
   DevBuf<int32_t> vals[2];    // vals[0] after a build: sorted position -> point
