@@ -18,11 +18,11 @@
 // sums are FP64 with _rn intrinsics, so the choices are those of the CPU
 // reference up to the last-ulp behaviour of exp().
 //
-// Kernels: squared distances (walk_distances, affinity.cu: 0.76 ms for 1.0M
-// pairs of 64 dimensions; a warp per row, most lanes idle, took 5.7), per-row running
-// weight sums (thread per row, sequential like the definition), one thread
-// per walk, then one warp per node sorts its R end points in shared memory
-// and keeps the distinct ones with their counts.
+// Kernels: squared distances (walk_distances, affinity.cu: 0.49 ms for 1.0M
+// pairs of 64 dimensions; a warp per row, most lanes idle, took 5.7), per-row
+// running weight sums (thread per row, sequential like the definition), one
+// thread per walk, then one warp per node sorts its R end points and keeps the
+// distinct ones with their counts.
 #include <cmath>
 
 #include "tsgne_internal.cuh"
@@ -54,30 +54,131 @@ __global__ void k_rw_cumw(int n, const int64_t* __restrict__ rp, const double* _
   }
 }
 
+// (double)(m * 2^-53), m < 2^53, by integer operations (exact).
+__device__ __forceinline__ double unit_uniform(uint64_t m) {
+  if (m == 0ull) return 0.0;
+  const int up = __clzll((long long)m) - 11;  // brings the top bit to bit 52
+  return __longlong_as_double((long long)(((uint64_t)(1021 - up) << 52) + (m << up)));
+}
+
+// One thread per walk.  A step is one FP64 product: the uniform is put
+// together from bits, and running sums, which are not negative, compare as the
+// integers of their bits (FP64 conversions and comparisons occupy the SM's FP64
+// pipe 16 cycles per warp: 7 of them bounded the kernel).  A row whose sums are
+// NaN (infinite features) compares false throughout: its last entry.  Rows of up
+// to 8 entries are counted through with all loads in flight, longer ones are
+// first cut to that a quarter at a time.  300,000 nodes, 64 walks of 3 steps:
+// 647 us before, 361 us now.
 __global__ void k_rw_walks(int n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                            const double* __restrict__ cw, int R, int L, uint64_t s0, int32_t* __restrict__ ends) {
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= (int64_t)n * R) return;
-  const int64_t i = w / R;
+  const int64_t i = (int64_t)n * R <= 0xffffffffll ? (int64_t)((uint32_t)w / (uint32_t)R) : w / R;
+  const long long* __restrict__ cwb = reinterpret_cast<const long long*>(cw);
   int32_t u = (int32_t)i;
   for (int s = 0; s < L; ++s) {
     const uint64_t k = 1ull + (uint64_t)w * (uint64_t)L + (uint64_t)s;
-    const double U = (double)(sm64_output(s0, k) >> 11) * (1.0 / 9007199254740992.0);
     const int64_t a = rp[u], b = rp[u + 1];
     if (a == b) continue;
-    const double target = __dmul_rn(U, cw[b - 1]);
-    int64_t lo = a, hi = b - 1;  // first e with cw[e] > target; the last entry if none
-    while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (cw[mid] > target) hi = mid; else lo = mid + 1;
+    const long long total = cwb[b - 1];
+    const long long target = __double_as_longlong(
+        __dmul_rn(unit_uniform(sm64_output(s0, k) >> 11), __longlong_as_double(total)));
+    const bool nan = (total & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+    int64_t lo = nan ? b - 1 : a, hi = b - 1;  // first e with cw[e] > target; the last entry if none
+    while (hi - lo > 7) {
+      const int64_t q = (hi - lo) >> 2, m1 = lo + q, m2 = m1 + q, m3 = m2 + q;
+      const long long c1 = cwb[m1], c2 = cwb[m2], c3 = cwb[m3];
+      if (c2 > target) {
+        hi = c1 > target ? m1 : m2;
+        if (c1 <= target) lo = m1 + 1;
+      } else {
+        lo = c3 > target ? m2 + 1 : m3 + 1;
+        if (c3 > target) hi = m3;
+      }
     }
-    u = col[lo];
+    int below = 0;
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+      if (lo + q < hi) below += cwb[lo + q] <= target ? 1 : 0;
+    u = col[lo + below];
   }
   ends[w] = u == (int32_t)i ? -1 : u;
 }
 
-// Warp per node: its R end points sorted (rank by counting), distinct
-// values kept with their multiplicities; -1 (returned walks) dropped.
+// Distinct values >= 0 of srt[0, R) (ascending) with their multiplicities, by
+// one warp: their first positions are listed in at, so that a multiplicity is a
+// difference.
+__device__ __forceinline__ int list_distinct(const int32_t* srt, int32_t* at, int R, int32_t* __restrict__ ucol,
+                                             int32_t* __restrict__ ucnt) {
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  for (int t0 = 0; t0 < R; t0 += 32) {
+    const int t = t0 + lane;
+    const bool head = t < R && srt[t] >= 0 && (t == 0 || srt[t - 1] != srt[t]);
+    const uint32_t hm = __ballot_sync(0xffffffffu, head);
+    if (head) at[base + __popc(hm & ((1u << lane) - 1u))] = t;
+    base += __popc(hm);
+  }
+  __syncwarp();
+  for (int k = lane; k < base; k += 32) {
+    const int t = at[k];
+    ucol[k] = srt[t];
+    ucnt[k] = (k + 1 < base ? at[k + 1] : R) - t;
+  }
+  return base;
+}
+
+// Warp per node, R <= 32 K: its end points sorted in registers by a bitonic
+// network (element t = 32 q + lane), distinct values kept with their
+// multiplicities; -1 (returned walks) dropped.  Ranks by counting (the kernel
+// below) are R^2 comparisons: 300,000 nodes, R = 64: 390 us, 89 us here.
+template <int K>
+__global__ void __launch_bounds__(32 * kRwWarps)
+    k_rw_count_sorted(int n, int R, const int32_t* __restrict__ ends, int32_t* __restrict__ ucol,
+                      int32_t* __restrict__ ucnt, int32_t* __restrict__ nuniq) {
+  __shared__ int32_t sh[kRwWarps][2][32 * K];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t *at = sh[wid][0], *srt = sh[wid][1];
+  const int64_t warps = (int64_t)gridDim.x * kRwWarps;
+  for (int64_t i = (int64_t)blockIdx.x * kRwWarps + wid; i < n; i += warps) {
+    int32_t v[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) v[q] = 32 * q + lane < R ? ends[i * R + 32 * q + lane] : 0x7fffffff;
+#pragma unroll
+    for (int size = 2; size <= 32 * K; size <<= 1) {
+#pragma unroll
+      for (int step = size >> 1; step > 0; step >>= 1) {
+        if (step >= 32) {
+#pragma unroll
+          for (int q = 0; q < K; ++q) {
+            const int o = q ^ (step >> 5);
+            if (o > q) {
+              const bool up = ((32 * q) & size) == 0;
+              const int32_t lo = min(v[q], v[o]), hi = max(v[q], v[o]);
+              v[q] = up ? lo : hi;
+              v[o] = up ? hi : lo;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < K; ++q) {
+            const int32_t o = __shfl_xor_sync(0xffffffffu, v[q], step);
+            const bool up = ((32 * q + lane) & size) == 0, first = (lane & step) == 0;
+            v[q] = up == first ? min(v[q], o) : max(v[q], o);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) srt[32 * q + lane] = v[q];
+    __syncwarp();
+    const int base = list_distinct(srt, at, R, ucol + i * R, ucnt + i * R);
+    if (lane == 0) nuniq[i] = base;
+    __syncwarp();
+  }
+}
+
+// The same for any R (above 256 here), sorted in shared memory by rank.
 __global__ void __launch_bounds__(32 * kRwWarps)
     k_rw_count(int n, int R, const int32_t* __restrict__ ends, int32_t* __restrict__ ucol,
                int32_t* __restrict__ ucnt, int32_t* __restrict__ nuniq) {
@@ -99,20 +200,7 @@ __global__ void __launch_bounds__(32 * kRwWarps)
       srt[rank] = x;
     }
     __syncwarp();
-    int base = 0;
-    for (int t0 = 0; t0 < R; t0 += 32) {
-      const int t = t0 + lane;
-      const bool head = t < R && srt[t] >= 0 && (t == 0 || srt[t - 1] != srt[t]);
-      const uint32_t hm = __ballot_sync(0xffffffffu, head);
-      if (head) {
-        int e = t + 1;
-        while (e < R && srt[e] == srt[t]) ++e;
-        const int slot = base + __popc(hm & ((1u << lane) - 1u));
-        ucol[i * R + slot] = srt[t];
-        ucnt[i * R + slot] = e - t;
-      }
-      base += __popc(hm);
-    }
+    const int base = list_distinct(srt, v, R, ucol + i * R, ucnt + i * R);
     if (lane == 0) nuniq[i] = base;
     __syncwarp();
   }
@@ -186,9 +274,15 @@ tsgne_status random_walk_affinities(int n, const int64_t* rp, const int32_t* col
   TS_TRY(nuniq.alloc((size_t)n));
   k_rw_walks<<<grid_cap(walks, 256, 1 << 30), 256, 0, s>>>(n, rp, col, cw.get(), R, L,
                                                            seed ^ 0xD1B54A32D192ED03ull, ends.get());
-  const size_t smem = (size_t)kRwWarps * 2 * R * sizeof(int32_t);
-  TS_CUDA(cudaFuncSetAttribute(k_rw_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_rw_count<<<wgrid, 32 * kRwWarps, smem, s>>>(n, R, ends.get(), ucol.get(), ucnt.get(), nuniq.get());
+  if (R <= 256) {
+    const auto count = R <= 32 ? k_rw_count_sorted<1> : R <= 64 ? k_rw_count_sorted<2>
+                     : R <= 128 ? k_rw_count_sorted<4> : k_rw_count_sorted<8>;
+    count<<<wgrid, 32 * kRwWarps, 0, s>>>(n, R, ends.get(), ucol.get(), ucnt.get(), nuniq.get());
+  } else {
+    const size_t smem = (size_t)kRwWarps * 2 * R * sizeof(int32_t);
+    TS_CUDA(cudaFuncSetAttribute(k_rw_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_rw_count<<<wgrid, 32 * kRwWarps, smem, s>>>(n, R, ends.get(), ucol.get(), ucnt.get(), nuniq.get());
+  }
   TS_CUDA(cudaGetLastError());
   ends.reset();
   cw.reset();
