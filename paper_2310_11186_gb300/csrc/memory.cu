@@ -18,11 +18,12 @@
 // and with every object destroyed.  All idle blocks go back to the device when
 // an allocation fails and when the library's memory limit is set.  Blocks
 // belong to one CUDA context (recognised by its id): what a context destroyed
-// by cudaDeviceReset held is forgotten.
+// by cudaDeviceReset held is forgotten.  A buffer carries its block's size,
+// device and context itself, so it goes back where it came from whatever the
+// freeing thread has selected, and nothing about it is kept here meanwhile.
 #include <atomic>
 #include <list>
 #include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "tsgne_internal.cuh"
@@ -43,9 +44,9 @@ struct Block {
 };
 struct Blocks {
   unsigned long long context = 0;
+  int device = 0;
   std::list<Block> idle;  // longest idle first
   size_t idle_bytes = 0;
-  std::unordered_map<void*, size_t> lent;  // sizes of the blocks in use
   std::vector<cudaEvent_t> spare;
 };
 std::mutex g_mu;
@@ -70,11 +71,30 @@ bool context_id(unsigned long long* id) {
   return fn != nullptr && fn(nullptr, id) == 0;
 }
 
-Blocks& blocks_of(unsigned long long id) {
+// Selects a device with its context current, and the caller's device again at the end.
+struct OnDevice {
+  int prev = -1;
+  unsigned long long context = 0;  // the current context; ok: there is one
+  bool ok;
+  explicit OnDevice(int device) {
+    if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
+    ok = prev == device && context_id(&context);  // a new thread has no context until it selects its device
+    if (!ok) ok = cudaSetDevice(device) == cudaSuccess && context_id(&context);
+    if (prev == device) prev = -1;
+  }
+  ~OnDevice() {
+    if (prev >= 0) cudaSetDevice(prev);
+  }
+  OnDevice(const OnDevice&) = delete;
+  OnDevice& operator=(const OnDevice&) = delete;
+};
+
+Blocks& blocks_of(unsigned long long id, int device) {
   for (Blocks& b : all_blocks())
     if (b.context == id) return b;
   all_blocks().emplace_back();
   all_blocks().back().context = id;
+  all_blocks().back().device = device;
   return all_blocks().back();
 }
 
@@ -97,51 +117,41 @@ void shrink(Blocks& b, size_t keep) {
   }
 }
 
-cudaError_t take(void** p, size_t bytes, cudaStream_t s, unsigned long long id) {
+cudaError_t take(DevMem* m, size_t bytes) {
   std::lock_guard<std::mutex> lk(g_mu);
-  Blocks& b = blocks_of(id);
+  Blocks& b = blocks_of(m->context, m->device);
   const size_t want = block_size(bytes);
   auto best = b.idle.end();
   for (auto it = b.idle.begin(); it != b.idle.end(); ++it)  // at most twice the size asked for
     if (it->bytes >= want && it->bytes <= 2 * want && (best == b.idle.end() || it->bytes < best->bytes)) best = it;
   if (best != b.idle.end()) {
     const Block k = *best;
-    if (cudaStreamWaitEvent(s, k.done, 0) == cudaSuccess) {
-      b.lent.emplace(k.p, k.bytes);
+    b.spare.reserve(b.spare.size() + 1);  // before anything changes
+    if (cudaStreamWaitEvent(m->stream, k.done, 0) == cudaSuccess) {
       b.idle.erase(best);
       b.idle_bytes -= k.bytes;
       b.spare.push_back(k.done);
-      *p = k.p;
+      m->p = k.p;
+      m->bytes = k.bytes;
       return cudaSuccess;
     }
     cudaGetLastError();
   }
-  cudaError_t e = cudaMalloc(p, want);
+  cudaError_t e = cudaMalloc(&m->p, want);
   if (e == cudaErrorMemoryAllocation && b.idle_bytes > 0) {
     cudaGetLastError();
     shrink(b, 0);
-    e = cudaMalloc(p, want);
+    e = cudaMalloc(&m->p, want);
   }
-  if (e == cudaSuccess) {
-    try {
-      b.lent.emplace(*p, want);
-    } catch (...) {
-      cudaFree(*p);
-      throw;
-    }
-  }
+  m->bytes = want;
   return e;
 }
 
 // False if the block has to be freed by the caller.
-bool give_back(void* p, cudaStream_t s, unsigned long long id) {
+bool give_back(const DevMem& m) {
+  if (m.bytes > kIdleBytes) return false;
   std::lock_guard<std::mutex> lk(g_mu);
-  Blocks& b = blocks_of(id);
-  const auto it = b.lent.find(p);
-  if (it == b.lent.end()) return false;
-  const size_t bytes = it->second;
-  b.lent.erase(it);
-  if (bytes > kIdleBytes) return false;
+  Blocks& b = blocks_of(m.context, m.device);
   cudaEvent_t ev = nullptr;
   if (!b.spare.empty()) {
     ev = b.spare.back();
@@ -150,22 +160,30 @@ bool give_back(void* p, cudaStream_t s, unsigned long long id) {
     cudaGetLastError();
     return false;
   }
-  if (cudaEventRecord(ev, s) != cudaSuccess) {
+  if (cudaEventRecord(ev, m.stream) != cudaSuccess) {
     cudaGetLastError();
     b.spare.push_back(ev);
     return false;
   }
-  b.idle.push_back(Block{p, bytes, ev});
-  b.idle_bytes += bytes;
+  b.idle.push_back(Block{m.p, m.bytes, ev});
+  b.idle_bytes += m.bytes;
   return true;
 }
 
+// Every context's idle blocks; a context that is no longer its device's is forgotten.
 void trim_to(size_t keep) {
-  unsigned long long id = 0;
-  if (!context_id(&id)) return;
   std::lock_guard<std::mutex> lk(g_mu);
-  for (Blocks& b : all_blocks())
-    if (b.context == id) shrink(b, keep);
+  for (auto b = all_blocks().begin(); b != all_blocks().end();) {
+    if (b->idle_bytes > keep) {
+      OnDevice on(b->device);
+      if (!on.ok || on.context != b->context) {
+        b = all_blocks().erase(b);
+        continue;
+      }
+      shrink(*b, keep);
+    }
+    ++b;
+  }
 }
 
 }  // namespace
@@ -187,29 +205,28 @@ bool device_bytes_reserve(size_t bytes) {
 
 void device_bytes_release(size_t bytes) { g_dev_bytes.fetch_sub((int64_t)bytes); }
 
-cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t* owner) {
+cudaError_t device_alloc(DevMem* m, size_t bytes) {
+  *m = DevMem{};
   const cudaStream_t s = alloc_stream();
-  unsigned long long id = 0;
-  *owner = nullptr;
-  if (!s || !context_id(&id)) return cudaMalloc(p, bytes);
+  if (!s || cudaGetDevice(&m->device) != cudaSuccess || !context_id(&m->context)) return cudaMalloc(&m->p, bytes);
+  m->stream = s;
   try {
-    const cudaError_t e = take(p, bytes, s, id);
-    if (e == cudaSuccess) *owner = s;
-    return e;
+    return take(m, bytes);
   } catch (const std::bad_alloc&) {  // no host memory for the list: CUDA's own answer decides
-    return cudaMalloc(p, bytes);
+    m->stream = nullptr;
+    return cudaMalloc(&m->p, bytes);
   }
 }
 
-void device_free(void* p, cudaStream_t owner) {
-  unsigned long long id = 0;
-  if (owner && context_id(&id)) {
+void device_free(const DevMem& m) {
+  if (m.stream) {
     try {
-      if (give_back(p, owner, id)) return;
+      OnDevice on(m.device);
+      if (on.ok && on.context == m.context && give_back(m)) return;
     } catch (const std::bad_alloc&) {
     }
   }
-  cudaFree(p);
+  cudaFree(m.p);
 }
 
 void trim_pool() { trim_to(kIdleBytes); }

@@ -9,6 +9,7 @@
 #include <cstdint>
 #include <new>
 #include <string>
+#include <utility>
 
 #include "tsgne.h"
 
@@ -168,11 +169,19 @@ struct AllocScope {
   AllocScope(const AllocScope&) = delete;
   AllocScope& operator=(const AllocScope&) = delete;
 };
-// Device memory, from the kept blocks when alloc_stream() is set (*owner is
-// then that stream, else NULL), and back once everything enqueued on owner is
-// done.
-cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t* owner);
-void device_free(void* p, cudaStream_t owner);
+// A piece of device memory with what its return needs (memory.cu).
+struct DevMem {
+  void* p = nullptr;
+  size_t bytes = 0;                // of the block, at least what was asked for
+  cudaStream_t stream = nullptr;   // orders its uses; NULL: plain cudaMalloc / cudaFree
+  int device = 0;
+  unsigned long long context = 0;  // CUDA's id of the context it belongs to
+};
+// Device memory on the current device, from the kept blocks when
+// alloc_stream() is set, and back once everything enqueued on that stream is
+// done.  device_free may be called with any device selected.
+cudaError_t device_alloc(DevMem* m, size_t bytes);
+void device_free(const DevMem& m);
 // Gives idle blocks above the bound (all of them) back to the device.
 void trim_pool();
 void release_idle_blocks();
@@ -194,24 +203,27 @@ template <class T>
 struct DevBuf {
   T* p = nullptr;
   size_t n = 0;
-  cudaStream_t as = nullptr;  // its owner's stream (device_alloc)
+  DevMem mem;
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
-  DevBuf(DevBuf&& o) noexcept : p(o.p), n(o.n), as(o.as) { o.p = nullptr; o.n = 0; o.as = nullptr; }
+  DevBuf(DevBuf&& o) noexcept { swap(o); }
   DevBuf& operator=(DevBuf&& o) noexcept {
-    if (this != &o) { reset(); p = o.p; n = o.n; as = o.as; o.p = nullptr; o.n = 0; o.as = nullptr; }
+    if (this != &o) {
+      reset();
+      swap(o);
+    }
     return *this;
   }
   ~DevBuf() { reset(); }
   void reset() {
     if (p) {
-      device_free(p, as);
+      device_free(mem);
       device_bytes_release(n * sizeof(T));
     }
     p = nullptr;
     n = 0;
-    as = nullptr;
+    mem = DevMem{};
   }
   tsgne_status alloc(size_t count) {
     reset();
@@ -220,17 +232,20 @@ struct DevBuf {
       last_msg() = "device memory limit reached (tsgne_set_device_memory_limit)";
       return TSGNE_ERR_OOM;
     }
-    void* q = nullptr;
-    const cudaError_t e = device_alloc(&q, count * sizeof(T), &as);
-    p = static_cast<T*>(q);
+    const cudaError_t e = device_alloc(&mem, count * sizeof(T));
     if (e != cudaSuccess) {
-      p = nullptr;
-      as = nullptr;
+      mem = DevMem{};
       device_bytes_release(count * sizeof(T));
       return cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
     }
+    p = static_cast<T*>(mem.p);
     n = count;
     return TSGNE_OK;
+  }
+  void swap(DevBuf& o) noexcept {
+    std::swap(p, o.p);
+    std::swap(n, o.n);
+    std::swap(mem, o.mem);
   }
   T* get() const { return p; }
 };

@@ -1,0 +1,199 @@
+// The calls of the CUDA runtime that memory.cu makes, over two pretended
+// devices with one context each, and scenarios over the library's buffers.
+// Addresses are handed out lowest first, so that a freed address comes back;
+// a thread has no context until it selects a device.  Every buffer's bytes
+// are checked against what its address was allocated with.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <memory>
+#include <mutex>
+#include <string>
+#include <thread>
+#include <vector>
+
+#include "tsgne_internal.cuh"
+
+namespace fake {
+std::mutex mu;
+struct Allocation {
+  size_t bytes;
+  int device;
+};
+std::map<uintptr_t, Allocation> live;
+struct Event {
+  int device;
+  cudaStream_t on;
+};
+thread_local int device = 0;
+thread_local bool bound = false;  // whether the thread has a context
+int bad = 0;
+long mallocs = 0, frees = 0;
+size_t capacity = (size_t)1 << 40;
+
+size_t held(int dev = -1) {
+  std::lock_guard<std::mutex> lk(mu);
+  size_t s = 0;
+  for (auto& a : live)
+    if (dev < 0 || a.second.device == dev) s += a.second.bytes;
+  return s;
+}
+int context_id(void*, unsigned long long* id) {
+  if (!bound) return 201;  // invalid context
+  *id = 1000 + device;
+  return 0;
+}
+}  // namespace fake
+
+#define EXPECT(c)                                                          \
+  do {                                                                     \
+    if (!(c)) {                                                            \
+      std::fprintf(stderr, "line %d: not true: %s\n", __LINE__, #c);       \
+      std::exit(1);                                                        \
+    }                                                                      \
+  } while (0)
+
+extern "C" {
+cudaError_t CUDARTAPI cudaGetDevice(int* d) {
+  *d = fake::device;
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaSetDevice(int d) {
+  if (d < 0 || d > 1) return cudaErrorInvalidDevice;
+  fake::device = d;
+  fake::bound = true;
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaMalloc(void** p, size_t bytes) {
+  fake::bound = true;
+  size_t all = fake::held(fake::device);
+  std::lock_guard<std::mutex> lk(fake::mu);
+  if (all + bytes > fake::capacity) return cudaErrorMemoryAllocation;
+  uintptr_t at = (uintptr_t)(fake::device + 1) << 44;
+  for (auto& a : fake::live) {
+    if (a.second.device != fake::device) continue;
+    if (at + bytes <= a.first) break;
+    at = (a.first + a.second.bytes + 511) / 512 * 512;
+  }
+  fake::live[at] = {bytes, fake::device};
+  ++fake::mallocs;
+  *p = reinterpret_cast<void*>(at);
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaFree(void* p) {
+  std::lock_guard<std::mutex> lk(fake::mu);
+  if (fake::live.erase(reinterpret_cast<uintptr_t>(p)) == 0) ++fake::bad;
+  ++fake::frees;
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaEventCreateWithFlags(cudaEvent_t* e, unsigned int) {
+  fake::bound = true;
+  *e = reinterpret_cast<cudaEvent_t>(new fake::Event{fake::device, nullptr});
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaEventDestroy(cudaEvent_t e) {
+  delete reinterpret_cast<fake::Event*>(e);
+  return cudaSuccess;
+}
+// streams 100..199 belong to device 0, 200..299 to device 1
+static int device_of(cudaStream_t s) { return (int)(reinterpret_cast<uintptr_t>(s) / 100) - 1; }
+cudaError_t CUDARTAPI cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+  auto* v = reinterpret_cast<fake::Event*>(e);
+  if (reinterpret_cast<uintptr_t>(s) >= 100 && device_of(s) != v->device) return cudaErrorInvalidResourceHandle;
+  v->on = s;
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t CUDARTAPI cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned int) { return cudaSuccess; }
+cudaError_t CUDARTAPI cudaGetLastError(void) { return cudaSuccess; }
+const char* CUDARTAPI cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t CUDARTAPI cudaGetDriverEntryPointByVersion(const char* symbol, void** fn, unsigned int, unsigned long long,
+                                                       cudaDriverEntryPointQueryResult* q) {
+  EXPECT(std::strcmp(symbol, "cuCtxGetId") == 0);
+  *fn = reinterpret_cast<void*>(&fake::context_id);
+  if (q) *q = cudaDriverEntryPointSuccess;
+  return cudaSuccess;
+}
+}  // extern "C"
+
+namespace tsgne {
+std::string& last_msg() {
+  static thread_local std::string m;
+  return m;
+}
+tsgne_status cuda_fail(cudaError_t e, const char*, const char*, int) {
+  return e == cudaErrorMemoryAllocation ? TSGNE_ERR_OOM : TSGNE_ERR_CUDA;
+}
+}  // namespace tsgne
+
+using tsgne::AllocScope;
+using Buf = tsgne::DevBuf<unsigned char>;
+
+static cudaStream_t stream(int k) { return reinterpret_cast<cudaStream_t>((uintptr_t)k); }
+static void holds(const Buf& b) {  // the buffer lies within one allocation
+  std::lock_guard<std::mutex> lk(fake::mu);
+  auto it = fake::live.find(reinterpret_cast<uintptr_t>(b.get()));
+  EXPECT(it != fake::live.end());
+  EXPECT(b.n <= it->second.bytes);
+}
+static tsgne_status take(Buf& b, size_t bytes, int s) {
+  AllocScope as(stream(s));
+  return b.alloc(bytes);
+}
+
+constexpr size_t KiB = 1 << 10, MiB = 1 << 20;
+
+// A buffer freed where its device is not the current one, or where the thread
+// has no context, leaves nothing behind that a later buffer could be given.
+static void freed_elsewhere(bool fresh_thread) {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
+  auto a = std::make_unique<Buf>();
+  EXPECT(take(*a, MiB, 100) == TSGNE_OK);
+  if (fresh_thread) {
+    std::thread([&] { a.reset(); }).join();
+  } else {
+    EXPECT(cudaSetDevice(1) == cudaSuccess);
+    a.reset();
+    EXPECT(fake::device == 1);  // the caller's device stays selected
+    EXPECT(cudaSetDevice(0) == cudaSuccess);
+  }
+  Buf keep;  // nothing idle is left to hide the driver's reuse of the address
+  tsgne_set_device_memory_limit(0);
+  for (size_t bytes : {64 * KiB, 48 * KiB, 4 * KiB}) {
+    Buf b;
+    EXPECT(take(b, bytes, 100) == TSGNE_OK);
+    holds(b);
+  }
+  std::vector<Buf> all(8);
+  for (Buf& b : all) {
+    EXPECT(take(b, MiB, 100) == TSGNE_OK);
+    holds(b);
+  }
+  EXPECT(fake::bad == 0);
+}
+
+// Buffers of both devices, freed under either, come back to their own device.
+static void two_devices() {
+  for (int round = 0; round < 4; ++round) {
+    std::vector<Buf> v(16);
+    for (int k = 0; k < 16; ++k) {
+      EXPECT(cudaSetDevice(k & 1) == cudaSuccess);
+      EXPECT(take(v[k], (size_t)(k + 1) * 96 * KiB, k & 1 ? 200 : 100) == TSGNE_OK);
+      holds(v[k]);
+      EXPECT(fake::live.at(reinterpret_cast<uintptr_t>(v[k].get())).device == (k & 1));
+    }
+    EXPECT(cudaSetDevice(round & 1) == cudaSuccess);
+  }
+  tsgne_set_device_memory_limit(0);
+  EXPECT(fake::held() == 0 && fake::bad == 0);
+}
+
+int main(int argc, char** argv) {
+  const std::string s = argc > 1 ? argv[1] : "";
+  if (s == "other_device") freed_elsewhere(false);
+  else if (s == "fresh_thread") freed_elsewhere(true);
+  else if (s == "two_devices") two_devices();
+  else return 2;
+  return 0;
+}
