@@ -617,7 +617,6 @@ void tsgne_destroy(tsgne_ctx* ctx) {
   DeviceGuard g(ctx->device, ctx->stream);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   delete ctx;
-  trim_pool();
 }
 
 const char* tsgne_last_error(const tsgne_ctx* ctx) { return ctx ? ctx->err.c_str() : last_msg().c_str(); }
@@ -677,7 +676,6 @@ tsgne_status tsgne_build_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, co
   if (h.flags & kFlagNonfiniteP) return fail(ctx, TSGNE_ERR_NONFINITE, "non-finite affinity (check X)");
   API_TRY(ctx, install(ctx, n, nnz, rp, col, P));
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  trim_pool();
   return TSGNE_OK;
 }
 
@@ -734,7 +732,6 @@ tsgne_status tsgne_set_P(tsgne_ctx* ctx, int32_t n, const int64_t* row_ptr, cons
   API_CUDA(ctx, cudaMemsetAsync(ctx->sched.get(), 0, sizeof(Sched), ctx->stream));
   API_TRY(ctx, install(ctx, n, nnz, rp, col, P));
   API_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  trim_pool();
   return TSGNE_OK;
 }
 

@@ -765,7 +765,6 @@ void tsgne_batch_destroy(tsgne_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
   delete b;
-  trim_pool();
 }
 
 const char* tsgne_batch_last_error(const tsgne_batch* b) { return b ? b->err.c_str() : ""; }

@@ -14,8 +14,10 @@
 // takes the block next makes its own stream wait for that event, so a block
 // never changes hands before the work that used it is done, whatever the
 // streams and threads.  At most kIdleBytes are kept per device, the longest
-// idle block goes first; trim_pool() sees to that at the end of every build
-// and with every object destroyed.  All idle blocks go back to the device when
+// idle block goes first: what an entry point's temporaries leave above that
+// goes back when the entry point returns (the end of its AllocScope, which
+// stands before them), what is freed outside of one at once.  All idle blocks
+// go back to the device when
 // an allocation fails and when the library's memory limit is set.  Blocks
 // belong to one CUDA context (recognised by its id): what a context destroyed
 // by cudaDeviceReset held is forgotten.  A buffer carries its block's size,
@@ -36,6 +38,7 @@ std::atomic<int64_t> g_dev_bytes{0};
 std::atomic<int64_t> g_dev_limit{0};  // 0: no limit
 
 constexpr size_t kIdleBytes = (size_t)256 << 20;  // freed bytes kept (0.1 % of a GB300)
+std::atomic<bool> g_over{false};                  // a device may hold more than that
 
 struct Block {
   void* p;
@@ -167,6 +170,10 @@ bool give_back(const DevMem& m) {
   }
   b.idle.push_back(Block{m.p, m.bytes, ev});
   b.idle_bytes += m.bytes;
+  if (b.idle_bytes > kIdleBytes) {
+    if (alloc_stream()) g_over = true;  // the end of the scope sees to it
+    else shrink(b, kIdleBytes);
+  }
   return true;
 }
 
@@ -229,7 +236,9 @@ void device_free(const DevMem& m) {
   cudaFree(m.p);
 }
 
-void trim_pool() { trim_to(kIdleBytes); }
+void trim_idle_blocks() {
+  if (g_over.exchange(false)) trim_to(kIdleBytes);
+}
 void release_idle_blocks() { trim_to(0); }
 
 }  // namespace tsgne

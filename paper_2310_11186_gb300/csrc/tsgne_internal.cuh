@@ -160,12 +160,19 @@ void device_bytes_release(size_t bytes);
 
 // Stream that orders the uses of what the calling thread allocates (NULL:
 // plain cudaMalloc / cudaFree); every entry point sets it to its object's
-// stream (AllocScope).  See memory.cu.
+// stream (AllocScope, declared before the buffers that the call frees: the
+// end of the outermost one brings the idle blocks back to their bound).  See
+// memory.cu.
 cudaStream_t& alloc_stream();
+void trim_idle_blocks();     // to the bound
+void release_idle_blocks();  // all of them
 struct AllocScope {
   cudaStream_t saved;
   explicit AllocScope(cudaStream_t s) : saved(alloc_stream()) { alloc_stream() = s; }
-  ~AllocScope() { alloc_stream() = saved; }
+  ~AllocScope() {
+    alloc_stream() = saved;
+    if (!saved) trim_idle_blocks();
+  }
   AllocScope(const AllocScope&) = delete;
   AllocScope& operator=(const AllocScope&) = delete;
 };
@@ -182,9 +189,6 @@ struct DevMem {
 // done.  device_free may be called with any device selected.
 cudaError_t device_alloc(DevMem* m, size_t bytes);
 void device_free(const DevMem& m);
-// Gives idle blocks above the bound (all of them) back to the device.
-void trim_pool();
-void release_idle_blocks();
 
 // A stream that its object destroys after everything declared behind it
 // (buffers are freed on it).

@@ -189,11 +189,41 @@ static void two_devices() {
   EXPECT(fake::held() == 0 && fake::bad == 0);
 }
 
+// At most 256 MiB stay idle once a call has returned (its scope has ended),
+// also when it failed, and at once where no call is running.
+static void idle_bound() {
+  const size_t bound = 256 * MiB;
+  for (int k = 0; k < 3; ++k) {
+    AllocScope as(stream(100));
+    std::vector<Buf> v(6);
+    for (Buf& b : v) EXPECT(b.alloc(100 * MiB) == TSGNE_OK);
+  }
+  EXPECT(fake::held() <= bound);
+  std::vector<Buf> v(6);
+  {
+    AllocScope outer(stream(100));
+    for (Buf& b : v) EXPECT(take(b, 90 * MiB, 101) == TSGNE_OK);
+    Buf t;  // the inner scopes' ends leave the call's own temporaries alone
+    EXPECT(t.alloc(30 * MiB) == TSGNE_OK);
+  }
+  const size_t before = fake::held();
+  size_t out = 0;
+  for (Buf& b : v) {
+    out += b.n;
+    b.reset();
+    EXPECT(fake::held() <= before - out + bound);
+  }
+  EXPECT(fake::held() <= bound && fake::held() > 0);
+  tsgne_set_device_memory_limit(0);
+  EXPECT(fake::held() == 0 && fake::bad == 0);
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   if (s == "other_device") freed_elsewhere(false);
   else if (s == "fresh_thread") freed_elsewhere(true);
   else if (s == "two_devices") two_devices();
+  else if (s == "idle_bound") idle_bound();
   else return 2;
   return 0;
 }
