@@ -249,11 +249,17 @@ tsgne_status tsgne_kernel_times(tsgne_ctx* ctx, double* ms, int64_t* launches, i
  * counterpart: the limit serves hosts that share a GPU among tenants, and
  * tests of the out-of-memory paths.  Freed memory of the library's objects
  * stays with the library for its next allocations, at most 256 MiB of it per
- * device; this call gives all of it back (as a failed allocation does).
+ * device between calls; this call gives all of it back (as a failed
+ * allocation does).  The limit covers it: it goes back before an allocation
+ * would pass the limit.  A buffer allocated while no limit is set lies in a
+ * block that may be larger than the buffer, by up to 9/16 below 2 MiB and by
+ * up to 1/16 and 2 MiB above (not at all above 256 MiB); the account counts
+ * the block.  While a limit is set every buffer gets exactly its bytes.
  */
 void tsgne_set_device_memory_limit(int64_t bytes);
 
-/* Device bytes the library holds at the moment (same account). */
+/* Device bytes the library's objects hold at the moment (same account,
+ * without the freed memory kept for the next allocations). */
 int64_t tsgne_device_memory_in_use(void);
 
 /* Launch geometry of the exact repulsion pass (cfg.repulsion = 0; with the
@@ -473,8 +479,9 @@ void tsgne_server_config_default(tsgne_server_config* cfg);
  * batch with the given tile (P, layout, optimiser state, initial layout,
  * fixed-point repulsion accumulators, Z partials, an upper bound for the hub-row
  * chunk lists); -1 for invalid arguments.  A tree-code member holds about
- * 144 bytes per point more (its tree); the server adds them.  Host
- * arithmetic only (no GPU needed). */
+ * 144 bytes per point more (its tree); the server adds them.  Bytes of the
+ * buffers, as under tsgne_set_device_memory_limit; their blocks may be larger
+ * as described there.  Host arithmetic only (no GPU needed). */
 int64_t tsgne_server_estimate_bytes(int32_t n, int64_t nnz, int32_t tile_warps);
 
 /* cfg (may be NULL: defaults) configures every layout; cuda_stream as for

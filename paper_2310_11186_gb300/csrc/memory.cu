@@ -1,5 +1,8 @@
 // Device memory of the library's objects: an account with an optional limit,
-// and freed blocks kept for the next allocation.
+// and freed blocks kept for the next allocation.  The account counts blocks as
+// they were allocated (block_size), not what their buffers asked for; under a
+// limit a buffer gets exactly what it asks for, from a block of that size or a
+// new one, and idle blocks count as long as they are there.
 //
 // Why blocks are kept: a P build makes about 30 allocations, most of them
 // temporaries.  On GB300 cudaMalloc takes 35 us and cudaFree 31 us (a wait for
@@ -34,8 +37,8 @@ namespace tsgne {
 
 namespace {
 
-std::atomic<int64_t> g_dev_bytes{0};
-std::atomic<int64_t> g_dev_limit{0};  // 0: no limit
+std::atomic<int64_t> g_used{0};   // bytes of the blocks in use, as they were allocated
+std::atomic<int64_t> g_limit{0};  // on those and the idle ones together; 0: none
 
 constexpr size_t kIdleBytes = (size_t)256 << 20;  // freed bytes kept (0.1 % of a GB300)
 std::atomic<bool> g_over{false};                  // a device may hold more than that
@@ -101,11 +104,23 @@ Blocks& blocks_of(unsigned long long id, int device) {
   return all_blocks().back();
 }
 
-// Sizes of blocks: quarter octaves from 4 KiB, so that similar requests share blocks.
+// Sizes of blocks, so that similar requests share them: quarter octaves from
+// 4 KiB, multiples of 2 MiB from there (the pages that cudaMalloc maps).
+constexpr size_t kPage = (size_t)2 << 20;
 size_t block_size(size_t bytes) {
   size_t step = 1024;
-  while (8 * step < bytes) step *= 2;
+  while (8 * step < bytes && step < kPage) step *= 2;
   return (bytes + step - 1) / step * step;
+}
+// Whether an idle block serves a request of want bytes.
+bool serves(size_t block, size_t want) { return block >= want && block - want <= (want < kPage ? want / 4 : want / 16); }
+
+void keep_event(Blocks& b, cudaEvent_t ev) {
+  try {
+    b.spare.push_back(ev);
+  } catch (const std::bad_alloc&) {
+    cudaEventDestroy(ev);
+  }
 }
 
 // Returns idle blocks to the device, longest idle first, until at most keep bytes are left.
@@ -116,37 +131,84 @@ void shrink(Blocks& b, size_t keep) {
     b.idle_bytes -= k.bytes;
     cudaEventSynchronize(k.done);
     cudaFree(k.p);
-    b.spare.push_back(k.done);
+    keep_event(b, k.done);
   }
 }
 
+// Every context's idle blocks down to keep bytes; a context that is no longer its device's is forgotten.
+void shrink_all(size_t keep) {
+  for (auto b = all_blocks().begin(); b != all_blocks().end();) {
+    if (b->idle_bytes > keep) {
+      OnDevice on(b->device);
+      if (!on.ok || on.context != b->context) {
+        b = all_blocks().erase(b);
+        continue;
+      }
+      shrink(*b, keep);
+    }
+    ++b;
+  }
+}
+
+// Whether the limit leaves room for a block of bytes in use beside the others;
+// fresh: one that is not among the idle ones yet, which then make way for it.
+bool within_limit(size_t bytes, bool fresh) {
+  const int64_t lim = g_limit.load();
+  if (lim <= 0) return true;
+  if (g_used.load() + (int64_t)bytes > lim) return false;
+  if (!fresh) return true;
+  int64_t idle = 0;
+  for (const Blocks& b : all_blocks()) idle += (int64_t)b.idle_bytes;
+  if (idle > 0 && g_used.load() + idle + (int64_t)bytes > lim) shrink_all(0);
+  return true;
+}
+
+cudaError_t fresh_block(DevMem* m, Blocks* b, size_t bytes) {
+  cudaError_t e = cudaMalloc(&m->p, bytes);
+  if (e == cudaErrorMemoryAllocation && b != nullptr && b->idle_bytes > 0) {
+    cudaGetLastError();
+    shrink(*b, 0);
+    e = cudaMalloc(&m->p, bytes);
+  }
+  m->bytes = bytes;
+  return e;
+}
+
+// A block for bytes (cudaErrorMemoryAllocation with m->bytes = 0: the limit forbids it).
 cudaError_t take(DevMem* m, size_t bytes) {
   std::lock_guard<std::mutex> lk(g_mu);
-  Blocks& b = blocks_of(m->context, m->device);
-  const size_t want = block_size(bytes);
-  auto best = b.idle.end();
-  for (auto it = b.idle.begin(); it != b.idle.end(); ++it)  // at most twice the size asked for
-    if (it->bytes >= want && it->bytes <= 2 * want && (best == b.idle.end() || it->bytes < best->bytes)) best = it;
-  if (best != b.idle.end()) {
-    const Block k = *best;
-    b.spare.reserve(b.spare.size() + 1);  // before anything changes
-    if (cudaStreamWaitEvent(m->stream, k.done, 0) == cudaSuccess) {
-      b.idle.erase(best);
-      b.idle_bytes -= k.bytes;
-      b.spare.push_back(k.done);
-      m->p = k.p;
-      m->bytes = k.bytes;
-      return cudaSuccess;
+  Blocks* const b = m->stream ? &blocks_of(m->context, m->device) : nullptr;
+  // Exactly what is asked for while a limit is set, so that rounding refuses
+  // nothing, and where the block can never be kept.
+  const bool exact = b == nullptr || g_limit.load() > 0 || bytes > kIdleBytes;
+  const size_t want = exact ? bytes : block_size(bytes);
+  if (b != nullptr) {
+    auto best = b->idle.end();
+    for (auto it = b->idle.begin(); it != b->idle.end(); ++it)
+      if ((exact ? it->bytes == want : serves(it->bytes, want)) && (best == b->idle.end() || it->bytes < best->bytes))
+        best = it;
+    if (best != b->idle.end()) {
+      const Block k = *best;
+      if (!within_limit(k.bytes, false)) return cudaErrorMemoryAllocation;
+      if (cudaStreamWaitEvent(m->stream, k.done, 0) == cudaSuccess) {
+        b->idle.erase(best);
+        b->idle_bytes -= k.bytes;
+        keep_event(*b, k.done);
+        m->p = k.p;
+        m->bytes = k.bytes;
+        g_used += (int64_t)k.bytes;
+        return cudaSuccess;
+      }
+      cudaGetLastError();
     }
-    cudaGetLastError();
   }
-  cudaError_t e = cudaMalloc(&m->p, want);
-  if (e == cudaErrorMemoryAllocation && b.idle_bytes > 0) {
+  if (!within_limit(want, true)) return cudaErrorMemoryAllocation;
+  cudaError_t e = fresh_block(m, b, want);
+  if (e == cudaErrorMemoryAllocation && want > bytes) {
     cudaGetLastError();
-    shrink(b, 0);
-    e = cudaMalloc(&m->p, want);
+    e = fresh_block(m, b, bytes);
   }
-  m->bytes = want;
+  if (e == cudaSuccess) g_used += (int64_t)m->bytes;
   return e;
 }
 
@@ -165,32 +227,22 @@ bool give_back(const DevMem& m) {
   }
   if (cudaEventRecord(ev, m.stream) != cudaSuccess) {
     cudaGetLastError();
-    b.spare.push_back(ev);
+    keep_event(b, ev);
     return false;
   }
-  b.idle.push_back(Block{m.p, m.bytes, ev});
+  try {
+    b.idle.push_back(Block{m.p, m.bytes, ev});
+  } catch (const std::bad_alloc&) {
+    keep_event(b, ev);
+    return false;
+  }
   b.idle_bytes += m.bytes;
+  g_used -= (int64_t)m.bytes;
   if (b.idle_bytes > kIdleBytes) {
     if (alloc_stream()) g_over = true;  // the end of the scope sees to it
     else shrink(b, kIdleBytes);
   }
   return true;
-}
-
-// Every context's idle blocks; a context that is no longer its device's is forgotten.
-void trim_to(size_t keep) {
-  std::lock_guard<std::mutex> lk(g_mu);
-  for (auto b = all_blocks().begin(); b != all_blocks().end();) {
-    if (b->idle_bytes > keep) {
-      OnDevice on(b->device);
-      if (!on.ok || on.context != b->context) {
-        b = all_blocks().erase(b);
-        continue;
-      }
-      shrink(*b, keep);
-    }
-    ++b;
-  }
 }
 
 }  // namespace
@@ -200,52 +252,51 @@ cudaStream_t& alloc_stream() {
   return s;
 }
 
-bool device_bytes_reserve(size_t bytes) {
-  const int64_t b = (int64_t)bytes;
-  const int64_t lim = g_dev_limit.load();
-  int64_t cur = g_dev_bytes.load();
-  do {
-    if (lim > 0 && cur + b > lim) return false;
-  } while (!g_dev_bytes.compare_exchange_weak(cur, cur + b));
-  return true;
-}
-
-void device_bytes_release(size_t bytes) { g_dev_bytes.fetch_sub((int64_t)bytes); }
-
-cudaError_t device_alloc(DevMem* m, size_t bytes) {
+tsgne_status device_alloc(DevMem* m, size_t bytes) {
   *m = DevMem{};
-  const cudaStream_t s = alloc_stream();
-  if (!s || cudaGetDevice(&m->device) != cudaSuccess || !context_id(&m->context)) return cudaMalloc(&m->p, bytes);
-  m->stream = s;
+  m->stream = alloc_stream();
+  if (m->stream && (cudaGetDevice(&m->device) != cudaSuccess || !context_id(&m->context))) m->stream = nullptr;
+  cudaError_t e;
   try {
-    return take(m, bytes);
-  } catch (const std::bad_alloc&) {  // no host memory for the list: CUDA's own answer decides
+    e = take(m, bytes);
+  } catch (const std::bad_alloc&) {  // no host memory for the list: a block without it
     m->stream = nullptr;
-    return cudaMalloc(&m->p, bytes);
+    e = take(m, bytes);
   }
+  if (e == cudaSuccess) return TSGNE_OK;
+  const bool limit = m->bytes == 0;
+  *m = DevMem{};
+  if (!limit) return cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
+  last_msg() = "device memory limit reached (tsgne_set_device_memory_limit)";
+  return TSGNE_ERR_OOM;
 }
 
 void device_free(const DevMem& m) {
+  bool kept = false;
   if (m.stream) {
     try {
       OnDevice on(m.device);
-      if (on.ok && on.context == m.context && give_back(m)) return;
+      kept = on.ok && on.context == m.context && give_back(m);
     } catch (const std::bad_alloc&) {
     }
   }
+  if (kept) return;
   cudaFree(m.p);
+  g_used -= (int64_t)m.bytes;
 }
 
 void trim_idle_blocks() {
-  if (g_over.exchange(false)) trim_to(kIdleBytes);
+  if (!g_over.exchange(false)) return;
+  std::lock_guard<std::mutex> lk(g_mu);
+  shrink_all(kIdleBytes);
 }
-void release_idle_blocks() { trim_to(0); }
 
 }  // namespace tsgne
 
 extern "C" void tsgne_set_device_memory_limit(int64_t bytes) {
-  tsgne::g_dev_limit.store(bytes > 0 ? bytes : 0);
-  tsgne::release_idle_blocks();
+  std::lock_guard<std::mutex> lk(tsgne::g_mu);
+  tsgne::g_limit.store(bytes > 0 ? bytes : 0);
+  tsgne::shrink_all(0);
 }
 
-extern "C" int64_t tsgne_device_memory_in_use(void) { return tsgne::g_dev_bytes.load(); }
+extern "C" int64_t tsgne_device_memory_in_use(void) { return tsgne::g_used.load(); }

@@ -152,20 +152,13 @@ tsgne_status cuda_fail(cudaError_t e, const char* what, const char* file, int li
     if (s_ != TSGNE_OK) return s_;          \
   } while (0)
 
-// Process-wide account of the device bytes held by DevBufs, checked against
-// an optional limit (tsgne_set_device_memory_limit).  reserve() returns false
-// when the allocation would pass the limit; release() gives bytes back.
-bool device_bytes_reserve(size_t bytes);
-void device_bytes_release(size_t bytes);
-
 // Stream that orders the uses of what the calling thread allocates (NULL:
 // plain cudaMalloc / cudaFree); every entry point sets it to its object's
 // stream (AllocScope, declared before the buffers that the call frees: the
 // end of the outermost one brings the idle blocks back to their bound).  See
 // memory.cu.
 cudaStream_t& alloc_stream();
-void trim_idle_blocks();     // to the bound
-void release_idle_blocks();  // all of them
+void trim_idle_blocks();
 struct AllocScope {
   cudaStream_t saved;
   explicit AllocScope(cudaStream_t s) : saved(alloc_stream()) { alloc_stream() = s; }
@@ -186,8 +179,10 @@ struct DevMem {
 };
 // Device memory on the current device, from the kept blocks when
 // alloc_stream() is set, and back once everything enqueued on that stream is
-// done.  device_free may be called with any device selected.
-cudaError_t device_alloc(DevMem* m, size_t bytes);
+// done.  TSGNE_ERR_OOM also where the process-wide limit
+// (tsgne_set_device_memory_limit) forbids it.  device_free may be called with
+// any device selected.
+tsgne_status device_alloc(DevMem* m, size_t bytes);
 void device_free(const DevMem& m);
 
 // A stream that its object destroys after everything declared behind it
@@ -221,10 +216,7 @@ struct DevBuf {
   }
   ~DevBuf() { reset(); }
   void reset() {
-    if (p) {
-      device_free(mem);
-      device_bytes_release(n * sizeof(T));
-    }
+    if (p) device_free(mem);
     p = nullptr;
     n = 0;
     mem = DevMem{};
@@ -232,16 +224,7 @@ struct DevBuf {
   tsgne_status alloc(size_t count) {
     reset();
     if (count == 0) count = 1;
-    if (!device_bytes_reserve(count * sizeof(T))) {
-      last_msg() = "device memory limit reached (tsgne_set_device_memory_limit)";
-      return TSGNE_ERR_OOM;
-    }
-    const cudaError_t e = device_alloc(&mem, count * sizeof(T));
-    if (e != cudaSuccess) {
-      mem = DevMem{};
-      device_bytes_release(count * sizeof(T));
-      return cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
-    }
+    TS_TRY(device_alloc(&mem, count * sizeof(T)));
     p = static_cast<T*>(mem.p);
     n = count;
     return TSGNE_OK;

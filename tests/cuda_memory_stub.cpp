@@ -218,12 +218,76 @@ static void idle_bound() {
   EXPECT(fake::held() == 0 && fake::bad == 0);
 }
 
+// The account is what the device has given, and rounding refuses nothing that
+// the device itself would give.
+static void account() {
+  std::vector<Buf> v(40);
+  for (int k = 0; k < 40; ++k) EXPECT(take(v[k], (size_t)(k * k * k) * 9001 + 1, 100) == TSGNE_OK);
+  EXPECT(fake::held() == (size_t)tsgne_device_memory_in_use());
+  size_t asked = 0;
+  for (int round = 0; round < 3; ++round)
+    for (int k = 0; k < 40; ++k) {
+      v[k].reset();
+      EXPECT(take(v[k], (size_t)((k + round) * k * k) * 8513 + 1, 100) == TSGNE_OK);
+      holds(v[k]);
+    }
+  for (const Buf& b : v) asked += b.n;
+  EXPECT((size_t)tsgne_device_memory_in_use() <= asked + asked / 16 + 40 * 2 * MiB);
+  for (Buf& b : v) b.reset();
+  tsgne_set_device_memory_limit(0);
+  EXPECT(fake::held() == 0 && tsgne_device_memory_in_use() == 0);
+  fake::capacity = 99 * MiB + 512 * KiB;
+  Buf b;
+  EXPECT(take(b, 99 * MiB + 1, 100) == TSGNE_OK);
+  EXPECT(fake::held() == 99 * MiB + 1 && tsgne_device_memory_in_use() == (int64_t)(99 * MiB + 1));
+  b.reset();
+  EXPECT(take(b, 99 * MiB, 100) == TSGNE_OK);  // makes the idle block go, if it is not used
+}
+
+// Under a limit the device never gives more than it, in use and idle
+// together, and exactly what fits is accepted.
+static void limit() {
+  const size_t lim = 50 * MiB;
+  tsgne_set_device_memory_limit((int64_t)lim);
+  unsigned long long x = 1;
+  auto rnd = [&](size_t below) { return (size_t)((x = x * 6364136223846793005ull + 1442695040888963407ull) >> 33) % below; };
+  for (int round = 0; round < 200; ++round) {
+    std::vector<Buf> v(12);
+    size_t asked = 0;
+    for (Buf& b : v) {
+      const size_t bytes = rnd(3) ? 1 + rnd(9 * MiB) : 4 * MiB;
+      const tsgne_status st = take(b, bytes, 100 + (int)rnd(3));
+      EXPECT((st == TSGNE_OK) == (asked + bytes <= lim));
+      EXPECT(st == TSGNE_OK || st == TSGNE_ERR_OOM);
+      if (st == TSGNE_OK) asked += bytes, holds(b);
+      EXPECT(tsgne_device_memory_in_use() == (int64_t)asked);
+      EXPECT(fake::held() <= lim);
+    }
+  }
+  EXPECT(tsgne_device_memory_in_use() == 0);
+  const long mallocs = fake::mallocs;  // the same sizes again: kept blocks serve them
+  for (int k = 0; k < 10; ++k) {
+    Buf a, b;
+    EXPECT(take(a, 3 * MiB + 7, 100) == TSGNE_OK && take(b, 5 * MiB, 100) == TSGNE_OK);
+  }
+  EXPECT(fake::mallocs <= mallocs + 2);
+  Buf plain;  // outside a scope: counted alike
+  EXPECT(plain.alloc(lim) == TSGNE_OK && tsgne_device_memory_in_use() == (int64_t)lim);
+  Buf more;
+  EXPECT(more.alloc(1) == TSGNE_ERR_OOM && fake::held() == lim);
+  plain.reset();
+  tsgne_set_device_memory_limit(0);
+  EXPECT(fake::held() == 0 && fake::bad == 0);
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   if (s == "other_device") freed_elsewhere(false);
   else if (s == "fresh_thread") freed_elsewhere(true);
   else if (s == "two_devices") two_devices();
   else if (s == "idle_bound") idle_bound();
+  else if (s == "account") account();
+  else if (s == "limit") limit();
   else return 2;
   return 0;
 }

@@ -27,7 +27,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["other_device", "fresh_thread", "two_devices", "idle_bound"])
+@pytest.mark.parametrize("scenario", ["other_device", "fresh_thread", "two_devices", "idle_bound", "account", "limit"])
 def test_blocks(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stderr
