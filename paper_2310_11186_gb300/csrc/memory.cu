@@ -16,7 +16,8 @@
 // ordered on that stream.  Giving it back records an event there, and whoever
 // takes the block next makes its own stream wait for that event, so a block
 // never changes hands before the work that used it is done, whatever the
-// streams and threads.  At most kIdleBytes are kept per device, the longest
+// streams and threads (cudaStreamPerThread names another stream in every
+// thread, so its buffers are not kept).  At most kIdleBytes are kept per device, the longest
 // idle block goes first: what an entry point's temporaries leave above that
 // goes back when the entry point returns (the end of its AllocScope, which
 // stands before them), what is freed outside of one at once.  All idle blocks
@@ -255,6 +256,7 @@ cudaStream_t& alloc_stream() {
 tsgne_status device_alloc(DevMem* m, size_t bytes) {
   *m = DevMem{};
   m->stream = alloc_stream();
+  if (m->stream == cudaStreamPerThread) m->stream = nullptr;  // orders nothing beyond this thread
   if (m->stream && (cudaGetDevice(&m->device) != cudaSuccess || !context_id(&m->context))) m->stream = nullptr;
   cudaError_t e;
   try {

@@ -280,6 +280,19 @@ static void limit() {
   EXPECT(fake::held() == 0 && fake::bad == 0);
 }
 
+// cudaStreamPerThread is another stream in every thread: an event recorded by
+// the thread that frees says nothing about the work of the one that used the
+// buffer.  Such a buffer is not kept; its cudaFree waits for the device.
+static void per_thread_stream() {
+  Buf a;
+  {
+    AllocScope as(cudaStreamPerThread);
+    EXPECT(a.alloc(MiB) == TSGNE_OK);
+  }
+  std::thread([&] { a.reset(); }).join();
+  EXPECT(fake::held() == 0 && fake::frees == 1 && tsgne_device_memory_in_use() == 0);
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   if (s == "other_device") freed_elsewhere(false);
@@ -288,6 +301,7 @@ int main(int argc, char** argv) {
   else if (s == "idle_bound") idle_bound();
   else if (s == "account") account();
   else if (s == "limit") limit();
+  else if (s == "per_thread_stream") per_thread_stream();
   else return 2;
   return 0;
 }

@@ -27,7 +27,8 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["other_device", "fresh_thread", "two_devices", "idle_bound", "account", "limit"])
+@pytest.mark.parametrize("scenario", ["other_device", "fresh_thread", "two_devices", "idle_bound", "account", "limit",
+                                      "per_thread_stream"])
 def test_blocks(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stderr
