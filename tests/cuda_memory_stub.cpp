@@ -192,6 +192,7 @@ static void two_devices() {
 // At most 256 MiB stay idle once a call has returned (its scope has ended),
 // also when it failed, and at once where no call is running.
 static void idle_bound() {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
   const size_t bound = 256 * MiB;
   for (int k = 0; k < 3; ++k) {
     AllocScope as(stream(100));
@@ -221,6 +222,7 @@ static void idle_bound() {
 // The account is what the device has given, and rounding refuses nothing that
 // the device itself would give.
 static void account() {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
   std::vector<Buf> v(40);
   for (int k = 0; k < 40; ++k) EXPECT(take(v[k], (size_t)(k * k * k) * 9001 + 1, 100) == TSGNE_OK);
   EXPECT(fake::held() == (size_t)tsgne_device_memory_in_use());
@@ -247,6 +249,7 @@ static void account() {
 // Under a limit the device never gives more than it, in use and idle
 // together, and exactly what fits is accepted.
 static void limit() {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
   const size_t lim = 50 * MiB;
   tsgne_set_device_memory_limit((int64_t)lim);
   unsigned long long x = 1;
@@ -284,6 +287,7 @@ static void limit() {
 // the thread that frees says nothing about the work of the one that used the
 // buffer.  Such a buffer is not kept; its cudaFree waits for the device.
 static void per_thread_stream() {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
   Buf a;
   {
     AllocScope as(cudaStreamPerThread);
