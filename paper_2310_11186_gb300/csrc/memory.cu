@@ -287,6 +287,15 @@ void device_free(const DevMem& m) {
   g_used -= (int64_t)m.bytes;
 }
 
+int64_t idle_device_bytes() {
+  unsigned long long id = 0;
+  if (!context_id(&id)) return 0;
+  std::lock_guard<std::mutex> lk(g_mu);
+  for (const Blocks& b : all_blocks())
+    if (b.context == id) return (int64_t)b.idle_bytes;
+  return 0;
+}
+
 void trim_idle_blocks() {
   if (!g_over.exchange(false)) return;
   std::lock_guard<std::mutex> lk(g_mu);

@@ -3,9 +3,10 @@
 // A request is a graph (CSR + embedding, optional Y0) to lay out for a fixed
 // number of iterations.  Submitted requests wait in a FIFO queue; every tick
 //   1. admits queued requests in order while the estimated device bytes of
-//      all resident layouts stay within the budget and below the free device
-//      memory (the first request is admitted whatever its size when nothing
-//      is resident, so no request starves);
+//      all resident layouts stay within the budget and below the device
+//      memory that is free or kept idle by the library (the first request is
+//      admitted whatever its size when nothing is resident, so no request
+//      starves);
 //   2. selects the resident layouts to advance: all of them (policy 0), or
 //      (policy 1, shortest remaining work first with aging) first the
 //      layouts left out of aging_ticks ticks in a row, longest waiting
@@ -21,9 +22,10 @@
 //      freed.
 // Admission overlaps with the running iterations: an admitted request is
 // handed to a worker thread that builds its member (structure, P, buffers,
-// tree) with tsgne_batch_prepare on the worker's own stream while the tick launches the resident layouts' iterations; prepared members
-// are attached at the start of the next tick.  A tick with nothing resident
-// waits for all admitted requests to be prepared instead of running nothing.
+// tree) with tsgne_batch_prepare on the worker's own stream while the tick
+// launches the resident layouts' iterations; prepared members are attached at
+// the start of the next tick.  A tick with nothing resident waits for all
+// admitted requests to be prepared instead of running nothing.
 // Every member's arithmetic is independent of the others (batch.cu), so a
 // request's layout is the same whatever else is resident.  Cancelling a
 // queued or resident request frees it at once; its result reports
@@ -44,6 +46,7 @@
 #include <vector>
 
 #include "tsgne.h"
+#include "tsgne_internal.cuh"
 
 namespace {
 
@@ -112,10 +115,11 @@ tsgne_status batch_fail(tsgne_server* s, tsgne_status st) {
   return st;
 }
 
+// What the device has free and what the library would give back for an allocation.
 int64_t free_device_bytes(int64_t fallback) {
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return fallback;
-  return (int64_t)fr;
+  return (int64_t)fr + tsgne::idle_device_bytes();
 }
 
 tsgne_status admit(tsgne_server* s) {

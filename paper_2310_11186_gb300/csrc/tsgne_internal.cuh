@@ -184,6 +184,8 @@ struct DevMem {
 // any device selected.
 tsgne_status device_alloc(DevMem* m, size_t bytes);
 void device_free(const DevMem& m);
+// Bytes kept idle on the current device.
+int64_t idle_device_bytes();
 
 // A stream that its object destroys after everything declared behind it
 // (buffers are freed on it).

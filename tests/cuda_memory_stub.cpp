@@ -3,6 +3,7 @@
 // Addresses are handed out lowest first, so that a freed address comes back;
 // a thread has no context until it selects a device.  Every buffer's bytes
 // are checked against what its address was allocated with.
+#include <chrono>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -108,6 +109,17 @@ cudaError_t CUDARTAPI cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t CUDARTAPI cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned int) { return cudaSuccess; }
 cudaError_t CUDARTAPI cudaGetLastError(void) { return cudaSuccess; }
 const char* CUDARTAPI cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t CUDARTAPI cudaMemGetInfo(size_t* free, size_t* total) {
+  *total = fake::capacity;
+  *free = fake::capacity - fake::held(fake::device);
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaStreamCreateWithFlags(cudaStream_t* s, unsigned int) {
+  *s = reinterpret_cast<cudaStream_t>((uintptr_t)150);
+  return cudaSuccess;
+}
+cudaError_t CUDARTAPI cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t CUDARTAPI cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t CUDARTAPI cudaGetDriverEntryPointByVersion(const char* symbol, void** fn, unsigned int, unsigned long long,
                                                        cudaDriverEntryPointQueryResult* q) {
   EXPECT(std::strcmp(symbol, "cuCtxGetId") == 0);
@@ -129,6 +141,46 @@ tsgne_status cuda_fail(cudaError_t e, const char*, const char*, int) {
 
 using tsgne::AllocScope;
 using Buf = tsgne::DevBuf<unsigned char>;
+
+// A batch whose members hold what the server estimates for them.
+struct tsgne_member {
+  Buf mem;
+};
+struct tsgne_batch {
+  std::vector<std::unique_ptr<tsgne_member>> members;
+};
+extern "C" {
+tsgne_status tsgne_batch_create(tsgne_batch** out, const tsgne_config*, int32_t, void*) {
+  *out = new tsgne_batch();
+  return TSGNE_OK;
+}
+void tsgne_batch_destroy(tsgne_batch* b) { delete b; }
+const char* tsgne_batch_last_error(const tsgne_batch*) { return ""; }
+const char* tsgne_last_error(const tsgne_ctx*) { return ""; }
+const char* tsgne_status_string(tsgne_status) { return ""; }
+tsgne_status tsgne_batch_prepare(tsgne_batch*, int32_t n, const int64_t* rp, const int32_t*, const float*, int32_t,
+                                 const float*, int32_t, int32_t, void* s, tsgne_member** out) {
+  AllocScope as(static_cast<cudaStream_t>(s));
+  *out = new tsgne_member();
+  return (*out)->mem.alloc((size_t)tsgne_server_estimate_bytes(n, 2 * rp[n], 1));
+}
+tsgne_status tsgne_batch_attach(tsgne_batch* b, tsgne_member* m, int32_t* id) {
+  *id = (int32_t)b->members.size();
+  b->members.emplace_back(m);
+  return TSGNE_OK;
+}
+void tsgne_batch_discard(tsgne_member* m) { delete m; }
+tsgne_status tsgne_batch_remove(tsgne_batch* b, int32_t id) {
+  b->members[id].reset();
+  return TSGNE_OK;
+}
+tsgne_status tsgne_batch_set_active(tsgne_batch*, int32_t, int32_t) { return TSGNE_OK; }
+tsgne_status tsgne_batch_run(tsgne_batch*, int32_t) { return TSGNE_OK; }
+tsgne_status tsgne_batch_get_Y(tsgne_batch*, int32_t, float*, int32_t* iter, int32_t) {
+  *iter = 20;
+  return TSGNE_OK;
+}
+}  // extern "C"
 
 static cudaStream_t stream(int k) { return reinterpret_cast<cudaStream_t>((uintptr_t)k); }
 static void holds(const Buf& b) {  // the buffer lies within one allocation
@@ -297,6 +349,43 @@ static void per_thread_stream() {
   EXPECT(fake::held() == 0 && fake::frees == 1 && tsgne_device_memory_in_use() == 0);
 }
 
+// A request waits for memory that is in use, not for memory that the library
+// only keeps for its next allocations.
+static void server_admission() {
+  EXPECT(cudaSetDevice(0) == cudaSuccess);
+  tsgne_server_config c{};
+  c.budget_bytes = (int64_t)1 << 40;
+  c.iters = 100000;
+  c.tick_iters = 10;
+  c.max_members = 8;
+  c.tile_warps = 1;
+  c.fill_pairs = 1e18;
+  tsgne_server* s = nullptr;
+  EXPECT(tsgne_server_create(&s, &c, nullptr, nullptr) == TSGNE_OK);
+  const int32_t n = 300000;
+  const int64_t need = tsgne_server_estimate_bytes(n, 0, 1);
+  std::vector<int64_t> rp(n + 1, 0);
+  std::vector<float> X(n, 0.f);
+  Buf kept;  // 200 MiB idle, and room for less than one more request beside the first
+  EXPECT(take(kept, 200 * MiB, 100) == TSGNE_OK);
+  kept.reset();
+  fake::capacity = 200 * MiB + (size_t)need + (size_t)need / 2;
+  int32_t resident = 0, queued = 0;
+  for (int want = 1; want <= 2; ++want) {
+    int64_t id;
+    EXPECT(tsgne_server_submit(s, n, rp.data(), nullptr, X.data(), 1, nullptr, &id) == TSGNE_OK);
+    for (int t = 0; t < 2000 && resident < want; ++t) {
+      EXPECT(tsgne_server_tick(s, &resident, &queued, nullptr) == TSGNE_OK);
+      std::this_thread::sleep_for(std::chrono::milliseconds(1));
+    }
+  }
+  EXPECT(resident == 2 && queued == 0);
+  EXPECT(fake::held() <= fake::capacity);
+  tsgne_server_destroy(s);
+  tsgne_set_device_memory_limit(0);
+  EXPECT(fake::held() == 0 && fake::bad == 0);
+}
+
 int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   if (s == "other_device") freed_elsewhere(false);
@@ -306,6 +395,7 @@ int main(int argc, char** argv) {
   else if (s == "account") account();
   else if (s == "limit") limit();
   else if (s == "per_thread_stream") per_thread_stream();
+  else if (s == "server_admission") server_admission();
   else return 2;
   return 0;
 }
