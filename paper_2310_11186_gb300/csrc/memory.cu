@@ -96,9 +96,12 @@ struct OnDevice {
   OnDevice& operator=(const OnDevice&) = delete;
 };
 
-Blocks& blocks_of(unsigned long long id, int device) {
+// The current context's blocks.
+Blocks& blocks_of(unsigned long long id) {
   for (Blocks& b : all_blocks())
     if (b.context == id) return b;
+  int device = 0;
+  cudaGetDevice(&device);
   all_blocks().emplace_back();
   all_blocks().back().context = id;
   all_blocks().back().device = device;
@@ -136,18 +139,19 @@ void shrink(Blocks& b, size_t keep) {
   }
 }
 
-// Every context's idle blocks down to keep bytes; a context that is no longer its device's is forgotten.
+// Every context's idle blocks down to keep bytes; those of a context that can
+// no longer be selected stay where they are.
 void shrink_all(size_t keep) {
-  for (auto b = all_blocks().begin(); b != all_blocks().end();) {
-    if (b->idle_bytes > keep) {
-      OnDevice on(b->device);
-      if (!on.ok || on.context != b->context) {
-        b = all_blocks().erase(b);
-        continue;
-      }
-      shrink(*b, keep);
+  unsigned long long id = 0;
+  context_id(&id);
+  for (Blocks& b : all_blocks()) {
+    if (b.idle_bytes <= keep) continue;
+    if (b.context == id) {
+      shrink(b, keep);
+      continue;
     }
-    ++b;
+    OnDevice on(b.device);
+    if (on.ok && on.context == b.context) shrink(b, keep);
   }
 }
 
@@ -178,7 +182,7 @@ cudaError_t fresh_block(DevMem* m, Blocks* b, size_t bytes) {
 // A block for bytes (cudaErrorMemoryAllocation with m->bytes = 0: the limit forbids it).
 cudaError_t take(DevMem* m, size_t bytes) {
   std::lock_guard<std::mutex> lk(g_mu);
-  Blocks* const b = m->stream ? &blocks_of(m->context, m->device) : nullptr;
+  Blocks* const b = m->stream ? &blocks_of(m->context) : nullptr;
   // Exactly what is asked for while a limit is set, so that rounding refuses
   // nothing, and where the block can never be kept.
   const bool exact = b == nullptr || g_limit.load() > 0 || bytes > kIdleBytes;
@@ -217,7 +221,7 @@ cudaError_t take(DevMem* m, size_t bytes) {
 bool give_back(const DevMem& m) {
   if (m.bytes > kIdleBytes) return false;
   std::lock_guard<std::mutex> lk(g_mu);
-  Blocks& b = blocks_of(m.context, m.device);
+  Blocks& b = blocks_of(m.context);
   cudaEvent_t ev = nullptr;
   if (!b.spare.empty()) {
     ev = b.spare.back();
@@ -257,7 +261,7 @@ tsgne_status device_alloc(DevMem* m, size_t bytes) {
   *m = DevMem{};
   m->stream = alloc_stream();
   if (m->stream == cudaStreamPerThread) m->stream = nullptr;  // orders nothing beyond this thread
-  if (m->stream && (cudaGetDevice(&m->device) != cudaSuccess || !context_id(&m->context))) m->stream = nullptr;
+  if (m->stream && !context_id(&m->context)) m->stream = nullptr;
   cudaError_t e;
   try {
     e = take(m, bytes);
@@ -274,15 +278,23 @@ tsgne_status device_alloc(DevMem* m, size_t bytes) {
 }
 
 void device_free(const DevMem& m) {
-  bool kept = false;
   if (m.stream) {
-    try {
-      OnDevice on(m.device);
-      kept = on.ok && on.context == m.context && give_back(m);
-    } catch (const std::bad_alloc&) {
+    unsigned long long id = 0;
+    if (context_id(&id) && id == m.context) {
+      if (give_back(m)) return;
+    } else {  // another device is selected, or the thread has no context
+      int device = -1;
+      {
+        std::lock_guard<std::mutex> lk(g_mu);
+        for (const Blocks& b : all_blocks())
+          if (b.context == m.context) device = b.device;
+      }
+      if (device >= 0) {
+        OnDevice on(device);
+        if (on.ok && on.context == m.context && give_back(m)) return;
+      }
     }
   }
-  if (kept) return;
   cudaFree(m.p);
   g_used -= (int64_t)m.bytes;
 }

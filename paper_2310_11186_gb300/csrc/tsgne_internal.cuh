@@ -174,7 +174,6 @@ struct DevMem {
   void* p = nullptr;
   size_t bytes = 0;                // of the block, at least what was asked for
   cudaStream_t stream = nullptr;   // orders its uses; NULL: plain cudaMalloc / cudaFree
-  int device = 0;
   unsigned long long context = 0;  // CUDA's id of the context it belongs to
 };
 // Device memory on the current device, from the kept blocks when
