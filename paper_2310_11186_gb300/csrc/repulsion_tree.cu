@@ -718,10 +718,12 @@ __global__ void __launch_bounds__(kTileLeaves)
   ClimbTile& t = *reinterpret_cast<ClimbTile*>(climb_smem);
   if (__ldcg(&o.st->sort_stall)) return;
   const int t0 = (int)blockIdx.x * kUpTiles, t1 = min(ntiles, t0 + kUpTiles);
-  const int c = load_items(t, in, t0, t1, n, keys);
-  if (c > kTileLeaves) {
+  // another CTA of this launch may be setting it: one thread looks for all
+  const bool gave_up = __syncthreads_or(threadIdx.x == 0 && __ldcg(&o.st->climb_global) != 0u);
+  const int c = gave_up ? 0 : load_items(t, in, t0, t1, n, keys);
+  if (gave_up || c > kTileLeaves) {
     if (threadIdx.x == 0) {
-      o.st->climb_global = 1u;
+      if (!gave_up) o.st->climb_global = 1u;
       out.counts[blockIdx.x] = 0;
     }
     return;
