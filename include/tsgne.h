@@ -193,7 +193,8 @@ tsgne_status tsgne_init_Y(tsgne_ctx* ctx, const float* Y0, int32_t ptr_kind);
 /*
  * One iteration, enqueued on the context's stream (no host synchronisation):
  * repulsion F^r_i = sum_{j != i} w_ij^2 (y_i - y_j) and Z = sum_{k != l} w_kl
- * (Eq. 4, w = (1 + ||y_k - y_l||^2)^-1, Z accumulated in FP64), attraction
+ * (Eq. 4, w = (1 + ||y_k - y_l||^2)^-1; Z sums FP32 partials of at most 1,024
+ * w exactly, in steps of 2^-96: points up to 2.8e14 apart count), attraction
  * F^a_i = sum_{j in N(i)} p_ij w_ij (y_i - y_j), gradient
  * g = 4 (alpha F^a - F^r / Z) of Eq. 5, then gains, momentum and y += update.
  * A non-finite layout is reported by the next synchronising call.

@@ -297,7 +297,7 @@ tsgne_status discard_forces(tsgne_ctx* ctx) {
 // Z of the last pass, from a copy of the device's scalars.
 double host_z(const tsgne_ctx* ctx, const Sched& h) {
   if (!symmetric_pass(ctx)) return h.Z;
-  return z_of(h.zacc[ctx->zpass][0], h.zacc[ctx->zpass][1], h.zbad[ctx->zpass], ctx->n);
+  return z_value(h.zacc[ctx->zpass], h.zbad[ctx->zpass], ctx->n);
 }
 
 // Reads of the current layout / P for the force kernels of the context.

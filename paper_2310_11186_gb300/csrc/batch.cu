@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
   float2* sacc = reinterpret_cast<float2*>(smem + T);
   longlong2* si = reinterpret_cast<longlong2*>(sacc + T);
   __shared__ int s_unit, s_g, s_a, s_b;
-  __shared__ u64 s_z[W];
+  __shared__ u64 s_z[2 * W];
   const int tid = threadIdx.x;
   for (bool first = true;; first = false) {
     if (tid == 0) {
@@ -126,14 +126,15 @@ __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
     }
     const float2* Y = d.Y[d.sched->t & 1];
     bool bad;
-    u64 zt;
+    ZSum zb;
     if (RI == 8 && d.split > 1) {  // only tiles of 8 i-points per lane are cut
-      zt = sym_units<W, 8, float2>(Y, d.n, d.acc, d.fscale, a, b, G / d.split, sj, sacc, si);
-      bad = zt == ~0ull;
+      zb = sym_units<W, 8, float2>(Y, d.n, d.acc, d.fscale, a, b, G / d.split, sj, sacc, si, s_z);
+      bad = zb.hi == ~0ull;
+      if (bad) zb = ZSum{};
     } else {
-      zt = sym_unit<W, RI, float2, true>(Y, d.n, d.acc, d.fscale, a, b, 0, G, sj, sacc, &bad);
+      const ZSum zt = sym_unit<W, RI, float2, true>(Y, d.n, d.acc, d.fscale, a, b, 0, G, sj, sacc, &bad);
+      zb = cta_z<W>(zt, &bad, s_z);
     }
-    const u64 zb = cta_z<W>(bad ? 0ull : zt, &bad, s_z);
     if (tid == 0) put_z(zb, bad, nullptr, d.sched->zacc[0], &d.sched->zbad[0]);
     __syncthreads();
   }
@@ -143,17 +144,17 @@ __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
 __global__ void __launch_bounds__(32 * kSmallWarps)
     k_batch_small(const GraphDesc* __restrict__ descs, const int* __restrict__ unit_off, int members) {
   __shared__ float4 sj[kSmallMaxChunk];
-  __shared__ u64 s_z[kSmallWarps];
+  __shared__ u64 s_z[2 * kSmallWarps];
   const int g = find_owner(unit_off, members, (int)blockIdx.x);
   const GraphDesc& d = descs[g];
   const int u = (int)blockIdx.x - unit_off[g], nc = small_chunks(d.n);
   bool bad;
-  const u64 zt = small_unit<float2>(d.Y[d.sched->t & 1], d.n, d.acc, d.fscale, u / nc, u % nc, sj, &bad);
-  const u64 zb = cta_z<kSmallWarps>(zt, &bad, s_z);
+  const ZSum zt = small_unit<float2>(d.Y[d.sched->t & 1], d.n, d.acc, d.fscale, u / nc, u % nc, sj, &bad);
+  const ZSum zb = cta_z<kSmallWarps>(zt, &bad, s_z);
   if (threadIdx.x == 0) put_z(zb, bad, nullptr, d.sched->zacc[0], &d.sched->zbad[0]);
 }
 
-// One thread per exact member: Z and 1 / Z from its units' sums, which are
+// One thread per exact member: Z and 1 / Z from its units' sum, which is
 // cleared for the next iteration, and its schedule.
 __global__ void k_batch_finalize(const GraphDesc* __restrict__ descs, int members, BatchCtr* ctr, float ee,
                                  int ee_iters, float mom0, float mom1) {
@@ -161,10 +162,10 @@ __global__ void k_batch_finalize(const GraphDesc* __restrict__ descs, int member
   if (g == 0) ctr->work_next[0] = ctr->work_next[1] = 0u;
   if (g >= members || descs[g].tree) return;  // a tree member's walk set Z and the schedule
   Sched* s = descs[g].sched;
-  const double Z = z_of(s->zacc[0][0], s->zacc[0][1], s->zbad[0], descs[g].n);
+  const double Z = z_value(s->zacc[0], s->zbad[0], descs[g].n);
   s->Z = Z;
   s->inv_z = inv_of(Z);
-  s->zacc[0][0] = s->zacc[0][1] = 0ull;
+  for (u64& w : s->zacc[0]) w = 0ull;
   s->zbad[0] = 0u;
   set_schedule(s, 1, ee, ee_iters, mom0, mom1);
 }

@@ -18,8 +18,8 @@
 // longer independent chains per lane hide the reciprocal latency better than
 // more warps do.  Unit (a, b), a < b, adds the forces of tile a's points and
 // of its j-points into their accumulators; a diagonal unit evaluates its
-// ordered pairs with the i-side only.  Z: each unit adds its fixed-point value
-// to two words of the slot of this pass; the rows that use the forces turn
+// ordered pairs with the i-side only.  Z: each unit adds its exact value
+// to the words of the slot of this pass; the rows that use the forces turn
 // them into 1 / Z, so the pass ends with its units.  Layouts of at most
 // kSmallPoints points take k_repulsion_small instead.
 //
@@ -49,8 +49,7 @@ namespace {
 __device__ __forceinline__ void open_pass(Sched* s, int slot, int advance, float ee, int ee_iters, float mom0,
                                           float mom1) {
   const int o = slot ^ 1;
-  s->zacc[o][0] = 0ull;
-  s->zacc[o][1] = 0ull;
+  for (u64& w : s->zacc[o]) w = 0ull;
   s->zbad[o] = 0u;
   s->work_next[o] = 0u;
   set_schedule(s, advance, ee, ee_iters, mom0, mom1);
@@ -71,7 +70,7 @@ __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
   float4* sj = smem;                                    // TJ x {-x, -x, -y, -y}
   float2* sacc = reinterpret_cast<float2*>(smem + TJ);  // TJ x force accumulator
   __shared__ int s_unit, s_a, s_b;
-  __shared__ u64 s_z[W];
+  __shared__ u64 s_z[2 * W];
   const int tid = threadIdx.x;
   const int pairs = tile_pairs(nt);
   if (blockIdx.x == 0 && tid == 0 && zunit == nullptr) open_pass(sched, slot, advance, ee, ee_iters, mom0, mom1);
@@ -94,8 +93,8 @@ __global__ void __launch_bounds__(W * 32, warps_per_sm(RI) / W)
       continue;
     }
     bool bad;
-    const u64 zt = sym_unit<W, RI, YT, kWhole>(Y, n, acc, fscale, a, b, sub, G / split, sj, sacc, &bad);
-    const u64 zb = cta_z<W>(zt, &bad, s_z);
+    const ZSum zt = sym_unit<W, RI, YT, kWhole>(Y, n, acc, fscale, a, b, sub, G / split, sj, sacc, &bad);
+    const ZSum zb = cta_z<W>(zt, &bad, s_z);
     if (tid == 0) put_z(zb, bad, zunit ? zunit + u : nullptr, sched->zacc[slot], &sched->zbad[slot]);
     __syncthreads();  // shared tiles are rewritten by the next unit
   }
@@ -108,13 +107,13 @@ __global__ void __launch_bounds__(32 * kSmallWarps)
                       double* __restrict__ zunit, Sched* sched, int slot, int u0, int advance, float ee,
                       int ee_iters, float mom0, float mom1) {
   __shared__ float4 sj[kSmallMaxChunk];
-  __shared__ u64 s_z[kSmallWarps];
+  __shared__ u64 s_z[2 * kSmallWarps];
   const int u = u0 + (int)blockIdx.x, nc = small_chunks(n);
   if (blockIdx.x == 0 && threadIdx.x == 0 && zunit == nullptr)
     open_pass(sched, slot, advance, ee, ee_iters, mom0, mom1);
   bool bad;
-  const u64 zt = small_unit<YT>(Y, n, acc, fscale, u / nc, u % nc, sj, &bad);
-  const u64 zb = cta_z<kSmallWarps>(zt, &bad, s_z);
+  const ZSum zt = small_unit<YT>(Y, n, acc, fscale, u / nc, u % nc, sj, &bad);
+  const ZSum zb = cta_z<kSmallWarps>(zt, &bad, s_z);
   if (threadIdx.x == 0) put_z(zb, bad, zunit ? zunit + u : nullptr, sched->zacc[slot], &sched->zbad[slot]);
 }
 
@@ -123,30 +122,27 @@ __global__ void __launch_bounds__(32 * kSmallWarps)
 __global__ void __launch_bounds__(1024)
     k_finalize_z(const double* __restrict__ zunit, int units, Sched* sched, int slot, int advance, float ee,
                  int ee_iters, float mom0, float mom1) {
-  __shared__ u64 low, high;
+  __shared__ u64 sum[kZWords];
   __shared__ uint32_t nan;
-  if (threadIdx.x == 0) {
-    low = high = 0ull;
-    nan = 0u;
-  }
+  if (threadIdx.x < kZWords) sum[threadIdx.x] = 0ull;
+  if (threadIdx.x == 0) nan = 0u;
   __syncthreads();
-  u64 l = 0ull, h = 0ull;
+  u64 words[kZWords] = {};
   bool bad = false;
   for (int k = threadIdx.x; k < units; k += blockDim.x) {
     const double z = zunit[k];
     bad |= z != z;
-    const u64 r = __double2ull_rn(z * (double)(1ull << kZShift));
-    l += r & 0xffffffffull;
-    h += r >> 32;
+    const ZSum v = z_fix(z);
+#pragma unroll
+    for (int w = 0; w < kZWords; ++w) words[w] += z_word(v, w);
   }
-  atomicAdd(&low, l);
-  atomicAdd(&high, h);
+#pragma unroll
+  for (int w = 0; w < kZWords; ++w) atomicAdd(&sum[w], words[w]);
   if (bad) atomicOr(&nan, 1u);
   __syncthreads();
   if (threadIdx.x == 0) {
     open_pass(sched, slot, advance, ee, ee_iters, mom0, mom1);
-    sched->zacc[slot][0] = low;
-    sched->zacc[slot][1] = high;
+    for (int w = 0; w < kZWords; ++w) sched->zacc[slot][w] = sum[w];
     sched->zbad[slot] = nan;
   }
 }

@@ -40,13 +40,14 @@
 // then all apply the round's accepted nodes and exact points, so the dependent
 // node loads along the tree are issued 32 at a time.  Z: FP32 partial sums of a
 // round, added without loss into a pair of FP32 sums per lane, the pairs over
-// the warp's lanes, and every group's total as an integer multiple of 2^-32 --
+// the warp's lanes, and every group's total as an exact integer (zsum.cuh) --
 // the same bits in whatever order groups finish.
 #include <cmath>
 
 #include "f32x2.cuh"
 #include "reduce.cuh"
 #include "tsgne_internal.cuh"
+#include "zsum.cuh"
 
 namespace tsgne {
 
@@ -1029,10 +1030,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
       two_sum(zs, ze, __shfl_xor_sync(0xffffffffu, zs, o), __shfl_xor_sync(0xffffffffu, ze, o));
     if (lane == 0) {
       const double z = (double)zs + (double)ze;
-      const long long whole = __double2ll_rd(z);
-      const unsigned long long part = __double2ull_rn((z - (double)whole) * 4294967296.0);
-      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&st->zsum[0]), "l"(part) : "memory");
-      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&st->zsum[1]), "l"(whole) : "memory");
+      z_add(st->zsum, z_fix(z));
       if (z != z) atomicOr(&st->zbad, 1u);
       if (overflow) atomicOr(&sched->flags, kFlagTreeOverflow);
     }
@@ -1045,10 +1043,12 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 4)
   }
   if (arrive_last(&st->walk_done)) {
     if (threadIdx.x == 0) {
-      const long long whole = (long long)__ldcg(&st->zsum[1]);
-      const double total = __ldcg(&st->zbad) ? (double)NAN
-                                             : (double)whole + (double)__ldcg(&st->zsum[0]) * (1.0 / 4294967296.0);
-      st->zsum[0] = st->zsum[1] = 0ull;
+      unsigned long long words[kZWords];
+      for (int k = 0; k < kZWords; ++k) {
+        words[k] = __ldcg(&st->zsum[k]);
+        st->zsum[k] = 0ull;
+      }
+      const double total = z_value(words, __ldcg(&st->zbad), 0);
       st->zbad = 0u;
       st->next_group = 0u;
       if (stalled)

@@ -8,6 +8,7 @@
 
 #include "storage.cuh"
 #include "tsgne_internal.cuh"
+#include "zsum.cuh"
 
 namespace tsgne {
 
@@ -152,18 +153,10 @@ __device__ __forceinline__ float inv_of(double Z) {
   return isfinite(e) ? fmaf(-r, e, r) : r;
 }
 
-// Z of the symmetric exact pass from its fixed-point words (NaN if a kernel
-// value was NaN).
-__host__ __device__ __forceinline__ double z_of(unsigned long long low, unsigned long long high, uint32_t bad, int n) {
-  static_assert(kZShift == 32, "the high word counts whole units");
-  const double z = (double)high + (double)low * (1.0 / (double)(1ull << kZShift)) - (double)n;
-  return bad ? (double)NAN : z;
-}
-
 // 1 / Z of the pass whose forces the rows use (see AttractArgs).
 __device__ __forceinline__ float pass_inv_z(const Sched* sched, int zslot, int n) {
   if (zslot < 0) return sched->inv_z;
-  return inv_of(z_of(sched->zacc[zslot][0], sched->zacc[zslot][1], sched->zbad[zslot], n));
+  return inv_of(z_value(sched->zacc[zslot], sched->zbad[zslot], n));
 }
 
 // Where a row's repulsive force comes from (see AttractArgs): F^r per row, or

@@ -13,7 +13,7 @@
 // Z: each lane's FP32 partial of a point covers one 64-point ring group
 // (64 terms w in (0, 1]), is then added into a second FP32 partial over the
 // unit's groups (at most 16 for 1,024-point tiles), and from there on the
-// sums are exact integers (kZShift).  The worst-case relative rounding of a
+// sums are exact integers (zsum.cuh).  The worst-case relative rounding of a
 // unit's row sum is then about (63 + 15) 2^-24 = 4.6e-6, against 1,023 2^-24 =
 // 6.1e-5 for one FP32 sum over the whole tile.  The integers also replace the
 // FP64 sums that ended every unit and the last CTA's sum over all of them: on
@@ -24,6 +24,7 @@
 #include "f32x2.cuh"
 #include "storage.cuh"
 #include "tsgne_internal.cuh"
+#include "zsum.cuh"
 
 namespace tsgne {
 
@@ -80,51 +81,42 @@ __device__ __forceinline__ void red_fix(unsigned long long* p, float v, float sc
   red_int(p, __float2ll_rn(v * scale));  // v * 2^s is exact: scale is a power of two
 }
 
-// The fixed-point value of a Z partial z >= 0 (NaN: the caller's check).
-__device__ __forceinline__ u64 z_fix(float z) { return __float2ull_rn(z * (float)(1ull << kZShift)); }
-
-// Sum over the warp's lanes of integers below 2^58, in every lane.
-__device__ __forceinline__ u64 warp_sum_u58(u64 v) {
-  const u64 m = (1ull << 27) - 1;
-  const u64 a = __reduce_add_sync(0xffffffffu, (uint32_t)(v & m));
-  const u64 b = __reduce_add_sync(0xffffffffu, (uint32_t)((v >> 27) & m));
-  const u64 c = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 54));
-  return a + (b << 27) + (c << 54);
-}
-
-// One thread: the Z of a unit to its place: as a double (exact: below 2^53
-// for every shape of a single layout) in zunit, for a share of a sharded pass,
-// or added to the two words of zacc.
-__device__ __forceinline__ void put_z(u64 q, bool bad, double* zunit, u64* zacc, uint32_t* zbad) {
+// One thread: the Z of a unit to its place: as a double (exact) in zunit, for
+// a share of a sharded pass, or added to the words of zacc.
+__device__ __forceinline__ void put_z(ZSum q, bool bad, double* zunit, u64* zacc, uint32_t* zbad) {
   if (zunit != nullptr) {
-    *zunit = bad ? (double)NAN : (double)q * (1.0 / (double)(1ull << kZShift));
+    *zunit = bad ? (double)NAN : z_double(q);
     return;
   }
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(zacc), "l"(q & 0xffffffffull) : "memory");
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(zacc + 1), "l"(q >> 32) : "memory");
+  z_add(zacc, q);
   if (bad) atomicOr(zbad, 1u);
 }
 
-// Sum over a CTA of W warps of the threads' Z (valid in thread 0); *bad: any
-// thread's.  zs: W words of shared memory, free again after a __syncthreads.
+// The Z of a unit: the sum over a CTA of W warps of the threads' (valid in
+// thread 0).  *bad: any thread's.  zs: 2 W words of shared memory, free again
+// after a __syncthreads.
 template <int W>
-__device__ __forceinline__ u64 cta_z(u64 q, bool* bad, u64* zs) {
+__device__ __forceinline__ ZSum cta_z(ZSum q, bool* bad, u64* zs) {
   const bool any = __any_sync(0xffffffffu, *bad);
-  u64 v = warp_sum_u58(q);
+  ZSum v = z_warp_sum(q);
   *bad = any;
-  if (W == 1) return v;
-  if ((threadIdx.x & 31) == 0) zs[threadIdx.x >> 5] = any ? ~0ull : v;
+  if (W == 1) return z_top53(v);
+  if ((threadIdx.x & 31) == 0) {
+    const int w = threadIdx.x >> 5;
+    zs[2 * w] = any ? ~0ull : v.hi;
+    zs[2 * w + 1] = v.lo;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    v = 0ull;
+    v = ZSum{};
     *bad = false;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-      *bad |= zs[w] == ~0ull;
-      v += zs[w];
+      *bad |= zs[2 * w] == ~0ull;
+      v.add(ZSum{zs[2 * w], zs[2 * w + 1]});
     }
   }
-  return v;
+  return z_top53(v);
 }
 
 // The schedule of the iteration that follows a pass (one thread).
@@ -231,28 +223,44 @@ __device__ __forceinline__ void add_j(int jb, int TJ, int n, const float2* sacc,
     }
 }
 
-// The thread's Z in fixed point from its lane partials (ordered pairs:
+// The Z of N lane partials, those that count (the others are 0); *bad: a NaN
+// among them.  The second half of the sum only where a lane of the warp needs
+// it (15 iterations of 2,000 points: 254 us with it throughout, 245 us so; a
+// BF16 gradient of 65,536 points: 783 and 768 us).
+template <int N>
+__device__ __forceinline__ ZSum lane_z(const float (&z)[N], bool* bad) {
+  ZSum s;
+  float zn = 0.f;  // NaN if any partial is
+  bool small = false;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    s.hi += z_hi(z[k]);
+    zn += z[k];
+    small |= z[k] < kZWhole;
+  }
+  *bad = zn != zn;
+  if (__any_sync(0xffffffffu, small && zn != 0.f)) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) s.add(ZSum{0ull, z_lo(z[k])});
+  }
+  return s;
+}
+
+// The thread's Z from its lane partials (ordered pairs:
 // twice the off-diagonal units', whose tile a holds no padding; the diagonal
 // units' real points, w_ii = 1 included); *bad: a NaN among them.
 template <int kH>
-__device__ __forceinline__ u64 unit_z(bool off_diagonal, int ibase, int n, const u64 (&ZG)[kH], bool* bad) {
-  u64 zt = 0ull;
-  float zn = 0.f;  // NaN if any partial is
+__device__ __forceinline__ ZSum unit_z(bool off_diagonal, int ibase, int n, const u64 (&ZG)[kH], bool* bad) {
+  const float twice = off_diagonal ? 2.f : 1.f;
+  float z[2 * kH];
 #pragma unroll
   for (int h = 0; h < kH; ++h) {
     float z0, z1;
     upk(ZG[h], z0, z1);
-    if (off_diagonal || ibase + (2 * h) * 32 < n) {
-      zt += z_fix(z0);
-      zn += z0;
-    }
-    if (off_diagonal || ibase + (2 * h + 1) * 32 < n) {
-      zt += z_fix(z1);
-      zn += z1;
-    }
+    z[2 * h] = off_diagonal || ibase + (2 * h) * 32 < n ? twice * z0 : 0.f;
+    z[2 * h + 1] = off_diagonal || ibase + (2 * h + 1) * 32 < n ? twice * z1 : 0.f;
   }
-  *bad = zn != zn;
-  return off_diagonal ? 2ull * zt : zt;
+  return lane_z(z, bad);
 }
 
 // Loads of the lane's i-points of tile a: i = a T + warp 32 RI + r 32 + lane, r < RI.
@@ -292,9 +300,9 @@ __device__ __forceinline__ void add_i(int ibase, int n, const u64 (&FX)[RI / 2],
 // compiler schedules the ring loop, where a large pass spends its time,
 // depends on what else is inlined beside it (300,000 points: 15.86 ms with
 // both calls, 16.07 with this one alone, 16.2 with neither; 100,000: 1.80,
-// 1.83, 1.92 ms).  A NaN comes back as ~0.
+// 1.83, 1.92 ms).  A NaN comes back as hi = ~0.
 template <int W, int RI, class YT>
-static __device__ __noinline__ u64 diag_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+static __device__ __noinline__ ZSum diag_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
                                              float fscale, int a, int sub, int G, float4* sj, float2* sacc) {
   constexpr int kH = RI / 2;
   const int TJ = G * kGroup;
@@ -307,9 +315,10 @@ static __device__ __noinline__ u64 diag_unit(const YT* __restrict__ Y, int n, un
   __syncthreads();
   unit_pairs<W, kH>(G, false, sj, sacc, X2, Y2, FX, FY, ZG);
   bool bad;
-  const u64 zt = unit_z<kH>(false, ibase, n, ZG, &bad);
+  ZSum zt = unit_z<kH>(false, ibase, n, ZG, &bad);
   add_i<RI>(ibase, n, FX, FY, acc, fscale);
-  return bad ? ~0ull : zt;
+  if (bad) zt.hi = ~0ull;
+  return zt;
 }
 
 // One unit of a layout: the points of tile a against the G ring groups of
@@ -317,12 +326,11 @@ static __device__ __noinline__ u64 diag_unit(const YT* __restrict__ Y, int n, un
 // tile, and sub = 0 for kWhole; see split_tiles).  Stages those j-points,
 // evaluates the pairs and adds tile a's forces and (a < b) the j-points'
 // forces into the fixed-point accumulators acc[2 p], acc[2 p + 1] of the real
-// points (p < n).  Returns this thread's share of the unit's Z in fixed point
-// (unit_z).  Every thread of the CTA must call it; it ends with the shared
+// points (p < n).  Returns this thread's share of the unit's Z (unit_z).  Every thread of the CTA must call it; it ends with the shared
 // tiles free for reuse only after a __syncthreads by the caller.  G is a power
 // of two, at least W.
 template <int W, int RI, class YT, bool kWhole>
-__device__ __forceinline__ u64 sym_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+__device__ __forceinline__ ZSum sym_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
                                         float fscale, int a, int b, int sub, int groups, float4* sj, float2* sacc,
                                         bool* bad) {
   constexpr int kH = RI / 2;  // FP32x2 pairs of i-points per lane
@@ -331,9 +339,9 @@ __device__ __forceinline__ u64 sym_unit(const YT* __restrict__ Y, int n, unsigne
   const int G = kWhole ? T / kGroup : groups;  // a constant for whole tiles
   const int TJ = G * kGroup;
   if (a == b) {
-    const u64 z = diag_unit<W, RI, YT>(Y, n, acc, fscale, a, sub, G, sj, sacc);
-    *bad = z == ~0ull;
-    return *bad ? 0ull : z;
+    const ZSum z = diag_unit<W, RI, YT>(Y, n, acc, fscale, a, sub, G, sj, sacc);
+    *bad = z.hi == ~0ull;
+    return *bad ? ZSum{} : z;
   }
   const int jb = b * T + sub * TJ;  // first j-point
   stage_j<W>(Y, jb, TJ, sj, sacc);
@@ -344,7 +352,7 @@ __device__ __forceinline__ u64 sym_unit(const YT* __restrict__ Y, int n, unsigne
   for (int h = 0; h < kH; ++h) FX[h] = FY[h] = ZG[h] = 0ull;
   __syncthreads();
   unit_pairs<W, kH>(G, true, sj, sacc, X2, Y2, FX, FY, ZG);
-  const u64 zt = unit_z<kH>(true, ibase, n, ZG, bad);
+  const ZSum zt = unit_z<kH>(true, ibase, n, ZG, bad);
   add_j<W>(jb, TJ, n, sacc, acc, fscale);
   add_i<RI>(ibase, n, FX, FY, acc, fscale);
   return zt;
@@ -354,11 +362,12 @@ __device__ __forceinline__ u64 sym_unit(const YT* __restrict__ Y, int n, unsigne
 // so the same bits, as S calls of sym_unit.  For a batch, whose members fill
 // the GPU together: both tiles are loaded once, the i-points' integer sums
 // stay in shared memory (si: T long2, each thread its own points) and reach
-// the accumulators once instead of S times.  Returns the thread's Z.
+// the accumulators once instead of S times.  Returns the sum of the units' Z
+// in thread 0 (a NaN as hi = ~0).  zs: 2 W words of shared memory.
 template <int W, int RI, class YT>
-static __device__ __noinline__ u64 sym_units(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+static __device__ __noinline__ ZSum sym_units(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
                                              float fscale, int a, int b, int G, float4* sj, float2* sacc,
-                                             longlong2* si) {
+                                             longlong2* si, u64* zs) {
   constexpr int kH = RI / 2;
   constexpr int T = W * 32 * RI;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -368,7 +377,7 @@ static __device__ __noinline__ u64 sym_units(const YT* __restrict__ Y, int n, un
   stage_j<W>(Y, b * T, T, sj, sacc);
   load_i<RI>(Y, ibase, X2, Y2);
   __syncthreads();
-  u64 zt = 0ull;
+  ZSum zt;
   bool bad = false;
   for (int j0 = 0; j0 < T; j0 += G * kGroup) {
     u64 FX[kH], FY[kH], ZG[kH];
@@ -376,8 +385,9 @@ static __device__ __noinline__ u64 sym_units(const YT* __restrict__ Y, int n, un
     for (int h = 0; h < kH; ++h) FX[h] = FY[h] = ZG[h] = 0ull;
     unit_pairs<W, kH>(G, a != b, sj + j0, sacc + j0, X2, Y2, FX, FY, ZG);
     bool nan;
-    zt += unit_z<kH>(a != b, ibase, n, ZG, &nan);
+    zt.add(cta_z<W>(unit_z<kH>(a != b, ibase, n, ZG, &nan), &nan, zs));
     bad |= nan;
+    if (W > 1) __syncthreads();
 #pragma unroll
     for (int h = 0; h < kH; ++h) {
       float fx[2], fy[2];
@@ -400,7 +410,8 @@ static __device__ __noinline__ u64 sym_units(const YT* __restrict__ Y, int n, un
       red_int(acc + 2 * (size_t)(ibase + r * 32), v.x);
       red_int(acc + 2 * (size_t)(ibase + r * 32) + 1, v.y);
     }
-  return bad ? ~0ull : zt;
+  if (bad) zt.hi = ~0ull;
+  return zt;
 }
 
 // The small pass (layouts of at most kSmallPoints points).  Such a pass has
@@ -421,7 +432,7 @@ __host__ __device__ inline int small_chunks(int n) { return (n + small_chunk(n) 
 __host__ __device__ inline int small_units(int n) { return ((n + kSmallBlock - 1) / kSmallBlock) * small_chunks(n); }
 
 template <class YT>
-__device__ __forceinline__ u64 small_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
+__device__ __forceinline__ ZSum small_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
                                           float fscale, int ib, int c, float4* sj, bool* bad) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u64 one2 = pk(1.f, 1.f);
@@ -458,22 +469,16 @@ __device__ __forceinline__ u64 small_unit(const YT* __restrict__ Y, int n, unsig
   upk(ZG, z0, z1);
   upk(FX, fx0, fx1);
   upk(FY, fy0, fy1);
-  u64 zt = 0ull;
-  float zn = 0.f;
   if (i0 < n) {
     red_fix(acc + 2 * (size_t)i0, fx0, fscale);
     red_fix(acc + 2 * (size_t)i0 + 1, fy0, fscale);
-    zt += z_fix(z0);
-    zn += z0;
   }
   if (i1 < n) {
     red_fix(acc + 2 * (size_t)i1, fx1, fscale);
     red_fix(acc + 2 * (size_t)i1 + 1, fy1, fscale);
-    zt += z_fix(z1);
-    zn += z1;
   }
-  *bad = zn != zn;
-  return zt;
+  const float z[2] = {i0 < n ? z0 : 0.f, i1 < n ? z1 : 0.f};
+  return lane_z(z, bad);
 }
 
 // Units per tile pair: j sub-tiles, a power of two.  Passes on tiles of 8

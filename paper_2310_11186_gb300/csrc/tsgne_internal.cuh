@@ -45,19 +45,10 @@ struct Sched {
   double red[4];       // results of the generic reductions
   // Symmetric exact pass, one slot for this pass and one for the next (each
   // pass clears the other slot, so none has to wait for its last CTA):
-  unsigned long long zacc[2][2];  // Z + n in fixed point: low and high 32 bits of every unit's value, summed
+  unsigned long long zacc[2][4];  // Z + n, exact (zsum.cuh)
   uint32_t zbad[2];               // 1: a pair's kernel value was NaN
   uint32_t work_next[2];          // work-queue head
 };
-
-// Z of the symmetric exact pass in fixed point.  A thread's partial of a
-// point (FP32 sums of at most 64 kernel values, then over a unit's groups) is
-// rounded to a multiple of 2^-32; integers add in any order to the same bits,
-// so the units need no partials in memory, no last CTA and no order.  2^-33
-// per partial is far below the FP32 rounding of the partials that hold a
-// point's own term (2^-25).  The low 32 bits of a unit's sum and the rest are
-// added apart: neither sum can pass 2^63 below 2^31 units.
-constexpr int kZShift = 32;
 
 constexpr uint32_t kFlagNonfiniteY = 1u;
 constexpr uint32_t kFlagNonfiniteP = 2u;
@@ -329,8 +320,8 @@ tsgne_status launch_repulsion_sym(const RepShape& sh, int n, const void* Y, int 
 tsgne_status launch_repulsion_sym_units(const RepShape& sh, int n, const void* Y, int y_bf16,
                                         unsigned long long* acc, double* zpart, Sched* sched, int slot, int u0,
                                         int u1, cudaStream_t s);
-// Z and 1 / Z from zpart[0..sh.units) and the schedule: the bits that a whole
-// pass's sums give.
+// The sums of Z from zpart[0..sh.units) into sched->zacc[slot], the bits that a
+// whole pass leaves there, and the schedule.
 tsgne_status launch_finalize_z(const RepShape& sh, const double* zpart, Sched* sched, int slot, int advance, float ee,
                                int ee_iters, float mom0, float mom1, cudaStream_t s);
 // F^r[i] = sum_k part[k * n_pad + i] for k < slots, in slot order (the
@@ -484,7 +475,7 @@ struct TreeState {
   uint32_t groups;               // groups of the last tree
   uint32_t zbad;                 // 1: a group's Z was NaN
   uint32_t climb_global;         // 1: a tile of the tree's second step held too many subtrees
-  unsigned long long zsum[2];    // Z of the walk: fractions of 2^-32 and whole units, summed apart
+  unsigned long long zsum[4];    // Z of the walk, exact (zsum.cuh)
 };
 
 // Device buffers of the tree code for n points.
