@@ -274,7 +274,7 @@ tsgne_status tsgne_repulsion_shape(tsgne_ctx* ctx, int32_t* grid, int32_t* block
  * Shape of the exact repulsion pass (cfg.repulsion = 0), after P is built.
  * symmetric = 1: each unordered pair once, tile_warps 1 or 2 warps per CTA,
  * i_per_lane 8 or 16 i-points per lane (the default is chosen from n:
- * 16 i-points, 2 warps once the tile pairs fill four waves of the grid);
+ * 16 i-points, 2 warps once the tile pairs fill seven waves of the grid);
  * symmetric = 0: the ordered-pair kernel (every ordered pair, partial forces
  * per j-chunk; FP32 storage only; tile_warps / i_per_lane ignored).  Results
  * depend on the shape only through the order of FP32 partial sums.  Layouts
@@ -282,7 +282,8 @@ tsgne_status tsgne_repulsion_shape(tsgne_ctx* ctx, int32_t* grid, int32_t* block
  * their size, which every symmetric request selects.
  * tsgne_autotune times trial_passes repulsion passes of each shape (in the
  * order (2, 16, 1), (1, 16, 1), (2, 8, 1), (1, 8, 1), (-, -, 0); -1 in
- * ms_per_pass, 5 floats, for a shape that does not apply), keeps the
+ * ms_per_pass, 5 floats, for a shape that does not apply; the one symmetric
+ * shape of a layout of at most 45,056 points is timed as (1, 8, 1)), keeps the
  * fastest and records it per (SM count, ceil log2 n, storage); the layout
  * and the iteration counter are unchanged.  Synchronises.
  */
@@ -398,7 +399,9 @@ tsgne_status tsgne_batch_reset(tsgne_batch* b);
  * with each tile (1, 2, 4 warps), keeps the fastest, records it in a
  * process-wide cache keyed by (SM count, log2 of the pair count, log2 of the
  * member count), and resets every member (tsgne_batch_reset).  *chosen gets
- * the tile; ms_per_iter (may be NULL) gets the 3 measured times.
+ * the tile; ms_per_iter (may be NULL) gets the 3 measured times.  Members of
+ * at most 45,056 points and tree-code members take no part in the tile: with
+ * no others the tile stays and its time is given for each.
  */
 tsgne_status tsgne_batch_autotune(tsgne_batch* b, int32_t trial_iters, int32_t* chosen, float* ms_per_iter);
 

@@ -927,6 +927,9 @@ std::map<std::tuple<int, int, int>, int> g_shape_cache;  // (SMs, ceil log2 n, b
 // Candidate shapes of the exact pass: (warps per CTA, i-points per lane,
 // symmetric); the last is the ordered-pair kernel (FP32 storage only).
 constexpr int kCtxShapes[5][3] = {{2, 16, 1}, {1, 16, 1}, {2, 8, 1}, {1, 8, 1}, {0, 0, 0}};
+// Which of them a layout of n points has: up to kMidPoints every symmetric one
+// selects the same kernel, which goes by the name of its last.
+bool has_shape(int n, const int* c) { return n > kMidPoints || !c[2] || (c[0] == 1 && c[1] == 8); }
 
 tsgne_status set_shape(tsgne_ctx* ctx, int warps, int ri, int symmetric) {
   if (symmetric) {
@@ -993,8 +996,8 @@ tsgne_status tsgne_autotune(tsgne_ctx* ctx, int32_t trial_passes, int32_t* tile_
   for (int k = 0; k < 5 && st == TSGNE_OK; ++k) {
     const int* c = kCtxShapes[k];
     float ms = -1.f;
-    if (!c[2] && ctx->bf16) {
-      if (ms_per_pass) ms_per_pass[k] = ms;  // not a candidate with BF16 storage
+    if ((!c[2] && ctx->bf16) || !has_shape(ctx->n, c)) {  // the ordered kernel reads FP32 layouts only
+      if (ms_per_pass) ms_per_pass[k] = ms;
       continue;
     }
     st = cudaStreamSynchronize(ctx->stream) == cudaSuccess ? TSGNE_OK : TSGNE_ERR_CUDA;

@@ -922,20 +922,26 @@ namespace {
 // Times trial_iters iterations of each candidate shape from the members'
 // initial state, keeps the fastest (the members are reset to their initial
 // state afterwards) and caches it per (SM count, log2 pairs, log2 members).
+// Without an exact member above kMidPoints no candidate changes a launch: the
+// shape stays what it is, and its time is every candidate's.
 tsgne_status autotune(tsgne_batch* b, int32_t trial_iters, const int (*cand)[2], int ncand, float* ms_out,
                       int* best_w, int* best_ri) {
   TS_TRY(refresh(b));
   double pairs = 0.0;
   for (auto& m : b->members) pairs += 0.5 * (double)m->n * (double)m->n;
   const auto key = std::make_tuple(b->sms, (int)std::log2(pairs + 1.0), (int)std::log2((double)b->members.size() + 1.0));
+  const int now[1][2] = {{b->W, b->RI}};
+  const bool one = b->U == 0;
+  const int timed = one ? 1 : ncand;
   int bw = -1, bri = -1;
   float best_ms = 0.f;
   cudaEvent_t e0, e1;
   TS_CUDA(cudaEventCreate(&e0));
   TS_CUDA(cudaEventCreate(&e1));
   tsgne_status st = TSGNE_OK;
-  for (int k = 0; k < ncand && st == TSGNE_OK; ++k) {
-    st = tsgne_batch_set_shape(b, cand[k][0], cand[k][1]);
+  for (int k = 0; k < timed && st == TSGNE_OK; ++k) {
+    const int* c = one ? now[0] : cand[k];
+    st = tsgne_batch_set_shape(b, c[0], c[1]);
     if (st == TSGNE_OK) st = run_iterations(b, 1, false);  // warm-up
     if (st == TSGNE_OK) st = cudaEventRecord(e0, b->stream) == cudaSuccess ? TSGNE_OK : TSGNE_ERR_CUDA;
     if (st == TSGNE_OK) st = run_iterations(b, trial_iters, false);
@@ -945,10 +951,11 @@ tsgne_status autotune(tsgne_batch* b, int32_t trial_iters, const int (*cand)[2],
     if (st == TSGNE_OK) st = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess ? TSGNE_OK : TSGNE_ERR_CUDA;
     if (st != TSGNE_OK) break;
     ms /= (float)trial_iters;
-    if (ms_out) ms_out[k] = ms;
+    if (ms_out)
+      for (int j = k; j < (one ? ncand : k + 1); ++j) ms_out[j] = ms;
     if (bw < 0 || ms < best_ms) {
-      bw = cand[k][0];
-      bri = cand[k][1];
+      bw = c[0];
+      bri = c[1];
       best_ms = ms;
     }
     st = tsgne_batch_reset(b);
