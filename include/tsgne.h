@@ -233,8 +233,8 @@ tsgne_status tsgne_set_state(tsgne_ctx* ctx, const float* Y, const float* update
  * of each kernel class since the last reset, measured with CUDA events on
  * the context's stream.  Classes: 0 repulsion (the tree walk when
  * cfg.repulsion = 1), 1 attraction+update (hub-row chunks included), 2
- * gradient export, 3 KL, 4 build, 5 sum of the ordered pass's partial forces, 6 hub-row
- * attraction chunks of the gradient export, 7 tree build
+ * gradient export, 3 KL, 4 build, 5 sum of the ordered pass's partial
+ * forces, 6 hub-row attraction chunks of the gradient export, 7 tree build
  * (bounding box, keys, sort, tree, summaries).  ms and launches hold n
  * entries (n <= 8).
  * reset != 0 clears the counters after reading.  Synchronises.
@@ -297,8 +297,9 @@ tsgne_status tsgne_sync(tsgne_ctx* ctx);
 /*
  * ---------------------------------------------------------------- batches
  * Many layouts advanced together: every iteration of every member runs in
- * four kernel launches (five when a member has rows of more than 32
- * entries; replayed as one CUDA graph per membership) instead of two
+ * at most six kernel launches (one of the exact pass per size class among
+ * the members, Z and schedule, hub rows of more than 32 entries if there are
+ * any, attraction and update; replayed as one CUDA graph per membership) instead of two
  * launches per member.  Each member keeps its own P, layout, optimiser
  * state and iteration counter on the device, may be added or removed between
  * runs (continuous batching), and evolves exactly as it would in a batch of
@@ -449,7 +450,8 @@ tsgne_status tsgne_build_P_shortest_path(tsgne_ctx* ctx, int32_t n, const int64_
  * layer).  Requests wait in a FIFO queue; each tsgne_server_tick
  *   1. admits queued requests in order while the estimated device bytes of
  *      the resident layouts (tsgne_server_estimate_bytes) stay within
- *      budget_bytes and below the free device memory -- the first request is
+ *      budget_bytes and below the device memory that is free or kept idle by
+ *      the library -- the first request is
  *      admitted whatever its size when nothing is resident;
  *   2. selects the resident layouts to advance: all (policy 0) or, policy 1,
  *      those with the least remaining iterations x n^2, in that order, until
@@ -481,8 +483,8 @@ void tsgne_server_config_default(tsgne_server_config* cfg);
 
 /* Device bytes a resident layout of n points and nnz affinities holds in a
  * batch with the given tile (P, layout, optimiser state, initial layout,
- * fixed-point repulsion accumulators, Z partials, an upper bound for the hub-row
- * chunk lists); -1 for invalid arguments.  A tree-code member holds about
+ * fixed-point repulsion accumulators, an upper bound for the hub-row chunk
+ * lists, and 8 bytes per tile pair in reserve); -1 for invalid arguments.  A tree-code member holds about
  * 144 bytes per point more (its tree); the server adds them.  Bytes of the
  * buffers, as under tsgne_set_device_memory_limit; their blocks may be larger
  * as described there.  Host arithmetic only (no GPU needed). */
@@ -532,9 +534,10 @@ tsgne_status tsgne_server_usage(tsgne_server* s, int64_t* used_bytes, int32_t* r
  * every context).  The paper runs on one CPU and describes no distribution;
  * the split follows from the form of Eq. 4: the repulsive forces and Z are
  * sums over pairs, which the exact pass evaluates in "units" (nt (nt + 1) / 2
- * tile pairs for nt tiles of a large layout), so the units can be divided among contexts and the sums added afterwards.  Each
- * context holds the whole (O(n + nnz)) state and updates every row itself;
- * only the O(n^2) repulsion is divided.
+ * tile pairs for nt tiles of a large layout), so the units can be divided
+ * among contexts and the sums added afterwards.  Each context holds the whole
+ * (O(n + nnz)) state and updates every row itself; only the O(n^2) repulsion
+ * is divided.
  *
  * An iteration on context r of w (rank and world set by tsgne_shard_set):
  *   1. tsgne_shard_repulsion: enqueues units [u0, u1) = [U r / w, U (r+1) / w)

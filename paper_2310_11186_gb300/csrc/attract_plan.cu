@@ -227,8 +227,9 @@ __global__ void __launch_bounds__(kPlanThreads, 6)
 //                  copied level by level, coalesced.
 // Bound by the reads of row_ptr, col and P and the writes of their copies
 // (16 B per entry).  A whole P build of 300,000 rows and 2.0M entries (device
-// arrays) takes 2.72 ms; with the lists built by host loops over a copy of
-// row_ptr, which these kernels replace, it took 16.5 ms.
+// arrays) took 16.5 ms with the lists built by host loops over a copy of
+// row_ptr, and 2.72 ms with these kernels instead (0.47 ms since allocations
+// come from kept blocks and a canonical structure is copied).
 enum RowList { kCodes = 0, kEntries, kHeavyRows, kChunks, kMedRows, kMedEntries, kBigChunks, kRowLists };
 
 struct RowAdds {

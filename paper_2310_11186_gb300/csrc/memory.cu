@@ -117,7 +117,9 @@ size_t block_size(size_t bytes) {
   return (bytes + step - 1) / step * step;
 }
 // Whether an idle block serves a request of want bytes.
-bool serves(size_t block, size_t want) { return block >= want && block - want <= (want < kPage ? want / 4 : want / 16); }
+bool serves(size_t block, size_t want) {
+  return block >= want && block - want <= (want < kPage ? want / 4 : want / 16);
+}
 
 void keep_event(Blocks& b, cudaEvent_t ev) {
   try {

@@ -9,22 +9,23 @@
 // bytes per point whatever the number of tiles, and its result does not
 // depend on the order in which units finish.
 //
-// Decomposition.  Points are padded to n_pad = nt * T (T = 512 W) with the
-// sentinel point.  A unit of work is a tile pair (a, b), a <= b, or one of the
-// j sub-tiles that split_tiles cuts it into; a persistent grid (8 warps per
-// SM; 2-warp CTAs once there are enough tile pairs, else 1-warp CTAs) takes
-// one unit per CTA and then the rest from a global queue.  Sixteen i-points per
-// lane and few warps beat eight i-points and 24 warps per SM on GB300: the
-// longer independent chains per lane hide the reciprocal latency better than
-// more warps do.  Unit (a, b), a < b, adds the forces of tile a's points and
-// of its j-points into their accumulators; a diagonal unit evaluates its
-// ordered pairs with the i-side only.  Z: each unit adds its exact value
-// to the words of the slot of this pass; the rows that use the forces turn
+// Decomposition.  Points are padded to n_pad = nt * T (T = 32 W points for each
+// of a lane's 8 or 16 i-points) with the sentinel point.  A unit of work is a
+// tile pair (a, b), a <= b, or one of the j sub-tiles that split_tiles cuts it
+// into; a persistent grid (warps_per_sm: 8 warps per SM with 16 i-points; 2-warp
+// CTAs once there are enough tile pairs, else 1-warp CTAs) takes one unit per
+// CTA and then the rest from a global queue.  Sixteen i-points per lane and few
+// warps beat eight i-points and 24 warps per SM on GB300 where there are tile
+// pairs enough: the longer independent chains per lane hide the reciprocal
+// latency better than more warps do.  Unit (a, b), a < b, adds the forces of
+// tile a's points and of its j-points into their accumulators; a diagonal unit
+// evaluates its ordered pairs with the i-side only.  Z: each unit adds its exact
+// value to the words of the slot of this pass; the rows that use the forces turn
 // them into 1 / Z, so the pass ends with its units.  Layouts of at most
 // kSmallPoints points take k_repulsion_small instead.
 //
-// Inside a unit (a < b).  Each of the W warps holds 512 points of tile a in
-// registers (16 per lane, as eight FP32x2 pairs).  Tile b sits in shared
+// Inside a unit (a < b), with 16 i-points per lane (8: half of each).  Each of
+// the W warps holds 512 points of tile a in registers (as eight FP32x2 pairs).  Tile b sits in shared
 // memory as {-x, -x, -y, -y} plus an FP32 force accumulator per point, cut
 // into 8W groups of 64 points.  In phase p warp w works on group (w + p) mod
 // 8W, so no two warps touch the same accumulators at once and no atomics are

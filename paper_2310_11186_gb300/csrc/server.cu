@@ -255,7 +255,7 @@ int64_t tsgne_server_estimate_bytes(int32_t n, int64_t nnz, int32_t tile_warps) 
   const int64_t hub_rows = nnz / 33 + 1, hub_chunks = nnz / 1024 + hub_rows;
   // row_ptr, col + P, Y x 2 / update / gains / F^r (n_pad_max float2 each),
   // the initial layout, the fixed-point force accumulators (16 B per
-  // point), the unit Z partials, the hub-row chunk lists
+  // point), 8 B per tile pair in reserve, the hub-row chunk lists
   return 8 * ((int64_t)n + 1) + 8 * nnz + 5 * 8 * n_pad_max + 8 * (int64_t)n + 16 * (int64_t)n + 8 * units +
          12 * hub_rows + 32 * hub_chunks + 256;
 }

@@ -326,9 +326,9 @@ static __device__ __noinline__ ZSum diag_unit(const YT* __restrict__ Y, int n, u
 // tile, and sub = 0 for kWhole; see split_tiles).  Stages those j-points,
 // evaluates the pairs and adds tile a's forces and (a < b) the j-points'
 // forces into the fixed-point accumulators acc[2 p], acc[2 p + 1] of the real
-// points (p < n).  Returns this thread's share of the unit's Z (unit_z).  Every thread of the CTA must call it; it ends with the shared
-// tiles free for reuse only after a __syncthreads by the caller.  G is a power
-// of two, at least W.
+// points (p < n).  Returns this thread's share of the unit's Z (unit_z).  Every
+// thread of the CTA must call it; it ends with the shared tiles free for reuse
+// only after a __syncthreads by the caller.  G is a power of two, at least W.
 template <int W, int RI, class YT, bool kWhole>
 __device__ __forceinline__ ZSum sym_unit(const YT* __restrict__ Y, int n, unsigned long long* __restrict__ acc,
                                         float fscale, int a, int b, int sub, int groups, float4* sj, float2* sacc,
