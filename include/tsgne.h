@@ -254,7 +254,7 @@ tsgne_status tsgne_kernel_times(tsgne_ctx* ctx, double* ms, int64_t* launches, i
  * allocation does).  The limit covers it: it goes back before an allocation
  * would pass the limit.  A buffer allocated while no limit is set lies in a
  * block that may be larger than the buffer, by up to 9/16 below 2 MiB and by
- * up to 1/16 and 2 MiB above (not at all above 256 MiB); the account counts
+ * up to 1/4 and 2.5 MiB above (not at all above 256 MiB); the account counts
  * the block.  While a limit is set every buffer gets exactly its bytes.
  */
 void tsgne_set_device_memory_limit(int64_t bytes);

@@ -17,14 +17,13 @@
 // takes the block next makes its own stream wait for that event, so a block
 // never changes hands before the work that used it is done, whatever the
 // streams and threads (cudaStreamPerThread names another stream in every
-// thread, so its buffers are not kept).  At most kIdleBytes are kept per device, the longest
-// idle block goes first: what an entry point's temporaries leave above that
-// goes back when the entry point returns (the end of its AllocScope, which
-// stands before them), what is freed outside of one at once.  All idle blocks
-// go back to the device when
-// an allocation fails and when the library's memory limit is set.  Blocks
-// belong to one CUDA context (recognised by its id): what a context destroyed
-// by cudaDeviceReset held is forgotten.  A buffer carries its block's size,
+// thread, so its buffers are not kept).  At most kIdleBytes are kept per device
+// between calls: what an entry point's temporaries leave above that goes back
+// when the entry point returns (the end of its AllocScope, which stands before
+// them), what is freed outside of one at once.  All idle blocks go back to the
+// device when an allocation fails and when the library's memory limit is set.
+// Blocks belong to one CUDA context (recognised by its id): what a context
+// destroyed by cudaDeviceReset held is not touched again.  A buffer carries its block's size,
 // device and context itself, so it goes back where it came from whatever the
 // freeing thread has selected, and nothing about it is kept here meanwhile.
 #include <atomic>
@@ -116,10 +115,11 @@ size_t block_size(size_t bytes) {
   while (8 * step < bytes && step < kPage) step *= 2;
   return (bytes + step - 1) / step * step;
 }
-// Whether an idle block serves a request of want bytes.
-bool serves(size_t block, size_t want) {
-  return block >= want && block - want <= (want < kPage ? want / 4 : want / 16);
-}
+// Whether an idle block serves a request of want bytes: up to a quarter more.
+// (A sixteenth above 2 MiB makes a call need so many blocks of its own
+// that they pass the bound and are allocated anew each time: P by walks on
+// 100,000 nodes takes 3.80 ms instead of 3.58, twice the size 3.46.)
+bool serves(size_t block, size_t want) { return block >= want && block - want <= want / 4; }
 
 void keep_event(Blocks& b, cudaEvent_t ev) {
   try {
@@ -129,11 +129,17 @@ void keep_event(Blocks& b, cudaEvent_t ev) {
   }
 }
 
-// Returns idle blocks to the device, longest idle first, until at most keep bytes are left.
+// Returns idle blocks to the device until at most keep bytes are left: the
+// longest idle one that is enough by itself, else the longest idle one and so
+// on, so that few of the blocks that a repeated call wants have to be allocated
+// again.
 void shrink(Blocks& b, size_t keep) {
   while (b.idle_bytes > keep) {
-    const Block k = b.idle.front();
-    b.idle.pop_front();
+    auto it = b.idle.begin();
+    while (it != b.idle.end() && it->bytes < b.idle_bytes - keep) ++it;
+    if (it == b.idle.end()) it = b.idle.begin();
+    const Block k = *it;
+    b.idle.erase(it);
     b.idle_bytes -= k.bytes;
     cudaEventSynchronize(k.done);
     cudaFree(k.p);

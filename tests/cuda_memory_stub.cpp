@@ -286,7 +286,7 @@ static void account() {
       holds(v[k]);
     }
   for (const Buf& b : v) asked += b.n;
-  EXPECT((size_t)tsgne_device_memory_in_use() <= asked + asked / 16 + 40 * 2 * MiB);
+  EXPECT((size_t)tsgne_device_memory_in_use() <= asked + asked / 4 + 40 * (2 * MiB + MiB / 2));
   for (Buf& b : v) b.reset();
   tsgne_set_device_memory_limit(0);
   EXPECT(fake::held() == 0 && tsgne_device_memory_in_use() == 0);
