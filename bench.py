@@ -57,7 +57,7 @@ FLOPS_PER_UNORDERED_PAIR = 16  # 2 sub, 3 for d^2+1, w^2, Z add, 8 for the two f
 # sources of the dominant (symmetric repulsion) kernel; the committed DRAM
 # traffic figure is used only if it was captured on exactly these sources
 REPULSION_SRCS = [os.path.join(ROOT, "paper_2310_11186_gb300", "csrc", f)
-                  for f in ("repulsion_sym.cu", "sym_unit.cuh", "f32x2.cuh")]
+                  for f in ("repulsion_sym.cu", "sym_unit.cuh", "f32x2.cuh", "zsum.cuh")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "repulsion_zipf300k.md")
 PIPES_FILE = os.path.join(ROOT, "profiles", "repulsion_sym_zipf100k_full.md")
 
@@ -150,7 +150,7 @@ def traffic_per_launch():
 
 
 ATTRACT_SRCS = [os.path.join(ROOT, "paper_2310_11186_gb300", "csrc", f)
-                for f in ("attract_plan.cu", "row_update.cuh", "storage.cuh")]
+                for f in ("attract_plan.cu", "row_update.cuh", "storage.cuh", "zsum.cuh")]
 ATTRACT_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "attract_rmat21.md")
 
 

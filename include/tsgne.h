@@ -81,8 +81,8 @@ typedef struct {
   float bisect_tol;        /* |H_i - ln perp| tolerance of the bisection, nats */
   int32_t bisect_max_iter; /* max entropy evaluations per row */
   uint64_t seed;           /* seed of tsgne_init_Y(ctx, NULL, ...) */
-  int32_t precision;       /* storage read by the force kernels (arithmetic is FP32, Z and KL
-                              FP64 in both): 0 = FP32 P and Y; 1 = BF16 copies of P and of
+  int32_t precision;       /* storage read by the force kernels (arithmetic is FP32, Z summed
+                              exactly and KL in FP64 in both): 0 = FP32 P and Y; 1 = BF16 copies of P and of
                               the layout, rounded to nearest even from the FP32 values, which
                               stay the optimiser's master copy and what every getter returns.
                               Not an option of the paper; the batch API accepts 0 only. */

@@ -221,8 +221,13 @@ __global__ void __launch_bounds__(256) k_batch_attract(const GraphDesc* __restri
   float ax = 0.f, ay = 0.f;
   float2 yi = make_float2(0.f, 0.f), fr = yi, u = yi, gn = yi;
   int t = 0;
-  if (valid && lane == 0) {  // the row's state, on its way while the neighbours are gathered
-    fr = RowForce{d.fsum, d.tree ? nullptr : d.acc, d.funscale}.take(i);
+  // The row's state, on its way while the neighbours are gathered: loads only.
+  // Converting and clearing the accumulators here waits for them first (256
+  // graphs of 2.8M rows, a whole iteration: 15.58 ms, 14.96 ms so).
+  ulonglong2 fa = make_ulonglong2(0ull, 0ull);
+  if (valid && lane == 0) {
+    if (d.tree) fr = d.fsum[i];
+    else fa = reinterpret_cast<const ulonglong2*>(d.acc)[i];
     u = d.upd[i];
     gn = d.gains[i];
   }
@@ -250,6 +255,10 @@ __global__ void __launch_bounds__(256) k_batch_attract(const GraphDesc* __restri
   ax = group_sum<G>(ax);
   ay = group_sum<G>(ay);
   if (!valid || lane != 0) return;
+  if (!d.tree) {
+    fr = fixed_force(fa, d.funscale);
+    reinterpret_cast<ulonglong2*>(d.acc)[i] = make_ulonglong2(0ull, 0ull);
+  }
   const Sched* s = d.sched;
   const float invZ = s->inv_z;
   const float gx = 4.0f * (s->alpha * ax - fr.x * invZ);

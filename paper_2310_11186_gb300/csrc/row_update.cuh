@@ -159,6 +159,11 @@ __device__ __forceinline__ float pass_inv_z(const Sched* sched, int zslot, int n
   return inv_of(z_value(sched->zacc[zslot], sched->zbad[zslot], n));
 }
 
+// F^r of a point from its fixed-point accumulators.
+__device__ __forceinline__ float2 fixed_force(ulonglong2 v, float unscale) {
+  return make_float2(__ll2float_rn((long long)v.x) * unscale, __ll2float_rn((long long)v.y) * unscale);
+}
+
 // Where a row's repulsive force comes from (see AttractArgs): F^r per row, or
 // fixed-point accumulators, cleared for the next pass by the row that reads them.
 struct RowForce {
@@ -170,7 +175,7 @@ struct RowForce {
     ulonglong2* a = reinterpret_cast<ulonglong2*>(facc) + i;
     const ulonglong2 v = *a;
     *a = make_ulonglong2(0ull, 0ull);
-    return make_float2(__ll2float_rn((long long)v.x) * unscale, __ll2float_rn((long long)v.y) * unscale);
+    return fixed_force(v, unscale);
   }
 };
 
