@@ -41,7 +41,7 @@ std::atomic<int64_t> g_used{0};   // bytes of the blocks in use, as they were al
 std::atomic<int64_t> g_limit{0};  // on those and the idle ones together; 0: none
 
 constexpr size_t kIdleBytes = (size_t)256 << 20;  // freed bytes kept (0.1 % of a GB300)
-std::atomic<bool> g_over{false};                  // a device may hold more than that
+thread_local bool t_over = false;                 // this thread's call left a device with more than that
 
 struct Block {
   void* p;
@@ -252,7 +252,7 @@ bool give_back(const DevMem& m) {
   b.idle_bytes += m.bytes;
   g_used -= (int64_t)m.bytes;
   if (b.idle_bytes > kIdleBytes) {
-    if (alloc_stream()) g_over = true;  // the end of the scope sees to it
+    if (alloc_stream()) t_over = true;  // the end of the scope sees to it
     else shrink(b, kIdleBytes);
   }
   return true;
@@ -317,7 +317,8 @@ int64_t idle_device_bytes() {
 }
 
 void trim_idle_blocks() {
-  if (!g_over.exchange(false)) return;
+  if (!t_over) return;
+  t_over = false;
   std::lock_guard<std::mutex> lk(g_mu);
   shrink_all(kIdleBytes);
 }

@@ -259,6 +259,20 @@ static void idle_bound() {
     Buf t;  // the inner scopes' ends leave the call's own temporaries alone
     EXPECT(t.alloc(30 * MiB) == TSGNE_OK);
   }
+  const long frees = fake::frees;  // a call that frees nothing leaves it to the one that does
+  std::thread([&] {
+    EXPECT(cudaSetDevice(0) == cudaSuccess);
+    AllocScope as(stream(102));
+    std::vector<Buf> w(4);
+    for (Buf& b : w) b.alloc(80 * MiB);
+    for (Buf& b : w) b.reset();
+    std::thread([] {
+      EXPECT(cudaSetDevice(0) == cudaSuccess);
+      AllocScope other(stream(103));
+    }).join();
+    EXPECT(fake::frees == frees);
+  }).join();
+  EXPECT(fake::frees > frees);
   const size_t before = fake::held();
   size_t out = 0;
   for (Buf& b : v) {
